@@ -1548,7 +1548,6 @@ extern "C" int fe_les_apriori(fe_ctx* c, int box, int m, double cs, fe_les_stats
   const size_t need = (size_t)23 * N * N * N * w;
   if (c->les_bytes < need) {
     cudaFree(c->les_work);
-  cudaFree(c->iso_work);
     c->les_work = nullptr;
     c->les_bytes = 0;
     if (cudaMalloc(&c->les_work, need) != cudaSuccess) {
