@@ -20,9 +20,11 @@ namespace fe {
 bool fft_supported(int N);
 template <typename T> int ic_spectral(T*, T*, T*, int, uint64_t, double, double, cudaStream_t);
 template <typename T> void fill(T*, long, double, cudaStream_t);
-template <typename T> int spectrum(const T*, const T*, const T*, int, double*, int, cudaStream_t);
-template <typename T> int diag_sums(const Launch&, const BoxDev&, int, int, double*);
-template <typename T> void qcrit(const Launch&, int, int, T*);
+size_t spectrum_work_bytes(int N);
+size_t diag_work_bytes(int N);
+template <typename T> int spectrum(const T*, const T*, const T*, int, double*, int, void*, cudaStream_t);
+template <typename T> int diag_sums(const Launch&, const BoxDev&, int, int, double*, void*);
+template <typename T> void qcrit(const Launch&, const BoxDev&, int, int, T*);
 struct UNet;
 template <typename T>
 int les_apriori(const T* rho, const T* u0, const T* u1, const T* u2, int N, int m, double cs, T* work, double* part,
@@ -136,6 +138,8 @@ struct fe_ctx {
   size_t les_bytes = 0;
   double* les_part = nullptr;  // its block partial sums (device) and their pinned host copy
   double* les_hpart = nullptr;
+  void* diag_work = nullptr;  // fe_diagnostics: block sums, and the half spectrum when one is asked for
+  size_t diag_bytes = 0;
   void* iso_work = nullptr;     // fe_isosurface: per-cube counts and block scan (allocated on first use)
   size_t iso_bytes = 0;
   std::vector<double> iso_host;
@@ -503,6 +507,7 @@ extern "C" void fe_destroy(fe_ctx* c) {
   cudaFree(c->gm_basis);
   cudaFree(c->gm_part);
   cudaFree(c->les_work);
+  cudaFree(c->diag_work);
   cudaFree(c->iso_work);
   cudaFree(c->les_part);
   if (c->les_hpart) cudaFreeHost(c->les_hpart);
@@ -1370,8 +1375,20 @@ extern "C" int fe_solve_pressure(fe_ctx* c, int box, const void* b, void* x, dou
 template <typename T>
 static int diag_box(fe_ctx* c, int box, fe_diag* out, double* spec, int nbins) {
   BoxDev& B = c->hbox[box];
+  const bool spectral = spec && nbins > 0 && fft_supported(B.N);
+  const size_t need = std::max(diag_work_bytes(B.N), spectral ? spectrum_work_bytes(B.N) : 0);
+  if (c->diag_bytes < need) {
+    cudaFree(c->diag_work);
+    c->diag_work = nullptr;
+    c->diag_bytes = 0;
+    if (cudaMalloc(&c->diag_work, need) != cudaSuccess) {
+      cudaGetLastError();
+      return FE_ERR_OOM;
+    }
+    c->diag_bytes = need;
+  }
   double sums[7 + MAXD];
-  int rc = diag_sums<T>(c->L(), B, box, c->cur, sums);
+  int rc = diag_sums<T>(c->L(), B, box, c->cur, sums, c->diag_work);
   if (rc != FE_OK) return rc;
   const double n = (double)B.N * B.N * B.N, vol = B.h * B.h * B.h;
   memset(out, 0, sizeof(*out));
@@ -1391,7 +1408,7 @@ static int diag_box(fe_ctx* c, int box, fe_diag* out, double* spec, int nbins) {
     if (!fft_supported(B.N)) return FE_ERR_UNSUPPORTED;
     const int s = c->cur;
     rc = spectrum<T>((const T*)B.f[S(s, F_U0)], (const T*)B.f[S(s, F_U1)], (const T*)B.f[S(s, F_U2)], B.N, spec, nbins,
-                     c->st);
+                     c->diag_work, c->st);
     if (rc != FE_OK) return rc;
   }
   return FE_OK;
@@ -1405,8 +1422,8 @@ extern "C" int fe_diagnostics(fe_ctx* c, int box, fe_diag* out, double* spectrum
 
 extern "C" int fe_q_criterion(fe_ctx* c, int box, void* q) {
   if (!c || !q || box < 0 || box >= c->nb) return FE_ERR_INVALID_ARG;
-  if (c->fp64) qcrit<double>(c->L(), box, c->cur, (double*)q);
-  else qcrit<float>(c->L(), box, c->cur, (float*)q);
+  if (c->fp64) qcrit<double>(c->L(), c->hbox[box], box, c->cur, (double*)q);
+  else qcrit<float>(c->L(), c->hbox[box], box, c->cur, (float*)q);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->st));
   return FE_OK;

@@ -41,3 +41,36 @@ def test_les_keeps_the_surface_memory(fe):
     assert float(other.min()) == 7.0 and float(other.max()) == 7.0
     assert np.array_equal(tri.cpu().numpy().reshape(-1, 3, 3), T)
     s.close()
+
+
+@pytest.mark.parametrize("fp64", [True, False])
+@pytest.mark.parametrize("N", [8, 9, 12, 21, 27, 32, 40, 48, 54, 64, 96, 128])
+def test_diagnostics_at_every_radix_and_ragged_tiles(fe, N, fp64):
+    """Sums, Q and the spectrum (N = 2^a 3^b) on grids that end tiles (32 x 8 x 16), groups of eight lines
+    and every butterfly (16, 8, 4, 2, 3), fewer and more bins than shells.  The sums, the transform and the
+    bins are FP64 for either field type: 1e-12 of the largest bin bounds log2(N) roundings of a transform
+    and a sum; Q of FP32 fields is one FP32 rounding of a 46-bit value."""
+    rho, u, Y, T = random_fields(N, 2, True, seed=N, noise=0.02)
+    dt = np.float64 if fp64 else np.float32
+    rho, T = rho.astype(dt), T.astype(dt)
+    u, Y = [c.astype(dt) for c in u], [y.astype(dt) for y in Y]
+    s = fe.Solver([dict(N=N, tau_p=[0.05, 0.1], Y0=[0.01, 0.02])], closure=fe.FE_FOURIER,
+                  precision=fe.FE_FP64 if fp64 else fe.FE_FP32_MIXED)
+    s.set_state(0, rho, u, Y, T)
+    r8, u8, h = rho.astype(np.float64), [c.astype(np.float64) for c in u], 2 * math.pi / N
+    smooth = N & (N - 1) == 0 or N in (9, 12, 27, 48, 54, 96)
+    for nbins in ((N // 2, N + 3) if smooth else (0,)):
+        ref, got = odiag.diagnostics(r8, u8, h, nbins), s.diagnostics(0, nbins)
+        for k in ("ke", "ke_u", "enstrophy", "taylor", "rho_rms"):
+            assert abs(got[k] - ref[k]) <= 1e-12 * abs(ref[k]), k
+        usq = sum(c * c for c in u8)
+        cv = 1.0 / 1.4 / 0.4
+        assert abs(got["energy"] / (h ** 3 * np.sum(r8 * (cv * T.astype(np.float64) + 0.5 * usq))) - 1) < 1e-12
+        for j in range(2):
+            assert abs(got["dust_mass"][j] / (h ** 3 * np.sum(r8 * Y[j].astype(np.float64))) - 1) < 1e-12
+        if nbins:
+            assert np.max(np.abs(got["spectrum"] - ref["spectrum"])) <= 1e-12 * np.max(ref["spectrum"])
+    q = s.q_criterion(0).cpu().numpy().astype(np.float64)
+    qr = odiag.q_criterion(u8, h)
+    assert np.all(np.abs(q - qr) <= (1e-15 if fp64 else 6e-8) * np.abs(qr) + 1e-12 * np.max(np.abs(qr)))
+    s.close()
