@@ -312,8 +312,8 @@ int fe_raster_depth(fe_ctx* ctx, const double* tri, long long ntri, int width, d
  * <tau^d:B>/<B:B> (least-squares Cs^2), corr = <tau^d:B>/sqrt(<tau^d:tau^d>
  * <B:B>), pi_model = -cs^2 <B:S>.  fields: NULL or a device array of 10 N^3
  * values of the context precision receiving rho_bar, u~_0..2 and tau in the
- * order 00 01 02 11 12 22.  Work memory (23 N^3 values) is allocated on the
- * first call and kept by the context (FE_ERR_OOM if it cannot be).  The model
+ * order 00 01 02 11 12 22.  Work memory (10 N^3 values, 20 in FP64 or for m > 4) is
+ * allocated on the first call and kept by the context (FE_ERR_OOM if it cannot be).  The model
  * is evaluated a priori only; it does not enter fe_step. */
 #define FE_LES_MAX_M 8
 typedef struct {

@@ -26,10 +26,10 @@ template <typename T> int spectrum(const T*, const T*, const T*, int, double*, i
 template <typename T> int diag_sums(const Launch&, const BoxDev&, int, int, double*, void*);
 template <typename T> void qcrit(const Launch&, const BoxDev&, int, int, T*);
 struct UNet;
+size_t les_work_bytes(int N, int m, int word);
 template <typename T>
-int les_apriori(const T* rho, const T* u0, const T* u1, const T* u2, int N, int m, double cs, T* work, double* part,
-                double* hpart, int nsm, T* out, double* stats, cudaStream_t st);
-int les_max_blocks(int nsm);
+int les_apriori(const T* rho, const T* u0, const T* u1, const T* u2, int N, int m, double cs, void* work, int nsm,
+                T* out, double* stats, cudaStream_t st);
 template <typename T>
 int isosurface(const T* f, int N, double iso, double* tri, long long max_tri, void* work,
                std::vector<double>& hscratch, int nsm, long long* ntri, double* area, cudaStream_t st);
@@ -134,10 +134,8 @@ struct fe_ctx {
   void* const* harvest_x = nullptr;
   int harvest_max = 0, harvest_n = 0;
   Prof prof;
-  void* les_work = nullptr;   // fe_les_apriori: 23 N^3 arrays of the largest box (allocated on first use)
+  void* les_work = nullptr;   // fe_les_apriori: filtered fields and block sums (allocated on first use)
   size_t les_bytes = 0;
-  double* les_part = nullptr;  // its block partial sums (device) and their pinned host copy
-  double* les_hpart = nullptr;
   void* diag_work = nullptr;  // fe_diagnostics: block sums, and the half spectrum when one is asked for
   size_t diag_bytes = 0;
   void* iso_work = nullptr;     // fe_isosurface: per-cube counts and block scan (allocated on first use)
@@ -509,8 +507,6 @@ extern "C" void fe_destroy(fe_ctx* c) {
   cudaFree(c->les_work);
   cudaFree(c->diag_work);
   cudaFree(c->iso_work);
-  cudaFree(c->les_part);
-  if (c->les_hpart) cudaFreeHost(c->les_hpart);
   if (c->gm_hpart) cudaFreeHost(c->gm_hpart);
   if (c->hactive) cudaFreeHost(c->hactive);
   if (c->hsc) cudaFreeHost(c->hsc);
@@ -1561,8 +1557,7 @@ extern "C" int fe_les_apriori(fe_ctx* c, int box, int m, double cs, fe_les_stats
   if (!c || !out || box < 0 || box >= c->nb || m < 1 || m > FE_LES_MAX_M || !(cs >= 0.0)) return FE_ERR_INVALID_ARG;
   const int N = c->N[box];
   if (2 * m + 1 > N) return FE_ERR_INVALID_ARG;
-  const size_t w = c->fp64 ? 8 : 4;
-  const size_t need = (size_t)23 * N * N * N * w;
+  const size_t need = les_work_bytes(N, m, c->fp64 ? 8 : 4);
   if (c->les_bytes < need) {
     cudaFree(c->les_work);
     c->les_work = nullptr;
@@ -1573,14 +1568,6 @@ extern "C" int fe_les_apriori(fe_ctx* c, int box, int m, double cs, fe_les_stats
     }
     c->les_bytes = need;
   }
-  const int nbl = les_max_blocks(c->nsm);
-  if (!c->les_part) {
-    if (cudaMalloc(&c->les_part, (size_t)nbl * 8 * sizeof(double)) != cudaSuccess ||
-        cudaMallocHost(&c->les_hpart, (size_t)nbl * 8 * sizeof(double)) != cudaSuccess) {
-      cudaGetLastError();
-      return FE_ERR_OOM;
-    }
-  }
   const BoxDev& B = c->hbox[box];
   const int s = c->cur;
   double st[6];
@@ -1588,11 +1575,11 @@ extern "C" int fe_les_apriori(fe_ctx* c, int box, int m, double cs, fe_les_stats
   if (c->fp64)
     rc = les_apriori<double>((const double*)B.f[S(s, F_RHO)], (const double*)B.f[S(s, F_U0)],
                              (const double*)B.f[S(s, F_U1)], (const double*)B.f[S(s, F_U2)], N, m, cs,
-                             (double*)c->les_work, c->les_part, c->les_hpart, c->nsm, (double*)fields, st, c->st);
+                             c->les_work, c->nsm, (double*)fields, st, c->st);
   else
     rc = les_apriori<float>((const float*)B.f[S(s, F_RHO)], (const float*)B.f[S(s, F_U0)],
                             (const float*)B.f[S(s, F_U1)], (const float*)B.f[S(s, F_U2)], N, m, cs,
-                            (float*)c->les_work, c->les_part, c->les_hpart, c->nsm, (float*)fields, st, c->st);
+                            c->les_work, c->nsm, (float*)fields, st, c->st);
   if (rc != FE_OK) return rc;
   out->delta = st[0];
   out->k_sgs = st[1];

@@ -11,16 +11,13 @@
 // slot: Smagorinsky B_ij = -2 rho_bar Delta^2 |S| S^d_ij.  Statistics: means
 // of tau_kk / 2, -tau^d:S, tau^d:B, B:B, tau^d:tau^d and B:S.
 //
-// Passes over HBM (N^3 words each): x pass reads rho, u (4) and writes the ten
-// x-filtered quantities (rho, rho u_i, rho u_i u_j); y and z passes read ten
-// and write ten (each thread eight consecutive outputs from a register window
-// when N is a multiple of eight and m <= 4); the Favre velocity reads four and
-// writes three; the statistics pass reads thirteen.  74 words per cell in all.
+// FP32 fields with m <= 4: one pass reads rho and u (4 words per cell), filters along all three
+// axes and writes rho_bar, u~ and tau (10); the statistics pass reads them back (10).  FP64 fields
+// (bound by the FP64 pipe, for which the halo rows of that pass are extra work) and wider filters:
+// an x pass (4 + 10), y and z passes (20 each) and the closing pass (20) first.
 #include <cmath>
-#include <cstring>
-#include <vector>
 
-#include "fe_internal.cuh"
+#include "gradtile.cuh"
 
 namespace fe {
 
@@ -128,29 +125,129 @@ __global__ void __launch_bounds__(LES_THREADS) k_les_win(LesPtrs<T> in, LesPtrs<
   }
 }
 
-// u~_i = bar(rho u_i) / rho_bar
+// rho_bar, u~ and tau from the ten filtered quantities of a cell
 template <typename T>
-__global__ void __launch_bounds__(LES_THREADS) k_les_favre(LesPtrs<T> F, T* __restrict__ ut0, T* __restrict__ ut1,
-                                                           T* __restrict__ ut2, long n) {
+__device__ __forceinline__ void les_close(const T (&v)[LES_NF], T (&o)[LES_NF]) {
+  const T ir = T(1) / v[0];
+  o[0] = v[0];
+#pragma unroll
+  for (int q = 1; q < 4; ++q) o[q] = v[q] * ir;
+  o[4] = v[4] - v[1] * v[1] * ir;
+  o[5] = v[5] - v[1] * v[2] * ir;
+  o[6] = v[6] - v[1] * v[3] * ir;
+  o[7] = v[7] - v[2] * v[2] * ir;
+  o[8] = v[8] - v[2] * v[3] * ir;
+  o[9] = v[9] - v[3] * v[3] * ir;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(LES_THREADS) k_les_close(LesPtrs<T> F, T* __restrict__ out, long n) {
   for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < n; c += (long)gridDim.x * blockDim.x) {
-    const T ir = T(1) / F.f[0][c];
-    ut0[c] = F.f[1][c] * ir;
-    ut1[c] = F.f[2][c] * ir;
-    ut2[c] = F.f[3][c] * ir;
+    T v[LES_NF], o[LES_NF];
+#pragma unroll
+    for (int q = 0; q < LES_NF; ++q) v[q] = F.f[q][c];
+    les_close<T>(v, o);
+#pragma unroll
+    for (int q = 0; q < LES_NF; ++q) out[q * n + c] = o[q];
   }
 }
 
-// Gauss cell gradient along d of a cell field (h * Gc), compact form
-template <typename T>
-__device__ __forceinline__ T les_gc_h(const T* __restrict__ f, long i, long j, long k, int N, int d) {
-  auto at = [&](int s) -> T {
-    long ii = i, jj = j, kk = k;
-    if (d == 0) ii = les_wrap(i + s, N);
-    else if (d == 1) jj = les_wrap(j + s, N);
-    else kk = les_wrap(k + s, N);
-    return f[ii + (long)N * (jj + (long)N * kk)];
+// All three filter passes and the closing in one (FP32 fields): a block walks kLesTz planes of a
+// 32 x 8 tile.  rho and u of a plane with a halo of M cells are staged, the ten quantities filtered
+// along x go to shared memory (tile rows and their y halo), a thread filters its column's along y
+// and keeps the last 2 M + 1 planes of them in registers for z.  24 words of traffic per cell with
+// the statistics pass instead of 74, at the price of (8 + 2 M) / 8 times the x work; products and
+// taps are summed in the order of the separate passes.  The next plane's loads are in flight while
+// a plane is filtered.
+constexpr int kLesTz = 32;
+template <int M>
+__global__ void __launch_bounds__(NTHR) k_les_fused(const float* __restrict__ rho, const float* __restrict__ u0,
+                                                    const float* __restrict__ u1, const float* __restrict__ u2, int N,
+                                                    float* __restrict__ out) {
+  constexpr int W = TX + 2 * M, R = TY + 2 * M, CELLS = W * R, PER = (CELLS + NTHR - 1) / NTHR;
+  __shared__ float in[4][CELLS];
+  __shared__ float xf[LES_NF][R][TX];
+  const int tid = threadIdx.x + TX * threadIdx.y;
+  const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y;
+  const int k0 = blockIdx.z * kLesTz, kend = min(k0 + kLesTz, N);
+  const size_t NN = (size_t)N * N;
+  const long n = (long)N * NN;
+  const float* f[4] = {rho, u0, u1, u2};
+  const float w = 1.f / (2 * M), we = 0.5f * w;
+  int off[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int t = min(tid + q * NTHR, CELLS - 1);
+    const int x = (int)(blockIdx.x * TX) - M + t % W, y = (int)(blockIdx.y * TY) - M + t / W;
+    off[q] = (x + N) % N + N * ((y + N) % N);
+  }
+  float ld[4][PER], win[LES_NF][2 * M + 1];
+  auto fetch = [&](int k) {
+    const size_t p = (size_t)((k + N) % N) * NN;
+#pragma unroll
+    for (int l = 0; l < 4; ++l)
+#pragma unroll
+      for (int q = 0; q < PER; ++q) ld[l][q] = f[l][p + off[q]];
   };
-  return ((at(-2) - at(2)) + T(10) * (at(1) - at(-1))) * T(0.0625);
+  fetch(k0 - M);
+  for (int k = k0 - M; k < kend + M; ++k) {
+#pragma unroll
+    for (int l = 0; l < 4; ++l)
+#pragma unroll
+      for (int q = 0; q < PER; ++q)
+        if (tid + q * NTHR < CELLS) in[l][tid + q * NTHR] = ld[l][q];
+    __syncthreads();
+    if (k + 1 < kend + M) fetch(k + 1);
+    for (int y = threadIdx.y; y < R; y += TY) {
+      float acc[LES_NF];
+#pragma unroll
+      for (int q = 0; q < LES_NF; ++q) acc[q] = 0.f;
+#pragma unroll
+      for (int o = 0; o <= 2 * M; ++o) {
+        const int s = y * W + threadIdx.x + o;
+        const float t = (o == 0 || o == 2 * M) ? we : w;
+        const float r = in[0][s], a = in[1][s], b = in[2][s], d = in[3][s];
+        const float ra = r * a, rb = r * b, rd = r * d;
+        acc[0] += t * r;
+        acc[1] += t * ra;
+        acc[2] += t * rb;
+        acc[3] += t * rd;
+        acc[4] += t * (ra * a);
+        acc[5] += t * (ra * b);
+        acc[6] += t * (ra * d);
+        acc[7] += t * (rb * b);
+        acc[8] += t * (rb * d);
+        acc[9] += t * (rd * d);
+      }
+#pragma unroll
+      for (int q = 0; q < LES_NF; ++q) xf[q][y][threadIdx.x] = acc[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < LES_NF; ++q) {
+      float acc = 0.f;
+#pragma unroll
+      for (int o = 0; o <= 2 * M; ++o)
+        acc += ((o == 0 || o == 2 * M) ? we : w) * xf[q][threadIdx.y + o][threadIdx.x];
+#pragma unroll
+      for (int o = 0; o < 2 * M; ++o) win[q][o] = win[q][o + 1];
+      win[q][2 * M] = acc;
+    }
+    if (k - M >= k0 && i < N && j < N) {
+      float v[LES_NF], o[LES_NF];
+#pragma unroll
+      for (int q = 0; q < LES_NF; ++q) {
+        float acc = 0.f;
+#pragma unroll
+        for (int t = 0; t <= 2 * M; ++t) acc += ((t == 0 || t == 2 * M) ? we : w) * win[q][t];
+        v[q] = acc;
+      }
+      les_close<float>(v, o);
+      const size_t c = (size_t)(k - M) * NN + (size_t)j * N + i;
+#pragma unroll
+      for (int q = 0; q < LES_NF; ++q) out[q * n + c] = o[q];
+    }
+  }
 }
 
 // symmetric tensors in the order 00 01 02 11 12 22
@@ -169,35 +266,36 @@ __device__ __forceinline__ void les_dev(T (&a)[6]) {
 
 constexpr int LES_NS = 6;  // sums: tr tau, tau^d:S, tau^d:B, B:B, tau^d:tau^d, B:S
 
-// statistics; optional output (rho_bar, u~ (3), tau (6)) as ten N^3 arrays
+// Statistics of the ten fields f (rho_bar, u~ (3), tau (6)): block sums part[block][LES_NS].
 template <typename T>
-__global__ void __launch_bounds__(LES_THREADS) k_les_stats(LesPtrs<T> F, const T* __restrict__ ut0,
-                                                           const T* __restrict__ ut1, const T* __restrict__ ut2,
-                                                           int N, double ih, double delta, double* part, T* out) {
+__global__ void __launch_bounds__(NTHR) k_les_stats(const T* __restrict__ f, int N, double ih, double delta,
+                                                    double* __restrict__ part) {
+  __shared__ T sh[3][kGradH][kGradW];
   const long n = (long)N * N * N;
-  const T* ut[3] = {ut0, ut1, ut2};
   const T ihT = (T)ih, d2 = (T)(delta * delta);
+  GradTile<T, T> t(f + n, f + 2 * n, f + 3 * n, N, sh);
+  const int k0 = blockIdx.z * kGradTz, kend = min(k0 + kGradTz, N);
   T acc[LES_NS];
 #pragma unroll
   for (int q = 0; q < LES_NS; ++q) acc[q] = T(0);
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < n; c += (long)gridDim.x * blockDim.x) {
-    const long i = c % N, j = (c / N) % N, k = c / ((long)N * N);
-    const T rb = F.f[0][c];
-    const T ir = T(1) / rb;
-    const T ru[3] = {F.f[1][c], F.f[2][c], F.f[3][c]};
+  t.start(k0);
+  for (int k = k0; k < kend; ++k) {
+    t.next(k);
+    if (t.i >= N || t.j >= N) continue;
+    const size_t c = t.plane(k) + t.own;
+    const T rb = f[c];
     T tau[6];
-    tau[0] = F.f[4][c] - ru[0] * ru[0] * ir;
-    tau[1] = F.f[5][c] - ru[0] * ru[1] * ir;
-    tau[2] = F.f[6][c] - ru[0] * ru[2] * ir;
-    tau[3] = F.f[7][c] - ru[1] * ru[1] * ir;
-    tau[4] = F.f[8][c] - ru[1] * ru[2] * ir;
-    tau[5] = F.f[9][c] - ru[2] * ru[2] * ir;
-    // g[a][b] = Gc_b u~_a
-    T g[3][3];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) tau[q] = f[(4 + q) * n + c];
+    T g[3][3];  // g[a][b] = Gc_b u~_a
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-      for (int b = 0; b < 3; ++b) g[a][b] = les_gc_h<T>(ut[a], i, j, k, N, b) * ihT;
+      for (int b = 0; b < 3; ++b) {
+        T v[4];
+        t.line(a, b, v);
+        g[a][b] = ((v[0] - v[3]) + T(10) * (v[2] - v[1])) * T(0.0625) * ihT;
+      }
     T S[6] = {g[0][0], T(0.5) * (g[0][1] + g[1][0]), T(0.5) * (g[0][2] + g[2][0]), g[1][1],
               T(0.5) * (g[1][2] + g[2][1]), g[2][2]};
     const T mag = sqrt(T(2) * les_contract<T>(S, S));
@@ -214,29 +312,20 @@ __global__ void __launch_bounds__(LES_THREADS) k_les_stats(LesPtrs<T> F, const T
     acc[3] += les_contract<T>(B, B);
     acc[4] += les_contract<T>(td, td);
     acc[5] += les_contract<T>(B, S);
-    if (out) {
-      out[c] = rb;
-      out[n + c] = ru[0] * ir;
-      out[2 * n + c] = ru[1] * ir;
-      out[3 * n + c] = ru[2] * ir;
-#pragma unroll
-      for (int q = 0; q < 6; ++q) out[(4 + q) * n + c] = tau[q];
-    }
   }
-  // block tree in double (fixed order); the host adds the block partials in order
-  __shared__ double red[LES_THREADS / 32][LES_NS];
+  __shared__ double red[NTHR / 32][LES_NS];
 #pragma unroll
   for (int q = 0; q < LES_NS; ++q) {
     double v = (double)acc[q];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][q] = v;
+    if ((t.tid & 31) == 0) red[t.tid >> 5][q] = v;
   }
   __syncthreads();
-  if (threadIdx.x < LES_NS) {
+  if (t.tid < LES_NS) {
     double s = 0.0;
-    for (int w = 0; w < LES_THREADS / 32; ++w) s += red[w][threadIdx.x];
-    part[(long)blockIdx.x * LES_NS + threadIdx.x] = s;
+    for (int w = 0; w < NTHR / 32; ++w) s += red[w][t.tid];
+    part[(size_t)(blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) * LES_NS + t.tid] = s;
   }
 }
 
@@ -246,47 +335,78 @@ static int les_grid(long n, int nsm) {
   return (int)(g < cap ? g : cap);
 }
 
-// work: 23 N^3 arrays of T (x/z output set, y output set, u~); part: les_grid
-// blocks x LES_NS doubles.  Statistics in stats[0..5]: delta, k_sgs, pi_sgs,
-// cs2_opt, corr, pi_model (fixed-order sums).
 template <typename T>
-int les_apriori(const T* rho, const T* u0, const T* u1, const T* u2, int N, int m, double cs, T* work, double* part,
-                double* hpart, int nsm, T* out, double* stats, cudaStream_t st) {
+static bool les_fused(int m) {
+  return sizeof(T) == 4 && m <= 4;
+}
+
+// Work memory: the ten fields of a caller that does not take them, or the two sets of the separate
+// passes; then the block sums of the statistics and the sums.
+size_t les_work_bytes(int N, int m, int word) {
+  const dim3 g = grad_grid(N);
+  const size_t n = (size_t)N * N * N, sets = word == 4 && les_fused<float>(m) ? 1 : 2;
+  return (sets * LES_NF * n * word + 255) / 256 * 256 + ((size_t)g.x * g.y * g.z + 1) * LES_NS * sizeof(double);
+}
+
+// Statistics in stats[0..5]: delta, k_sgs, pi_sgs, cs2_opt, corr, pi_model (fixed-order sums); out: the
+// ten fields rho_bar, u~ (3), tau (6), or null.
+template <typename T>
+int les_apriori(const T* rho, const T* u0, const T* u1, const T* u2, int N, int m, double cs, void* work, int nsm,
+                T* out, double* stats, cudaStream_t st) {
   const long n = (long)N * N * N;
-  LesPtrs<T> A, Bp;
-  for (int q = 0; q < LES_NF; ++q) {
-    A.f[q] = work + q * n;
-    Bp.f[q] = work + (LES_NF + q) * n;
-  }
-  T* ut = work + 2 * LES_NF * n;
-  const int grid = les_grid(n, nsm);
-  k_les_x<T><<<grid, LES_THREADS, 0, st>>>(rho, u0, u1, u2, N, m, A);
-  if (N % LES_OUTS == 0 && m <= 4) {
-    const int gw = les_grid(n / LES_OUTS, nsm);
-    for (int axis = 1; axis <= 2; ++axis) {
-      const LesPtrs<T>& src = axis == 1 ? A : Bp;
-      const LesPtrs<T>& dst = axis == 1 ? Bp : A;
+  const bool fused = les_fused<T>(m);
+  T* A0 = static_cast<T*>(work);
+  double* part = reinterpret_cast<double*>(static_cast<char*>(work) +
+                                           ((size_t)(fused ? 1 : 2) * LES_NF * n * sizeof(T) + 255) / 256 * 256);
+  T* f = out ? out : A0;
+  if constexpr (sizeof(T) == 4) {
+    if (fused) {
+      const dim3 g((N + TX - 1) / TX, (N + TY - 1) / TY, (N + kLesTz - 1) / kLesTz), b(TX, TY);
       switch (m) {
-        case 1: k_les_win<T, 1><<<gw, LES_THREADS, 0, st>>>(src, dst, N, axis); break;
-        case 2: k_les_win<T, 2><<<gw, LES_THREADS, 0, st>>>(src, dst, N, axis); break;
-        case 3: k_les_win<T, 3><<<gw, LES_THREADS, 0, st>>>(src, dst, N, axis); break;
-        default: k_les_win<T, 4><<<gw, LES_THREADS, 0, st>>>(src, dst, N, axis); break;
+        case 1: k_les_fused<1><<<g, b, 0, st>>>(rho, u0, u1, u2, N, f); break;
+        case 2: k_les_fused<2><<<g, b, 0, st>>>(rho, u0, u1, u2, N, f); break;
+        case 3: k_les_fused<3><<<g, b, 0, st>>>(rho, u0, u1, u2, N, f); break;
+        default: k_les_fused<4><<<g, b, 0, st>>>(rho, u0, u1, u2, N, f); break;
       }
     }
-  } else {
-    k_les_line<T><<<grid, LES_THREADS, 0, st>>>(A, Bp, N, m, 1);
-    k_les_line<T><<<grid, LES_THREADS, 0, st>>>(Bp, A, N, m, 2);
   }
-  k_les_favre<T><<<grid, LES_THREADS, 0, st>>>(A, ut, ut + n, ut + 2 * n, n);
+  if (!fused) {
+    LesPtrs<T> A, Bp;
+    for (int q = 0; q < LES_NF; ++q) {
+      A.f[q] = A0 + q * n;
+      Bp.f[q] = A0 + (LES_NF + q) * n;
+    }
+    const int grid = les_grid(n, nsm);
+    k_les_x<T><<<grid, LES_THREADS, 0, st>>>(rho, u0, u1, u2, N, m, A);
+    if (N % LES_OUTS == 0 && m <= 4) {
+      const int gw = les_grid(n / LES_OUTS, nsm);
+      for (int axis = 1; axis <= 2; ++axis) {
+        const LesPtrs<T>& src = axis == 1 ? A : Bp;
+        const LesPtrs<T>& dst = axis == 1 ? Bp : A;
+        switch (m) {
+          case 1: k_les_win<T, 1><<<gw, LES_THREADS, 0, st>>>(src, dst, N, axis); break;
+          case 2: k_les_win<T, 2><<<gw, LES_THREADS, 0, st>>>(src, dst, N, axis); break;
+          case 3: k_les_win<T, 3><<<gw, LES_THREADS, 0, st>>>(src, dst, N, axis); break;
+          default: k_les_win<T, 4><<<gw, LES_THREADS, 0, st>>>(src, dst, N, axis); break;
+        }
+      }
+    } else {
+      k_les_line<T><<<grid, LES_THREADS, 0, st>>>(A, Bp, N, m, 1);
+      k_les_line<T><<<grid, LES_THREADS, 0, st>>>(Bp, A, N, m, 2);
+    }
+    if (!out) f = Bp.f[0];  // the closing pass reads A
+    k_les_close<T><<<grid, LES_THREADS, 0, st>>>(A, f, n);
+  }
   const double h = 2.0 * M_PI / N, delta = 2.0 * m * h;
-  k_les_stats<T><<<grid, LES_THREADS, 0, st>>>(A, ut, ut + n, ut + 2 * n, N, 1.0 / h, delta, part, out);
-  if (cudaMemcpyAsync(hpart, part, (size_t)grid * LES_NS * sizeof(double), cudaMemcpyDeviceToHost, st) !=
-          cudaSuccess ||
+  const dim3 g = grad_grid(N);
+  const int blocks = (int)(g.x * g.y * g.z);
+  double* sums = part + (size_t)blocks * LES_NS;
+  double s[LES_NS];
+  k_les_stats<T><<<g, dim3(TX, TY), 0, st>>>(f, N, 1.0 / h, delta, part);
+  k_sum_parts<<<LES_NS, NTHR, 0, st>>>(part, blocks, LES_NS, sums);
+  if (cudaMemcpyAsync(s, sums, sizeof(s), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
     return FE_ERR_CUDA;
-  double s[LES_NS] = {0, 0, 0, 0, 0, 0};
-  for (int b = 0; b < grid; ++b)
-    for (int q = 0; q < LES_NS; ++q) s[q] += hpart[(long)b * LES_NS + q];
   for (int q = 0; q < LES_NS; ++q) s[q] /= (double)n;
   stats[0] = delta;
   stats[1] = 0.5 * s[0];
@@ -297,11 +417,9 @@ int les_apriori(const T* rho, const T* u0, const T* u1, const T* u2, int N, int 
   return FE_OK;
 }
 
-int les_max_blocks(int nsm) { return nsm * 8; }
-
-template int les_apriori<double>(const double*, const double*, const double*, const double*, int, int, double,
-                                 double*, double*, double*, int, double*, double*, cudaStream_t);
-template int les_apriori<float>(const float*, const float*, const float*, const float*, int, int, double, float*,
-                                double*, double*, int, float*, double*, cudaStream_t);
+template int les_apriori<double>(const double*, const double*, const double*, const double*, int, int, double, void*,
+                                 int, double*, double*, cudaStream_t);
+template int les_apriori<float>(const float*, const float*, const float*, const float*, int, int, double, void*, int,
+                                float*, double*, cudaStream_t);
 
 }  // namespace fe
