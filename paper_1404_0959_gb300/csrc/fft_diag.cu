@@ -474,17 +474,17 @@ __global__ void __launch_bounds__(NTHR) k_diag(const BoxDev* boxes, int box, int
       }
     const double w0 = g[1][2] - g[2][1], w1 = g[2][0] - g[0][2], w2 = g[0][1] - g[1][0];
     const size_t c = t.plane(k) + t.own;
-    const double r = (double)rho[c];
+    const double r = widen(rho[c]);
     const double uu = t.z[0][2] * t.z[0][2] + t.z[1][2] * t.z[1][2] + t.z[2][2] * t.z[2][2];
     acc[0] += r * uu;
     acc[1] += uu;
     acc[2] += w0 * w0 + w1 * w1 + w2 * w2;
     acc[3] += g[0][0] * g[0][0] + g[1][1] * g[1][1] + g[2][2] * g[2][2];
     acc[4] += r;
-    if (fourier) acc[5] += r * (double)Tf[c];
+    if (fourier) acc[5] += r * widen(Tf[c]);
 #pragma unroll
     for (int q = 0; q < MAXD; ++q)
-      if (q < nd) acc[6 + q] += r * (double)F<T>(B, S(s, F_Y0 + q))[c];
+      if (q < nd) acc[6 + q] += r * widen(F<T>(B, S(s, F_Y0 + q))[c]);
   }
   __shared__ double red[NDIAG][NTHR / 32];
   const int lane = t.tid & 31, warp = t.tid >> 5;
