@@ -279,8 +279,8 @@ int fe_q_criterion(fe_ctx* ctx, int box, void* q_dev);
  * The surface is closed (the split is the same in every cube).  tri: NULL
  * (max_tri = 0) or a device array of 9 * max_tri doubles (x, y, z of the three
  * corners); the first min(total, max_tri) triangles are written.  *ntri
- * receives the total count, *area the total area.  Work memory (16 bytes per
- * cell) is allocated on the first call and kept by the context. */
+ * receives the total count, *area the total area.  Work memory (20 bytes per
+ * 128 cells) is allocated on the first call and kept by the context. */
 int fe_isosurface(fe_ctx* ctx, int box, const void* field, double iso, double* tri, long long max_tri,
                   long long* ntri, double* area);
 /* Depth image of ntri triangles (device, 9 doubles each) viewed along +z

@@ -31,9 +31,9 @@ template <typename T>
 int les_apriori(const T* rho, const T* u0, const T* u1, const T* u2, int N, int m, double cs, void* work, int nsm,
                 T* out, double* stats, cudaStream_t st);
 template <typename T>
-int isosurface(const T* f, int N, double iso, double* tri, long long max_tri, void* work,
-               std::vector<double>& hscratch, int nsm, long long* ntri, double* area, cudaStream_t st);
-size_t iso_work_bytes(long n);
+int isosurface(const T* f, int N, double iso, double* tri, long long max_tri, void* work, long long* ntri,
+               double* area, cudaStream_t st);
+size_t iso_work_bytes(int N);
 int raster_depth(const double* tri, long long ntri, int W, double extent, float* depth, int nsm, cudaStream_t st);
 UNet* unet_create(int N, bool training, int* rc);
 void unet_destroy(UNet* U);
@@ -138,9 +138,8 @@ struct fe_ctx {
   size_t les_bytes = 0;
   void* diag_work = nullptr;  // fe_diagnostics: block sums, and the half spectrum when one is asked for
   size_t diag_bytes = 0;
-  void* iso_work = nullptr;     // fe_isosurface: per-cube counts and block scan (allocated on first use)
+  void* iso_work = nullptr;     // fe_isosurface: block counts, offsets and areas (allocated on first use)
   size_t iso_bytes = 0;
-  std::vector<double> iso_host;
   Launch L() {
     Launch l{dbox,           dwork,         nblocks,       dework, neblocks, dpart, dactive, st, &prof,
              prm.closure == FE_FOURIER, prm.transonic, prm.n_dust, ring_ok, use_bulk && nbblocks > 0 ? dbwork : nullptr,
@@ -1597,8 +1596,7 @@ extern "C" int fe_isosurface(fe_ctx* c, int box, const void* field, double iso, 
       !std::isfinite(iso))
     return FE_ERR_INVALID_ARG;
   const int N = c->N[box];
-  const long n = (long)N * N * N;
-  const size_t need = iso_work_bytes(n);
+  const size_t need = iso_work_bytes(N);
   if (c->iso_bytes < need) {
     cudaFree(c->iso_work);
     c->iso_work = nullptr;
@@ -1609,11 +1607,8 @@ extern "C" int fe_isosurface(fe_ctx* c, int box, const void* field, double iso, 
     }
     c->iso_bytes = need;
   }
-  if (c->fp64)
-    return isosurface<double>((const double*)field, N, iso, tri, max_tri, c->iso_work, c->iso_host, c->nsm, ntri, area,
-                              c->st);
-  return isosurface<float>((const float*)field, N, iso, tri, max_tri, c->iso_work, c->iso_host, c->nsm, ntri, area,
-                           c->st);
+  if (c->fp64) return isosurface<double>((const double*)field, N, iso, tri, max_tri, c->iso_work, ntri, area, c->st);
+  return isosurface<float>((const float*)field, N, iso, tri, max_tri, c->iso_work, ntri, area, c->st);
 }
 
 extern "C" int fe_raster_depth(fe_ctx* c, const double* tri, long long ntri, int width, double extent,

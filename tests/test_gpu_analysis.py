@@ -74,3 +74,26 @@ def test_diagnostics_at_every_radix_and_ragged_tiles(fe, N, fp64):
     qr = odiag.q_criterion(u8, h)
     assert np.all(np.abs(q - qr) <= (1e-15 if fp64 else 6e-8) * np.abs(qr) + 1e-12 * np.max(np.abs(qr)))
     s.close()
+
+
+@pytest.mark.parametrize("fp64", [True, False])
+@pytest.mark.parametrize("N", [8, 9, 13])
+def test_surface_of_noise(fe, N, fp64):
+    """White noise cuts cubes in every sign pattern: triangles bit for bit the oracle's, on grids that do and
+    do not fill the blocks of 128 cubes, with a level that is no FP32 number and with values equal to it."""
+    import torch
+    rng = np.random.default_rng(N)
+    f = rng.standard_normal((N, N, N))
+    if not fp64:
+        f = f.astype(np.float32).astype(np.float64)
+    f.reshape(-1)[::17] = 0.25
+    s = fe.Solver([dict(N=N, tau_p=[], Y0=[])], precision=fe.FE_FP64 if fp64 else fe.FE_FP32_MIXED)
+    fd = torch.as_tensor(f, device="cuda", dtype=torch.float64 if fp64 else torch.float32).contiguous()
+    for iso in (0.1, 0.25):
+        T, area = oiso.extract(f, iso, 2 * math.pi / N)
+        tri = torch.zeros((len(T) + 3, 9), dtype=torch.float64, device="cuda")
+        n, a = fe.fe_isosurface(s.ctx, 0, fd.data_ptr(), iso, tri.data_ptr(), len(T) + 3)
+        assert n == len(T) and abs(a - area) <= 1e-12 * area
+        assert np.array_equal(tri[:n].cpu().numpy().reshape(-1, 3, 3), T)
+        assert not tri[n:].any()
+    s.close()
