@@ -34,7 +34,9 @@ template <typename T>
 int isosurface(const T* f, int N, double iso, double* tri, long long max_tri, void* work, long long* ntri,
                double* area, cudaStream_t st);
 size_t iso_work_bytes(int N);
-int raster_depth(const double* tri, long long ntri, int W, double extent, float* depth, int nsm, cudaStream_t st);
+size_t raster_work_bytes(int W);
+int raster_depth(const double* tri, long long ntri, int W, double extent, float* depth, void* work, int nsm,
+                 cudaStream_t st);
 UNet* unet_create(int N, bool training, int* rc);
 void unet_destroy(UNet* U);
 long unet_param_count();
@@ -138,6 +140,8 @@ struct fe_ctx {
   size_t les_bytes = 0;
   void* diag_work = nullptr;  // fe_diagnostics: block sums, and the half spectrum when one is asked for
   size_t diag_bytes = 0;
+  void* raster_work = nullptr;  // fe_raster_depth: pixel centres
+  size_t raster_bytes = 0;
   void* iso_work = nullptr;     // fe_isosurface: block counts, offsets and areas (allocated on first use)
   size_t iso_bytes = 0;
   Launch L() {
@@ -506,6 +510,7 @@ extern "C" void fe_destroy(fe_ctx* c) {
   cudaFree(c->les_work);
   cudaFree(c->diag_work);
   cudaFree(c->iso_work);
+  cudaFree(c->raster_work);
   if (c->gm_hpart) cudaFreeHost(c->gm_hpart);
   if (c->hactive) cudaFreeHost(c->hactive);
   if (c->hsc) cudaFreeHost(c->hsc);
@@ -1615,7 +1620,17 @@ extern "C" int fe_raster_depth(fe_ctx* c, const double* tri, long long ntri, int
                                float* depth) {
   if (!c || !depth || width < 1 || width > 65536 || ntri < 0 || (ntri > 0 && !tri) || !(extent > 0.0))
     return FE_ERR_INVALID_ARG;
-  int rc = raster_depth(tri, ntri, width, extent, depth, c->nsm, c->st);
+  if (c->raster_bytes < raster_work_bytes(width)) {
+    cudaFree(c->raster_work);
+    c->raster_work = nullptr;
+    c->raster_bytes = 0;
+    if (cudaMalloc(&c->raster_work, raster_work_bytes(width)) != cudaSuccess) {
+      cudaGetLastError();
+      return FE_ERR_OOM;
+    }
+    c->raster_bytes = raster_work_bytes(width);
+  }
+  int rc = raster_depth(tri, ntri, width, extent, depth, c->raster_work, c->nsm, c->st);
   if (rc != FE_OK) return rc;
   CK(cudaStreamSynchronize(c->st));
   return FE_OK;

@@ -355,43 +355,170 @@ __device__ __forceinline__ float edge_fn(float xa, float ya, float xb, float yb,
   return fsub(fmul(fsub(xb, xa), fsub(py, ya)), fmul(fsub(yb, ya), fsub(px, xa)));
 }
 
-__global__ void k_fill_u32(unsigned* a, long n, unsigned v) {
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) a[q] = v;
+// Pixel range of one coordinate: floor(x / step - 1/2) and ceil(x / step - 1/2), the quotient and the
+// difference rounded to double.  Formed with the reciprocal of the step; where that lies within 1e-6 of a
+// whole number (or is not an ordinary pixel number) the division decides.
+__device__ __forceinline__ void pixel_range(double x, double step, double inv, int& lo, int& hi) {
+  const double magic = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to a whole number, kept in the low word
+  const double q = fma(x, inv, -0.5), r = q + magic, d = q - (r - magic);
+  const unsigned mag = (unsigned)__double2hiint(d) & 0x7fffffffu, size = (unsigned)__double2hiint(q) & 0x7fffffffu;
+  const int n = __double2loint(r);
+  if (size < 0x41300000u && mag > 0x3eb00000u) {  // |q| < 2^20, |q - n| > 1e-6
+    const bool below = __double2hiint(d) < 0;
+    lo = below ? n - 1 : n;
+    hi = below ? n : n + 1;
+  } else {
+    const double e = x / step - 0.5;
+    lo = (int)floor(e);
+    hi = (int)ceil(e);
+  }
 }
 
-// one thread per triangle; the bits of a float z >= 0 are ordered like z
-__global__ void __launch_bounds__(ISO_THREADS) k_raster(const double* __restrict__ tri, long long ntri, int W,
-                                                        double step, unsigned* __restrict__ depth) {
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ntri;
-       q += (long long)gridDim.x * blockDim.x) {
-    const double* p = tri + q * 9;
-    const double x0 = p[0], y0 = p[1];
-    const float X1 = (float)(p[3] - x0), Y1 = (float)(p[4] - y0), X2 = (float)(p[6] - x0), Y2 = (float)(p[7] - y0);
-    const float Z0 = (float)p[2], Z1 = (float)p[5], Z2 = (float)p[8];
-    if (fsub(fmul(X1, Y2), fmul(Y1, X2)) == 0.f) continue;
-    const int lo_x = max((int)floor(fmin(x0, fmin(p[3], p[6])) / step - 0.5) - 1, 0);
-    const int hi_x = min((int)ceil(fmax(x0, fmax(p[3], p[6])) / step - 0.5) + 1, W - 1);
-    const int lo_y = max((int)floor(fmin(y0, fmin(p[4], p[7])) / step - 0.5) - 1, 0);
-    const int hi_y = min((int)ceil(fmax(y0, fmax(p[4], p[7])) / step - 0.5) + 1, W - 1);
-    for (int py = lo_y; py <= hi_y; ++py) {
-      const float CY = (float)__dsub_rn(__dmul_rn((double)py + 0.5, step), y0);
-      for (int px = lo_x; px <= hi_x; ++px) {
-        const float CX = (float)__dsub_rn(__dmul_rn((double)px + 0.5, step), x0);
-        const float e12 = edge_fn(X1, Y1, X2, Y2, CX, CY);
-        const float e20 = edge_fn(X2, Y2, 0.f, 0.f, CX, CY);
-        const float e01 = edge_fn(0.f, 0.f, X1, Y1, CX, CY);
-        if ((e12 >= 0.f && e20 >= 0.f && e01 >= 0.f) || (e12 <= 0.f && e20 <= 0.f && e01 <= 0.f)) {
-          const float num = fadd(fadd(fmul(e12, Z0), fmul(e20, Z1)), fmul(e01, Z2));
-          const float z = __fdiv_rn(num, fadd(fadd(e12, e20), e01));
-          // the depth only decreases, so a read that is already <= z (even an older value) means the
-          // atomic would change nothing: most covered pixels of a many-layered surface skip it
-          unsigned* d = &depth[(long)py * W + px];
-          const unsigned zb = __float_as_uint(z);
-          if (z >= 0.f && zb < *d) atomicMin(d, zb);
-        }
+__device__ __forceinline__ double pixel_centre(int p, double step) { return __dmul_rn((double)p + 0.5, step); }
+
+// Depth of the pixel at (CX, CY) and its minimum in the image; the bits of a float z >= 0 are ordered
+// like z.  The depth only decreases, so a read that is already <= z (even an older value) means the
+// atomic would change nothing: most covered pixels of a many-layered surface skip it.
+__device__ __forceinline__ void put_depth(float e12, float e20, float e01, float Z0, float Z1, float Z2, unsigned* d) {
+  const float num = fadd(fadd(fmul(e12, Z0), fmul(e20, Z1)), fmul(e01, Z2));
+  const float z = __fdiv_rn(num, fadd(fadd(e12, e20), e01));
+  const unsigned zb = __float_as_uint(z);
+  if (z >= 0.f && zb < *d) atomicMin(d, zb);
+}
+
+// A warp takes 32 triangles at a time.  Each lane sets one up (corners relative to the first one, pixel
+// range); the pixel columns and rows of all 32 are then two lists: a lane forms the centre of one row
+// (CY, kept in shared memory) and, after that, walks one column of one triangle through its rows.  So
+// the FP64 work (the centres, one subtraction each) is done once per row and column on full warps, and
+// the FP32 pixel tests run with their column's products in registers; neighbouring lanes work on
+// neighbouring columns.  Triangles with more than kRastRows rows go pixel by pixel over the warp.  One
+// triangle per lane with both centres formed for every pixel took 15.8 ms for the Q surface of a 192^3
+// turbulent flow on 2048^2 pixels, this 1.65 ms.
+constexpr int kRastRows = 24;
+constexpr int kRastWarps = 4;
+struct RastWarp {
+  double raw[32 * 9];
+  double x0[32], y0[32];
+  float X1[32], Y1[32], X2[32], Y2[32], Z0[32], Z1[32], Z2[32];
+  int lox[32], loy[32], h[32], cols[32], rows[32];  // cols, rows: inclusive scans of the list lengths
+  float cy[32 * kRastRows];
+};
+
+__global__ void __launch_bounds__(32 * kRastWarps) k_raster(const double* __restrict__ tri, long long ntri, int W,
+                                                            double step, const double* __restrict__ cen,
+                                                            unsigned* __restrict__ depth) {
+  extern __shared__ char rast_smem[];
+  RastWarp& s = reinterpret_cast<RastWarp*>(rast_smem)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const double inv = 1.0 / step;
+  // a pixel more on both sides, inside the image (the conversions saturate, so clamp before adding)
+  auto first = [&](int a, int b, int c) { return min(max(min(a, min(b, c)), 1) - 1, W); };
+  auto last = [&](int a, int b, int c) { return max(min(max(a, max(b, c)), W - 2) + 1, -1); };
+  const long long warps = (long long)gridDim.x * kRastWarps;
+  for (long long q0 = ((long long)blockIdx.x * kRastWarps + (threadIdx.x >> 5)) * 32; q0 < ntri; q0 += warps * 32) {
+    const int cnt = (int)min(32LL, ntri - q0);
+    __syncwarp();
+    for (int x = lane; x < cnt * 9; x += 32) s.raw[x] = __ldg(&tri[q0 * 9 + x]);
+    __syncwarp();
+    int w = 0, h = 0;
+    bool big = false;
+    int lox = 0, loy = 0;
+    if (lane < cnt) {
+      const double* p = &s.raw[lane * 9];
+      const double x0 = p[0], y0 = p[1];
+      const float X1 = narrow(p[3] - x0), Y1 = narrow(p[4] - y0), X2 = narrow(p[6] - x0), Y2 = narrow(p[7] - y0);
+      if (fsub(fmul(X1, Y2), fmul(Y1, X2)) != 0.f) {
+        int a0, a1, b0, b1, c0, c1;
+        pixel_range(x0, step, inv, a0, a1);
+        pixel_range(p[3], step, inv, b0, b1);
+        pixel_range(p[6], step, inv, c0, c1);
+        lox = first(a0, b0, c0);
+        w = last(a1, b1, c1) - lox + 1;
+        pixel_range(y0, step, inv, a0, a1);
+        pixel_range(p[4], step, inv, b0, b1);
+        pixel_range(p[7], step, inv, c0, c1);
+        loy = first(a0, b0, c0);
+        h = last(a1, b1, c1) - loy + 1;
+        if (w <= 0 || h <= 0) w = h = 0;
+      }
+      s.x0[lane] = x0;
+      s.y0[lane] = y0;
+      s.X1[lane] = X1;
+      s.Y1[lane] = Y1;
+      s.X2[lane] = X2;
+      s.Y2[lane] = Y2;
+      s.Z0[lane] = narrow(p[2]);
+      s.Z1[lane] = narrow(p[5]);
+      s.Z2[lane] = narrow(p[8]);
+      big = h > kRastRows;
+    }
+    s.lox[lane] = lox;
+    s.loy[lane] = loy;
+    s.h[lane] = h;
+    int sc = big ? 0 : w, sr = big ? 0 : h;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int tc = __shfl_up_sync(0xffffffffu, sc, o), tr = __shfl_up_sync(0xffffffffu, sr, o);
+      if (lane >= o) sc += tc, sr += tr;
+    }
+    s.cols[lane] = sc;
+    s.rows[lane] = sr;
+    const int nc = __shfl_sync(0xffffffffu, sc, 31), nr = __shfl_sync(0xffffffffu, sr, 31);
+    __syncwarp();
+    auto owner = [&](const int* scan, int item) {  // first triangle whose inclusive scan exceeds item
+      int t = 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        if (scan[t + o - 1] <= item) t += o;
+      return t;
+    };
+    for (int item = lane; item < nr; item += 32) {
+      const int t = owner(s.rows, item), row = item - (t ? s.rows[t - 1] : 0);
+      s.cy[item] = narrow(__dsub_rn(__ldg(&cen[s.loy[t] + row]), s.y0[t]));
+    }
+    __syncwarp();
+    for (int item = lane; item < nc; item += 32) {
+      const int t = owner(s.cols, item), px = s.lox[t] + item - (t ? s.cols[t - 1] : 0);
+      const float CX = narrow(__dsub_rn(__ldg(&cen[px]), s.x0[t]));
+      const float X1 = s.X1[t], Y1 = s.Y1[t], X2 = s.X2[t], Y2 = s.Y2[t];
+      // E_ab = (X_b - X_a)(CY - Y_a) - (Y_b - Y_a)(CX - X_a): the factors and products of the column
+      const float d12 = fsub(X2, X1), d20 = fsub(0.f, X2), d01 = fsub(X1, 0.f);
+      const float m12 = fmul(fsub(Y2, Y1), fsub(CX, X1)), m20 = fmul(fsub(0.f, Y2), fsub(CX, X2)),
+                  m01 = fmul(fsub(Y1, 0.f), fsub(CX, 0.f));
+      const float* cy = &s.cy[t ? s.rows[t - 1] : 0];
+      unsigned* d = depth + (long)s.loy[t] * W + px;
+      const int rows = s.h[t];
+      for (int r = 0; r < rows; ++r, d += W) {
+        const float CY = cy[r];
+        const float e12 = fsub(fmul(d12, fsub(CY, Y1)), m12);
+        const float e20 = fsub(fmul(d20, fsub(CY, Y2)), m20);
+        const float e01 = fsub(fmul(d01, fsub(CY, 0.f)), m01);
+        if ((e12 >= 0.f && e20 >= 0.f && e01 >= 0.f) || (e12 <= 0.f && e20 <= 0.f && e01 <= 0.f))
+          put_depth(e12, e20, e01, s.Z0[t], s.Z1[t], s.Z2[t], d);
+      }
+    }
+    // triangles with many rows: the warp over the pixels of one at a time
+    for (unsigned todo = __ballot_sync(0xffffffffu, big); todo; todo &= todo - 1) {
+      const int t = __ffs(todo) - 1, wt = __shfl_sync(0xffffffffu, w, t);
+      const float X1 = s.X1[t], Y1 = s.Y1[t], X2 = s.X2[t], Y2 = s.Y2[t];
+      const long px_all = (long)wt * s.h[t];
+      for (long q = lane; q < px_all; q += 32) {
+        const int py = s.loy[t] + (int)(q / wt), px = s.lox[t] + (int)(q % wt);
+        const float CX = narrow(__dsub_rn(__ldg(&cen[px]), s.x0[t])), CY = narrow(__dsub_rn(__ldg(&cen[py]), s.y0[t]));
+        const float e12 = edge_fn(X1, Y1, X2, Y2, CX, CY), e20 = edge_fn(X2, Y2, 0.f, 0.f, CX, CY),
+                    e01 = edge_fn(0.f, 0.f, X1, Y1, CX, CY);
+        if ((e12 >= 0.f && e20 >= 0.f && e01 >= 0.f) || (e12 <= 0.f && e20 <= 0.f && e01 <= 0.f))
+          put_depth(e12, e20, e01, s.Z0[t], s.Z1[t], s.Z2[t], &depth[(long)py * W + px]);
       }
     }
   }
+}
+
+// empty image, and the pixel centres
+__global__ void k_raster_start(unsigned* depth, long npx, double* cen, int W, double step) {
+  const long t0 = blockIdx.x * (long)blockDim.x + threadIdx.x, nt = (long)gridDim.x * blockDim.x;
+  for (long q = t0; q < npx; q += nt) depth[q] = 0x7F800000u;
+  for (long q = t0; q < W; q += nt) cen[q] = pixel_centre((int)q, step);
 }
 
 static int iso_grid(long n, int nsm) {
@@ -434,11 +561,22 @@ int isosurface(const T* f, int N, double iso, double* tri, long long max_tri, vo
   return FE_OK;
 }
 
-int raster_depth(const double* tri, long long ntri, int W, double extent, float* depth, int nsm, cudaStream_t st) {
+size_t raster_work_bytes(int W) { return (size_t)W * sizeof(double); }
+
+// work: the W pixel centres
+int raster_depth(const double* tri, long long ntri, int W, double extent, float* depth, void* work, int nsm,
+                 cudaStream_t st) {
   const long npx = (long)W * W;
-  k_fill_u32<<<iso_grid(npx, nsm), ISO_THREADS, 0, st>>>((unsigned*)depth, npx, 0x7F800000u);
-  if (ntri > 0)
-    k_raster<<<iso_grid((long)ntri, nsm), ISO_THREADS, 0, st>>>(tri, ntri, W, extent / W, (unsigned*)depth);
+  double* cen = static_cast<double*>(work);
+  k_raster_start<<<iso_grid(npx, nsm), ISO_THREADS, 0, st>>>((unsigned*)depth, npx, cen, W, extent / W);
+  if (ntri > 0) {
+    const int smem = kRastWarps * (int)sizeof(RastWarp);
+    const long long groups = (ntri + 32 * kRastWarps - 1) / (32 * kRastWarps);
+    if (cudaFuncSetAttribute(k_raster, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+      return FE_ERR_CUDA;
+    k_raster<<<(unsigned)(groups < 64LL * nsm ? groups : 64LL * nsm), 32 * kRastWarps, smem, st>>>(
+        tri, ntri, W, extent / W, cen, (unsigned*)depth);
+  }
   return cudaGetLastError() == cudaSuccess ? FE_OK : FE_ERR_CUDA;
 }
 

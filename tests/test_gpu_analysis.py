@@ -97,3 +97,24 @@ def test_surface_of_noise(fe, N, fp64):
         assert np.array_equal(tri[:n].cpu().numpy().reshape(-1, 3, 3), T)
         assert not tri[n:].any()
     s.close()
+
+
+@pytest.mark.parametrize("W,share", [(1, 1.0), (37, 1.0), (250, 1.0), (700, 1.0), (257, 0.3)])
+def test_depth_image_of_small_and_large_triangles(fe, W, share):
+    """Depth images bit for bit the oracle's: triangles below a pixel, of a few pixels, of more rows than the
+    kernel's row lists hold (24), partly and wholly outside the image."""
+    import torch
+    N = 9
+    f = np.random.default_rng(3).standard_normal((N, N, N))
+    h = 2 * math.pi / N
+    T, _ = oiso.extract(f, 0.4, h)
+    T = np.concatenate([T[:4000 if W < 100 else 70], [[[-1.0, -2.0, 0.5], [9.0, 1.0, 0.1], [2.0, 8.0, 0.3]],     # large, beyond all edges
+                            [[50.0, 1.0, 0.1], [51.0, 2.0, 0.1], [50.0, 3.0, 0.1]],    # outside
+                            [[1.0, 1.0, 0.1], [2.0, 2.0, 0.1], [3.0, 3.0, 0.1]]]])     # no area
+    s = fe.Solver([dict(N=N, tau_p=[], Y0=[])])
+    tri = torch.as_tensor(T.reshape(-1, 9), device="cuda").contiguous()
+    L = share * (N + 1) * h
+    depth = torch.empty((W, W), dtype=torch.float32, device="cuda")
+    fe.fe_raster_depth(s.ctx, tri.data_ptr(), len(T), W, L, depth.data_ptr())
+    assert np.array_equal(depth.cpu().numpy(), oiso.raster_depth(T, W, L))
+    s.close()
