@@ -418,8 +418,8 @@ int fe_plane_streaming_active(const fe_ctx* ctx);
 
 /* Tile depth of the stencil kernels: every kernel launch covers all boxes
  * with 32 x 8-cell column tiles that walk tz z-planes.  fe_set_tiling sets tz
- * for every box, fe_set_box_tiling for one (0 = built-in default: 8 for
- * N >= 128, else 4).  fe_autotune times `trials` trial steps (computed from
+ * for every box, fe_set_box_tiling for one (0 = built-in default, chosen
+ * from the context's boxes so that the tiles fill the multiprocessors).  fe_autotune times `trials` trial steps (computed from
  * the current state and discarded: the state and clock are unchanged) for
  * tz in {4, 8, 16, 24, 32, 48, 64} for all boxes, then, when the boxes have several
  * sizes, for each size in turn (largest first) with the other boxes fixed;

@@ -602,6 +602,9 @@ struct Launch {
   int* rstart = nullptr;  // right-hand-side kernels: also start the refined solve (outer counter)
   int ysum = -1;          // two-way coupling: slot of the dust loading sum_j Y_j^n (-1: one-way)
   int poly = 0;           // streamed CG with the Neumann polynomial preconditioner (needs bwork)
+  const BoxDev* kboxes = nullptr;  // the boxes under the tiling of the Krylov kernels (their sums follow it)
+  const int2* kwork = nullptr;
+  int nkblocks = 0;
   int bcells = 0;         // cells per block of the streamed CG kernels (kBulkCells or kBulkCellsPoly)
 };
 

@@ -1861,14 +1861,14 @@ __global__ void __launch_bounds__(NTHR) k_fcg_matvec(const BoxDev* boxes, const 
 }
 
 // ---- launchers ------------------------------------------------------------------------
-#define GRID L.nblocks, dim3(TX, TY), 0, L.st
+#define GRID L.nkblocks, dim3(TX, TY), 0, L.st  // tile kernels: the Krylov tiling
 #define EGRID L.neblocks, dim3(TX, TY), 0, L.st
 template <typename T> void launch_cg_init(const Launch& L, double) {
   FE_LAUNCH(L, KID_CG_INIT, (k_cg_init<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
 }
 template <typename T> void launch_cg_matvec(const Launch& L) {
-  if (L.transonic) FE_LAUNCH(L, KID_CG_MATVEC, (k_cg_matvec<T><<<GRID>>>(L.boxes, L.work, L.part)));
-  else FE_LAUNCH(L, KID_CG_MATVEC, (kz_cg_matvec<T><<<GRID>>>(L.boxes, L.work, L.part)));
+  if (L.transonic) FE_LAUNCH(L, KID_CG_MATVEC, (k_cg_matvec<T><<<GRID>>>(L.kboxes, L.kwork, L.part)));
+  else FE_LAUNCH(L, KID_CG_MATVEC, (kz_cg_matvec<T><<<GRID>>>(L.kboxes, L.kwork, L.part)));
 }
 template <typename T> void launch_cg_update(const Launch& L) {
   FE_LAUNCH(L, KID_CG_UPDATE, (k_cg_update<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
@@ -1886,8 +1886,8 @@ template <typename T> void launch_cg_fused(const Launch& L) {
       FE_LAUNCH(L, KID_CG_RUPDATE, (kb_cg_rpoly<T, false, kBulkCells><<<L.nbblocks, kBulkThreads, L.bsmem, L.st>>>(
                                        L.boxes, L.bwork, L.part, L.active)));
     } else {
-      FE_LAUNCH(L, KID_CG_DIRMATVEC, (kz_cg_dirmatvec<T, true><<<GRID>>>(L.boxes, L.work, L.part)));
-      FE_LAUNCH(L, KID_CG_RUPDATE, (kz_cg_rpoly<T, false><<<GRID>>>(L.boxes, L.work, L.part, L.active)));
+      FE_LAUNCH(L, KID_CG_DIRMATVEC, (kz_cg_dirmatvec<T, true><<<GRID>>>(L.kboxes, L.kwork, L.part)));
+      FE_LAUNCH(L, KID_CG_RUPDATE, (kz_cg_rpoly<T, false><<<GRID>>>(L.kboxes, L.kwork, L.part, L.active)));
     }
     return;
   }
@@ -1895,7 +1895,7 @@ template <typename T> void launch_cg_fused(const Launch& L) {
     FE_LAUNCH(L, KID_CG_DIRMATVEC, (kb_cg_dirmatvec<T, false, kBulkCells><<<L.nbblocks, kBulkThreads, L.bsmem, L.st>>>(
                                        L.boxes, L.bwork, L.part)));
   else
-    FE_LAUNCH(L, KID_CG_DIRMATVEC, (kz_cg_dirmatvec<T, false><<<GRID>>>(L.boxes, L.work, L.part)));
+    FE_LAUNCH(L, KID_CG_DIRMATVEC, (kz_cg_dirmatvec<T, false><<<GRID>>>(L.kboxes, L.kwork, L.part)));
   FE_LAUNCH(L, KID_CG_RUPDATE, (k_cg_rupdate<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
 }
 // First polynomial-preconditioned residual z = P r of an inner solve and <r, z> (nothing without it)
@@ -1908,7 +1908,7 @@ template <typename T> void launch_cg_start(const Launch& L) {
     FE_LAUNCH(L, KID_CG_START, (kb_cg_rpoly<T, true, kBulkCells><<<L.nbblocks, kBulkThreads, L.bsmem, L.st>>>(
                                    L.boxes, L.bwork, L.part, L.active)));
   else
-    FE_LAUNCH(L, KID_CG_START, (kz_cg_rpoly<T, true><<<GRID>>>(L.boxes, L.work, L.part, L.active)));
+    FE_LAUNCH(L, KID_CG_START, (kz_cg_rpoly<T, true><<<GRID>>>(L.kboxes, L.kwork, L.part, L.active)));
 }
 template <typename T> void launch_cg_xfinal(const Launch& L) {
   FE_LAUNCH(L, KID_CG_XFINAL, (k_cg_xfinal<T><<<EGRID>>>(L.boxes, L.ework)));
@@ -1917,37 +1917,37 @@ template <typename T> void launch_cg_dir(const Launch& L) {
   FE_LAUNCH(L, KID_CG_DIR, (k_cg_dir<T><<<EGRID>>>(L.boxes, L.ework)));
 }
 template <typename T> void launch_true_res(const Launch& L, int xs) {
-  FE_LAUNCH(L, KID_TRUE_RES, (k_true_res<T><<<GRID>>>(L.boxes, L.work, L.part, xs)));
+  FE_LAUNCH(L, KID_TRUE_RES, (k_true_res<T><<<GRID>>>(L.kboxes, L.kwork, L.part, xs)));
 }
 template <typename T> void launch_bicg_init(const Launch& L) {
-  FE_LAUNCH(L, KID_BICG_INIT, (k_bicg_init<T><<<GRID>>>(L.boxes, L.work, L.part, L.active)));
+  FE_LAUNCH(L, KID_BICG_INIT, (k_bicg_init<T><<<GRID>>>(L.kboxes, L.kwork, L.part, L.active)));
 }
 template <typename T> void launch_bicg_p(const Launch& L) {
-  FE_LAUNCH(L, KID_BICG_P, (k_bicg_p<T><<<GRID>>>(L.boxes, L.work)));
+  FE_LAUNCH(L, KID_BICG_P, (k_bicg_p<T><<<GRID>>>(L.kboxes, L.kwork)));
 }
 template <typename T> void launch_bicg_v(const Launch& L) {
-  FE_LAUNCH(L, KID_BICG_V, (k_bicg_v<T><<<GRID>>>(L.boxes, L.work, L.part)));
+  FE_LAUNCH(L, KID_BICG_V, (k_bicg_v<T><<<GRID>>>(L.kboxes, L.kwork, L.part)));
 }
 template <typename T> void launch_bicg_s(const Launch& L) {
-  FE_LAUNCH(L, KID_BICG_S, (k_bicg_s<T><<<GRID>>>(L.boxes, L.work)));
-  FE_LAUNCH(L, KID_BICG_T, (k_bicg_t<T><<<GRID>>>(L.boxes, L.work, L.part)));
+  FE_LAUNCH(L, KID_BICG_S, (k_bicg_s<T><<<GRID>>>(L.kboxes, L.kwork)));
+  FE_LAUNCH(L, KID_BICG_T, (k_bicg_t<T><<<GRID>>>(L.kboxes, L.kwork, L.part)));
 }
 template <typename T> void launch_bicg_x(const Launch& L) {
-  FE_LAUNCH(L, KID_BICG_X, (k_bicg_x<T><<<GRID>>>(L.boxes, L.work, L.part, L.active)));
+  FE_LAUNCH(L, KID_BICG_X, (k_bicg_x<T><<<GRID>>>(L.kboxes, L.kwork, L.part, L.active)));
 }
 template <typename T> void launch_fcg(const Launch& L, const float* z) {
   FE_LAUNCH(L, KID_FCG_DOTS, (k_fcg_dots<T><<<EGRID>>>(L.boxes, L.ework, L.part, z)));
   FE_LAUNCH(L, KID_FCG_DIR, (k_fcg_dir<T><<<EGRID>>>(L.boxes, L.ework, z)));
-  FE_LAUNCH(L, KID_FCG_MATVEC, (k_fcg_matvec<T><<<GRID>>>(L.boxes, L.work, L.part)));
+  FE_LAUNCH(L, KID_FCG_MATVEC, (k_fcg_matvec<T><<<GRID>>>(L.kboxes, L.kwork, L.part)));
   FE_LAUNCH(L, KID_CG_UPDATE, (k_cg_update<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
 }
 template <typename T> void launch_mix_residual(const Launch& L, int first, int* outer_active) {
   if (first)
     FE_LAUNCH(L, KID_MIX_RES, (k_mix_first<T><<<EGRID>>>(L.boxes, L.ework, L.part, outer_active)));
   else if (L.transonic)
-    FE_LAUNCH(L, KID_MIX_RES, (k_mix_residual<T><<<GRID>>>(L.boxes, L.work, L.part, first, outer_active)));
+    FE_LAUNCH(L, KID_MIX_RES, (k_mix_residual<T><<<GRID>>>(L.kboxes, L.kwork, L.part, first, outer_active)));
   else
-    FE_LAUNCH(L, KID_MIX_RES, (kz_mix_residual<T><<<GRID>>>(L.boxes, L.work, L.part, outer_active)));
+    FE_LAUNCH(L, KID_MIX_RES, (kz_mix_residual<T><<<GRID>>>(L.kboxes, L.kwork, L.part, outer_active)));
 }
 template <typename T> void launch_refine_start(const Launch& L, int* outer_active) {
   FE_LAUNCH(L, KID_MIX_RES, (k_refine_start<T><<<EGRID>>>(L.boxes, L.ework, L.part, outer_active, L.active)));
@@ -1956,10 +1956,10 @@ template <typename T> void launch_refine_start(const Launch& L, int* outer_activ
 template <typename T> void launch_refine(const Launch& L, int* outer_active) {
   if (L.ring_ok)  // every box's N a multiple of the 16-byte chunk, so even: column pairs
     FE_LAUNCH(L, KID_REFINE,
-              (kp_refine<T><<<L.nblocks, dim3(RTX, TY), 0, L.st>>>(L.boxes, L.work, L.part, outer_active, L.active,
+              (kp_refine<T><<<L.nkblocks, dim3(RTX, TY), 0, L.st>>>(L.kboxes, L.kwork, L.part, outer_active, L.active,
                                                                      L.poly)));
   else
-    FE_LAUNCH(L, KID_REFINE, (kz_refine<T><<<GRID>>>(L.boxes, L.work, L.part, outer_active, L.active, L.poly)));
+    FE_LAUNCH(L, KID_REFINE, (kz_refine<T><<<GRID>>>(L.kboxes, L.kwork, L.part, outer_active, L.active, L.poly)));
   launch_cg_start<T>(L);
 }
 template <typename T> void launch_mix_finish_pp(const Launch& L) {
