@@ -37,6 +37,8 @@ size_t iso_work_bytes(int N);
 size_t raster_work_bytes(int W);
 int raster_depth(const double* tri, long long ntri, int W, double extent, float* depth, void* work, int nsm,
                  cudaStream_t st);
+int persist_plan(const int* N, int nb, int nsm, bool bicg, std::vector<int4>& work, long* units, int* upc);
+size_t persist_packet_bytes(long units);
 UNet* unet_create(int N, bool training, int* rc);
 void unet_destroy(UNet* U);
 long unet_param_count();
@@ -86,7 +88,7 @@ static const char* kKernelNames[] = {
     "dust",    "derive",    "cg_init",   "cg_matvec", "cg_update", "cg_dir", "true_res", "bicg_init",
     "bicg_p",  "bicg_v",    "bicg_s",    "bicg_t", "bicg_x",   "commit",    "dinv",
     "mix_residual", "mix_accum", "mix_finish", "fcg_dots", "fcg_dir", "fcg_matvec",
-    "cg_dirmatvec", "cg_rupdate", "cg_xfinal", "refine", "unet", "tf_pred", "tf_corr", "fe_cell", "fe_face", "cg_start",
+    "cg_dirmatvec", "cg_rupdate", "cg_xfinal", "refine", "unet", "tf_pred", "tf_corr", "fe_cell", "fe_face", "cg_start", "solve",
     "other"};
 static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == KID_COUNT, "kernel name table");
 static_assert(KID_COUNT <= FE_PROFILE_MAX_KERNELS, "profile counters");
@@ -107,6 +109,10 @@ struct fe_ctx {
   BoxDev* dkbox = nullptr;  // FP64 default tiling: the Krylov kernels' own tiles (null: the step's)
   int2* dkwork = nullptr;
   int nkblocks = 0;
+  int4* dpwork = nullptr;   // one-launch FP64 solve (null: the boxes do not fit): blocks, packets
+  unsigned long long* dpackets = nullptr;
+  int npblocks = 0, pupc = 0;
+  long punits = 0;
   int2* dework = nullptr;
   int2* dbwork = nullptr;   // plane-streaming blocks (box, block of box)
   int nbblocks = 0, bsmem = 0, bcells = 0, npart = 0;
@@ -153,6 +159,11 @@ struct fe_ctx {
              nbblocks, bsmem};
     l.poly = prm.solver == FE_PCG_POLY && !fp64;  // FP64 contexts run Jacobi-PCG
     l.bcells = bcells;
+    l.pwork = dpwork;
+    l.npblocks = npblocks;
+    l.pupc = pupc;
+    l.packets = dpackets;
+    l.punits = punits;
     l.kboxes = dkbox ? dkbox : dbox;
     l.kwork = dkbox ? dkwork : dwork;
     l.nkblocks = dkbox ? nkblocks : nblocks;
@@ -536,6 +547,20 @@ extern "C" int fe_create(const fe_params* prm, void* stream, fe_ctx** out) {
         cudaMallocHost(&c->gm_hpart, parts * sizeof(double)) != cudaSuccess)
       rc = FE_ERR_OOM;
   }
+  if (rc == FE_OK && c->fp64 &&
+      (prm->solver == FE_PCG_JACOBI || prm->solver == FE_PCG_POLY || prm->solver == FE_BICGSTAB_JACOBI)) {
+    std::vector<int4> pwork;
+    c->npblocks = persist_plan(c->N.data(), nb, c->nsm, prm->solver == FE_BICGSTAB_JACOBI, pwork, &c->punits, &c->pupc);
+    if (c->npblocks > 0) {
+      if (cudaMalloc(&c->dpwork, pwork.size() * sizeof(int4)) != cudaSuccess ||
+          cudaMalloc(&c->dpackets, persist_packet_bytes(c->punits)) != cudaSuccess)
+        rc = FE_ERR_OOM;
+      else if (cudaMemcpyAsync(c->dpwork, pwork.data(), pwork.size() * sizeof(int4), cudaMemcpyHostToDevice, c->st) !=
+                   cudaSuccess ||
+               cudaStreamSynchronize(c->st) != cudaSuccess)
+        rc = FE_ERR_CUDA;
+    }
+  }
   if (rc == FE_OK) rc = set_tiling(c, 0);
   if (rc != FE_OK) {
     fe_destroy(c);
@@ -560,6 +585,8 @@ extern "C" void fe_destroy(fe_ctx* c) {
   cudaFree(c->dwork);
   cudaFree(c->dkbox);
   cudaFree(c->dkwork);
+  cudaFree(c->dpwork);
+  cudaFree(c->dpackets);
   cudaFree(c->dework);
   cudaFree(c->dbwork);
   cudaFree(c->dpart);
@@ -633,8 +660,9 @@ __global__ void k_sub_from(const T* a, T* y, long n) {
 template <typename T>
 static int krylov(fe_ctx* c, int maxit, int key) {
   Launch L = c->L();
-  CK(cudaMemsetAsync(c->dactive, 0, sizeof(int), c->st));
   const bool bicg = c->prm.solver == FE_BICGSTAB_JACOBI;
+  if (sizeof(T) == 8 && L.pwork && !c->harvest_b) return launch_persist(L, bicg);
+  CK(cudaMemsetAsync(c->dactive, 0, sizeof(int), c->st));
   if (bicg) launch_bicg_init<T>(L);
   else launch_cg_init<T>(L, 0.0);
   int it = 0;
@@ -1027,8 +1055,9 @@ static int krylov_graph(fe_ctx* c, int lev) {
   Launch L = c->L();
   L.st = cs;
   const int maxit = c->prm.p_maxit;
-  CK(cudaMemsetAsync(c->dactive, 0, sizeof(int), cs));
   const bool bicg = c->prm.solver == FE_BICGSTAB_JACOBI;
+  if (sizeof(T) == 8 && L.pwork) return launch_persist(L, bicg);
+  CK(cudaMemsetAsync(c->dactive, 0, sizeof(int), cs));
   const bool learned = c->prm.solver == FE_FCG_LEARNED;
   BoxDev& B0 = c->hbox[0];
   if (bicg) launch_bicg_init<T>(L);

@@ -574,7 +574,7 @@ enum KernelId {
   KID_BICG_INIT, KID_BICG_P, KID_BICG_V, KID_BICG_S, KID_BICG_T, KID_BICG_X,
   KID_COMMIT, KID_DINV, KID_MIX_RES, KID_MIX_ACC, KID_MIX_FIN, KID_FCG_DOTS, KID_FCG_DIR, KID_FCG_MATVEC,
   KID_CG_DIRMATVEC, KID_CG_RUPDATE, KID_CG_XFINAL, KID_REFINE, KID_UNET, KID_TF_PRED, KID_TF_CORR, KID_FE_CELL,
-  KID_FE_FACE, KID_CG_START, KID_OTHER,
+  KID_FE_FACE, KID_CG_START, KID_SOLVE, KID_OTHER,
   KID_COUNT
 };
 
@@ -605,6 +605,10 @@ struct Launch {
   const BoxDev* kboxes = nullptr;  // the boxes under the tiling of the Krylov kernels (their sums follow it)
   const int2* kwork = nullptr;
   int nkblocks = 0;
+  const int4* pwork = nullptr;     // blocks of the one-launch FP64 solve (null: the boxes do not fit)
+  int npblocks = 0, pupc = 0;      // their number, units per block
+  unsigned long long* packets = nullptr;
+  long punits = 0;
   int bcells = 0;         // cells per block of the streamed CG kernels (kBulkCells or kBulkCellsPoly)
 };
 
@@ -672,6 +676,7 @@ template <typename V> void launch_bicg_p(const Launch& L);
 template <typename V> void launch_bicg_v(const Launch& L);
 template <typename V> void launch_bicg_s(const Launch& L);
 template <typename V> void launch_bicg_x(const Launch& L);
+int launch_persist(const Launch& L, bool bicg);  // krylov_persist.cu: whole FP64 solves of small boxes
 template <typename V> void launch_mix_residual(const Launch& L, int first, int* outer_active);
 template <typename V> void launch_mix_accum(const Launch& L);
 template <typename V> void launch_mix_finish(const Launch& L);

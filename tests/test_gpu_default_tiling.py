@@ -45,3 +45,37 @@ def test_default_depth_matches_an_explicit_one(fe, sizes, fp64):
             assert np.linalg.norm(p - q) <= bar * np.linalg.norm(q)
         if fp64:
             assert out[0][1][b]["iters"] == out[1][1][b]["iters"]
+
+
+@pytest.mark.parametrize("transonic", [False, True])
+@pytest.mark.parametrize("N", [8, 9, 24, 45, 53, 67, 84, 86])
+def test_one_launch_solves(fe, N, transonic):
+    """The FP64 solves of small boxes in one launch (up to 8 units of 256 cells per block, 4 for BiCGStab; larger
+    boxes run kernel by kernel) against the oracle's: ragged last units, one to many units per block, both sides of
+    the limits.  A solution to residual 1e-12 of a system of condition number below 10 is within 1e-11; iteration
+    counts agree up to the rounding of the stopping test."""
+    import torch
+    from oracle import krylov, piso
+    from paper_1404_0959_gb300.inputs import random_vector
+    rho, u, Y, _ = random_fields(N, 1, False, seed=N, mach=0.3, noise=0.01)
+    s = fe.Solver([dict(N=N, nu=0.005, tau_p=[0.05], Y0=[0.01])], transonic=transonic,
+                  solver=fe.FE_BICGSTAB_JACOBI if transonic else fe.FE_PCG_JACOBI)
+    s.set_state(0, rho, u, Y)
+    prm = piso.Params(N=N, nu=0.005, transonic=transonic, p_tol=1e-12)
+    st = piso.make_state(prm, rho, u, Y)
+    psi = piso.compressibility(prm, st["rho"], st["p"])
+    dt = piso.time_step(prm, st["u"], float("inf"))
+    M, diag = piso.helmholtz(prm, psi, dt, st["u"] if transonic else None)
+    b = random_vector(N, 100 + N)
+    xr, itr, _, _ = (krylov.bicgstab if transonic else krylov.pcg)(M, b, diag, 1e-12, 500)
+    bd = torch.as_tensor(b, device="cuda")
+    for _ in range(2):  # the second call finds the first one's packets and vectors
+        code, x, info = s.solve_pressure(0, bd, dt, 1e-12, 500)
+        assert code == fe.FE_OK and abs(info.iters - itr) <= 1 and info.rel_res_true <= 2e-12
+        x = x.cpu().numpy()
+        assert np.linalg.norm(x - xr) <= 1e-11 * np.linalg.norm(xr)
+    code, x, info = s.solve_pressure(0, bd, dt, 1e-12, 2)  # the cap is a verdict, not a hang
+    assert code == fe.FE_ERR_NOT_CONVERGED and info.iters == 2
+    code, x, info = s.solve_pressure(0, torch.zeros_like(bd), dt, 1e-12, 50)
+    assert code == fe.FE_OK and info.iters == 0 and not x.any()
+    s.close()
