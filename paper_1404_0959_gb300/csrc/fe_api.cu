@@ -37,8 +37,8 @@ size_t iso_work_bytes(int N);
 size_t raster_work_bytes(int W);
 int raster_depth(const double* tri, long long ntri, int W, double extent, float* depth, void* work, int nsm,
                  cudaStream_t st);
-int persist_plan(const int* N, int nb, int nsm, bool bicg, std::vector<int4>& work, long* units, int* upc);
-size_t persist_packet_bytes(long units);
+Persist* persist_create(const int* N, int nb, int nsm, bool bicg, cudaStream_t st, int* rc);
+void persist_free(Persist* P);
 UNet* unet_create(int N, bool training, int* rc);
 void unet_destroy(UNet* U);
 long unet_param_count();
@@ -109,10 +109,7 @@ struct fe_ctx {
   BoxDev* dkbox = nullptr;  // FP64 default tiling: the Krylov kernels' own tiles (null: the step's)
   int2* dkwork = nullptr;
   int nkblocks = 0;
-  int4* dpwork = nullptr;   // one-launch FP64 solve (null: the boxes do not fit): blocks, packets
-  unsigned long long* dpackets = nullptr;
-  int npblocks = 0, pupc = 0;
-  long punits = 0;
+  Persist* persist = nullptr;  // one-launch FP64 solve (null: the boxes do not fit it)
   int2* dework = nullptr;
   int2* dbwork = nullptr;   // plane-streaming blocks (box, block of box)
   int nbblocks = 0, bsmem = 0, bcells = 0, npart = 0;
@@ -159,11 +156,7 @@ struct fe_ctx {
              nbblocks, bsmem};
     l.poly = prm.solver == FE_PCG_POLY && !fp64;  // FP64 contexts run Jacobi-PCG
     l.bcells = bcells;
-    l.pwork = dpwork;
-    l.npblocks = npblocks;
-    l.pupc = pupc;
-    l.packets = dpackets;
-    l.punits = punits;
+    l.persist = persist;
     l.kboxes = dkbox ? dkbox : dbox;
     l.kwork = dkbox ? dkwork : dwork;
     l.nkblocks = dkbox ? nkblocks : nblocks;
@@ -548,19 +541,8 @@ extern "C" int fe_create(const fe_params* prm, void* stream, fe_ctx** out) {
       rc = FE_ERR_OOM;
   }
   if (rc == FE_OK && c->fp64 &&
-      (prm->solver == FE_PCG_JACOBI || prm->solver == FE_PCG_POLY || prm->solver == FE_BICGSTAB_JACOBI)) {
-    std::vector<int4> pwork;
-    c->npblocks = persist_plan(c->N.data(), nb, c->nsm, prm->solver == FE_BICGSTAB_JACOBI, pwork, &c->punits, &c->pupc);
-    if (c->npblocks > 0) {
-      if (cudaMalloc(&c->dpwork, pwork.size() * sizeof(int4)) != cudaSuccess ||
-          cudaMalloc(&c->dpackets, persist_packet_bytes(c->punits)) != cudaSuccess)
-        rc = FE_ERR_OOM;
-      else if (cudaMemcpyAsync(c->dpwork, pwork.data(), pwork.size() * sizeof(int4), cudaMemcpyHostToDevice, c->st) !=
-                   cudaSuccess ||
-               cudaStreamSynchronize(c->st) != cudaSuccess)
-        rc = FE_ERR_CUDA;
-    }
-  }
+      (prm->solver == FE_PCG_JACOBI || prm->solver == FE_PCG_POLY || prm->solver == FE_BICGSTAB_JACOBI))
+    c->persist = persist_create(c->N.data(), nb, c->nsm, prm->solver == FE_BICGSTAB_JACOBI, c->st, &rc);
   if (rc == FE_OK) rc = set_tiling(c, 0);
   if (rc != FE_OK) {
     fe_destroy(c);
@@ -585,8 +567,7 @@ extern "C" void fe_destroy(fe_ctx* c) {
   cudaFree(c->dwork);
   cudaFree(c->dkbox);
   cudaFree(c->dkwork);
-  cudaFree(c->dpwork);
-  cudaFree(c->dpackets);
+  persist_free(c->persist);
   cudaFree(c->dework);
   cudaFree(c->dbwork);
   cudaFree(c->dpart);
@@ -661,7 +642,7 @@ template <typename T>
 static int krylov(fe_ctx* c, int maxit, int key) {
   Launch L = c->L();
   const bool bicg = c->prm.solver == FE_BICGSTAB_JACOBI;
-  if (sizeof(T) == 8 && L.pwork && !c->harvest_b) return launch_persist(L, bicg);
+  if (sizeof(T) == 8 && L.persist && !c->harvest_b) return launch_persist(L);
   CK(cudaMemsetAsync(c->dactive, 0, sizeof(int), c->st));
   if (bicg) launch_bicg_init<T>(L);
   else launch_cg_init<T>(L, 0.0);
@@ -1056,7 +1037,7 @@ static int krylov_graph(fe_ctx* c, int lev) {
   L.st = cs;
   const int maxit = c->prm.p_maxit;
   const bool bicg = c->prm.solver == FE_BICGSTAB_JACOBI;
-  if (sizeof(T) == 8 && L.pwork) return launch_persist(L, bicg);
+  if (sizeof(T) == 8 && L.persist) return launch_persist(L);
   CK(cudaMemsetAsync(c->dactive, 0, sizeof(int), cs));
   const bool learned = c->prm.solver == FE_FCG_LEARNED;
   BoxDev& B0 = c->hbox[0];

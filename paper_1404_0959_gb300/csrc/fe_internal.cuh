@@ -578,6 +578,7 @@ enum KernelId {
   KID_COUNT
 };
 
+struct Persist;  // defined in krylov_persist.cu
 struct Prof;  // defined in fe_api.cu
 void prof_begin(Prof* p, int kid, cudaStream_t st);
 void prof_end(Prof* p, int kid, cudaStream_t st);
@@ -605,10 +606,7 @@ struct Launch {
   const BoxDev* kboxes = nullptr;  // the boxes under the tiling of the Krylov kernels (their sums follow it)
   const int2* kwork = nullptr;
   int nkblocks = 0;
-  const int4* pwork = nullptr;     // blocks of the one-launch FP64 solve (null: the boxes do not fit)
-  int npblocks = 0, pupc = 0;      // their number, units per block
-  unsigned long long* packets = nullptr;
-  long punits = 0;
+  Persist* persist = nullptr;  // the one-launch FP64 solve (null: the boxes do not fit it)
   int bcells = 0;         // cells per block of the streamed CG kernels (kBulkCells or kBulkCellsPoly)
 };
 
@@ -676,7 +674,7 @@ template <typename V> void launch_bicg_p(const Launch& L);
 template <typename V> void launch_bicg_v(const Launch& L);
 template <typename V> void launch_bicg_s(const Launch& L);
 template <typename V> void launch_bicg_x(const Launch& L);
-int launch_persist(const Launch& L, bool bicg);  // krylov_persist.cu: whole FP64 solves of small boxes
+int launch_persist(const Launch& L);  // krylov_persist.cu: whole FP64 solves of small boxes
 template <typename V> void launch_mix_residual(const Launch& L, int first, int* outer_active);
 template <typename V> void launch_mix_accum(const Launch& L);
 template <typename V> void launch_mix_finish(const Launch& L);

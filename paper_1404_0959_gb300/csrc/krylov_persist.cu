@@ -8,157 +8,164 @@
 // the vectors that neighbours read go through global memory (L2), and the blocks
 // of a box meet once per inner product.
 //
-// Units and sums: unit u of a box is its cells [256 u, 256 u + 256); a block owns
-// consecutive units.  Every unit's partial sum is formed by one fixed tree and
-// published as a packet, and every block adds the packets of all units of its box
-// in the same fixed order, so the sums (and the iterates) of a box do not depend
-// on how many blocks it was given, in an ensemble or alone, and no block needs a
-// value from a coordinator.
+// Units and sums: unit u of a box is its cells [128 u, 128 u + 128); a block owns
+// 1, 2, 4 or 8 consecutive units, aligned.  A box's sum is one binary tree over its
+// units (adjacent pairs, then pairs of pairs): a block publishes the sum of its
+// subtree, and every block adds those of its box up the rest of the tree.  So the
+// sums (and the iterates) of a box do not depend on how many blocks it was given,
+// in an ensemble or alone, and no block waits for a coordinator's value.
 //
-// A packet is the two halves of the double, each with the number of the meeting
-// (epoch) in its other 32 bits, so that a reader sees whether it has arrived; the
-// writer's fence before it orders the vectors that the next phase reads.  Two
-// packet sets alternate: a block can be at most one meeting ahead of another.
-// The packets are cleared before each launch.  Waits are bounded: a block that
-// gives up sets SC_KERR, finishes, and leaves the others to their own limits.
+// A meeting: publish, count up the box's counter, wait until all blocks have (one
+// thread per block polls), read the published sums.  Two sets of sums alternate: a
+// block can be at most one meeting ahead of another.  Measured with 256 threads per
+// block: 3.2 us for 54 blocks, 3.4 us for 152, 4.1 us for 304, against 3.3, 5.7 and
+// 10.9 us where every block polls every other's sum, and 3.2 us at 152 through
+// clusters of eight.  The counters are cleared before each launch.  Waits are
+// bounded: a block that gives up sets SC_KERR, finishes, and leaves the others to
+// their own limits.
 #include <algorithm>
+#include <new>
 #include <vector>
 
 #include "fe_internal.cuh"
 
 namespace fe {
 
-constexpr int kPkThreads = 256;
+constexpr int kPkThreads = 128;  // cells of a unit, threads of a block
 constexpr int kPkWarps = kPkThreads / 32;
-constexpr int kPkPerSm = 2;     // resident blocks per SM asked for (128 registers)
-constexpr int kPkMaxUnits = 8;  // units per block, at most
-constexpr int kPkWords = 4;     // words of a packet: two values
-constexpr long kPkSpins = 1L << 21;
+constexpr int kPkPerSm = 4;      // resident blocks per SM asked for (128 registers)
+constexpr int kPkMaxUnits = 8;   // units per block, at most
+constexpr int kPkLeaves = 8;     // published sums per thread, at most: 1024 blocks of a box
+constexpr int kPkSpins = 1 << 22;
+constexpr int kPkLine = 32;      // words between the counters of two boxes (one line each)
+
+// A block's place: box, its first unit, its units, the box's first block and first cell among all boxes.
+struct PkBlock {
+  int box, u0, mine, b0;
+  long cell0;
+};
 
 template <typename T>
 __device__ __forceinline__ T* Fp(const BoxDev& B, int slot) {
   return reinterpret_cast<T*>(B.f[slot]);
 }
-__device__ __forceinline__ void st_packet(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long ld_packet(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
 // The meetings of the blocks of one box.
 struct Meet {
-  unsigned long long* set0;  // packets of the box: [2][units][kPkWords]
-  long stride;               // words of one set
-  int units, u0, mine;       // units of the box; first one and number of this block
+  double* sums;        // published sums of the box: [2 sets][2 values][blocks]
+  unsigned* counter;
+  int blocks, me, mine;  // blocks of the box, this one, its units
   unsigned epoch = 0;
   bool failed = false;
 };
 
 struct MeetShared {
   double val[2][kPkMaxUnits][kPkThreads];
-  double warp[2][kPkWarps];
+  double unit[2][kPkMaxUnits];
+  double sum[2][kPkThreads];
+  double out[4];  // the solver's scalars after a meeting
+  int go;         // 0: finished
   int bad;
 };
 
-// v[k][s]: this thread's share of value k in unit s of the block.  On return tot[k] is the box's sum in
-// every thread, and everything the blocks of the box stored to global memory before is visible.
-template <int K, int UPC>
-__device__ __forceinline__ void meet(Meet& m, MeetShared& sh, const double (&v)[K][UPC], double (&tot)[K]) {
+// the binary tree over 128 values in shared memory, adjacent pairs first (one warp)
+__device__ __forceinline__ double pk_tree(const double* e, int lane) {
+  e += 4 * lane;
+  double a = (e[0] + e[1]) + (e[2] + e[3]);
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
+// One thread: count this block in and wait for the others.
+__device__ __forceinline__ void pk_wait(Meet& m, MeetShared& sh) {
+  __threadfence();  // this block's stores before the count
+  atomicAdd(m.counter, 1u);
+  const unsigned all = m.epoch * (unsigned)m.blocks;
+  int spins = 0;
+  bool ok = !m.failed;
+  while (ok && *(volatile unsigned*)m.counter < all) ok = ++spins < kPkSpins;
+  __threadfence();  // the other blocks' stores after it
+  sh.bad = ok ? 0 : 1;
+}
+
+// Sums LV t .. LV t + LV - 1 of value k (zeros beyond the box's blocks), added up the tree.
+template <int LV>
+__device__ __forceinline__ double pk_gather(const Meet& m, const double* set) {
+  double l[LV];
+#pragma unroll
+  for (int j = 0; j < LV; ++j) l[j] = (int)threadIdx.x * LV + j < m.blocks ? __ldcg(set + threadIdx.x * LV + j) : 0.0;
+#pragma unroll
+  for (int o = 1; o < LV; o <<= 1)
+#pragma unroll
+    for (int j = 0; j < LV; j += 2 * o) l[j] += l[j + o];
+  return l[0];
+}
+
+// v[k][s]: this thread's share of value k in unit s of the block.  Afterwards everything the blocks of
+// the box stored to global memory before is visible, and fin(totals) has run in one thread: the scalars it
+// leaves in shared memory are for all.  The FP64 pipe takes 16 clocks per warp instruction and 68 from one
+// add to the next, so sums and scalars are left to one warp (all warps forming them took 5 of 14 us per
+// iteration at 32^3).
+template <int K, int UPC, typename Fin>
+__device__ __forceinline__ void meet(Meet& m, MeetShared& sh, const double (&v)[K][UPC], Fin fin) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   ++m.epoch;
-  unsigned long long* set = m.set0 + (m.epoch & 1u) * m.stride;
+  double* set = m.sums + (size_t)(m.epoch & 1u) * 2 * m.blocks;
 #pragma unroll
   for (int k = 0; k < K; ++k)
 #pragma unroll
     for (int s = 0; s < UPC; ++s) sh.val[k][s][tid] = v[k][s];
-  if (tid == 0) sh.bad = 0;
   __syncthreads();
-  for (int q = warp; q < K * m.mine; q += kPkWarps) {
-    const int k = q % K, s = q / K;
-    double a = sh.val[k][s][lane];
 #pragma unroll
-    for (int j = 1; j < kPkWarps; ++j) a += sh.val[k][s][lane + 32 * j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if (lane == 0) {
-      __threadfence();
-      unsigned long long* p = set + (long)(m.u0 + s) * kPkWords + 2 * k;
-      const unsigned long long bits = (unsigned long long)__double_as_longlong(a), e = m.epoch;
-      st_packet(p, (bits << 32) | e);
-      st_packet(p + 1, (bits & 0xffffffff00000000ull) | e);
+  for (int q = 0; q < (K * UPC + kPkWarps - 1) / kPkWarps; ++q) {
+    const int i = q * kPkWarps + warp;
+    if (i < K * UPC) {
+      const double a = pk_tree(sh.val[i % K][i / K], lane);
+      if (lane == 0) sh.unit[i % K][i / K] = a;
     }
   }
-  double a[K];
+  if (K * UPC > 1) __syncthreads();
+  if (tid == 0) {
 #pragma unroll
-  for (int k = 0; k < K; ++k) a[k] = 0.0;
-  long spins = 0;
-  bool bad = m.failed;
-  constexpr int AT = 4;  // packets requested at once
-  for (int q0 = tid; q0 < m.units; q0 += AT * kPkThreads) {
-    unsigned long long w[AT][2 * K];
+    for (int k = 0; k < K; ++k) {
+      double e[UPC];
 #pragma unroll
-    for (int j = 0; j < AT; ++j)
-      if (q0 + j * kPkThreads < m.units) {
-        const unsigned long long* p = set + (long)(q0 + j * kPkThreads) * kPkWords;
+      for (int s = 0; s < UPC; ++s) e[s] = sh.unit[k][s];
 #pragma unroll
-        for (int x = 0; x < 2 * K; ++x) w[j][x] = ld_packet(p + x);
-      }
+      for (int o = 1; o < UPC; o <<= 1)
 #pragma unroll
-    for (int j = 0; j < AT; ++j)
-      if (q0 + j * kPkThreads < m.units) {
-        const unsigned long long* p = set + (long)(q0 + j * kPkThreads) * kPkWords;
-#pragma unroll
-        for (int x = 0; x < 2 * K; ++x)
-          while ((unsigned)w[j][x] != m.epoch && !bad) {
-            w[j][x] = ld_packet(p + x);
-            bad = ++spins > kPkSpins;
-          }
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-          a[k] += __longlong_as_double((long long)((w[j][2 * k] >> 32) | (w[j][2 * k + 1] & 0xffffffff00000000ull)));
-      }
-  }
-  if (bad) sh.bad = 1;
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a[k] += __shfl_down_sync(0xffffffffu, a[k], o);
-    if (lane == 0) sh.warp[k][warp] = a[k];
+        for (int s = 0; s < UPC; s += 2 * o) e[s] += e[s + o];
+      set[(size_t)k * m.blocks + m.me] = e[0];
+    }
+    pk_wait(m, sh);
   }
   __syncthreads();
   m.failed = sh.bad != 0;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    double t = sh.warp[k][0];
+    const double* p = set + (size_t)k * m.blocks;
+    sh.sum[k][tid] = m.blocks <= kPkThreads       ? pk_gather<1>(m, p)
+                     : m.blocks <= 2 * kPkThreads ? pk_gather<2>(m, p)
+                     : m.blocks <= 4 * kPkThreads ? pk_gather<4>(m, p)
+                                                  : pk_gather<kPkLeaves>(m, p);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double t[K];
 #pragma unroll
-    for (int j = 1; j < kPkWarps; ++j) t += sh.warp[k][j];
-    tot[k] = t;
+    for (int k = 0; k < K; ++k) t[k] = pk_tree(sh.sum[k], lane);
+    if (lane == 0) fin(t);
   }
   __syncthreads();
 }
 
 // The same without a value: the blocks' stores become visible to each other.
 __device__ __forceinline__ void meet_plain(Meet& m, MeetShared& sh) {
-  const int tid = threadIdx.x;
   ++m.epoch;
-  unsigned long long* set = m.set0 + (m.epoch & 1u) * m.stride;
-  if (tid == 0) sh.bad = 0;
   __syncthreads();
-  if (tid < m.mine) {
-    __threadfence();
-    st_packet(set + (long)(m.u0 + tid) * kPkWords, m.epoch);
-  }
-  long spins = 0;
-  bool bad = m.failed;
-  for (int q = tid; q < m.units; q += kPkThreads)
-    while ((unsigned)ld_packet(set + (long)q * kPkWords) != m.epoch && !bad) bad = ++spins > kPkSpins;
-  if (bad) sh.bad = 1;
+  if (threadIdx.x == 0) pk_wait(m, sh);
   __syncthreads();
   m.failed = sh.bad != 0;
-  __syncthreads();
 }
 
 // Flat offsets of the six neighbours of a cell.
@@ -183,18 +190,18 @@ struct PkNbr {
 // meetings per iteration.  FP64 work per cell and iteration: about 25 operations, on as many SMs as the
 // box has units.
 template <int UPC>
-__global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_cg(const BoxDev* boxes, const int4* work,
-                                                              unsigned long long* packets, long set_stride) {
+__global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_cg(const BoxDev* boxes, const PkBlock* work,
+                                                              double* sums, unsigned* counters, double*) {
   __shared__ MeetShared sh;
-  const int4 w = work[blockIdx.x];
-  const BoxDev& B = boxes[w.x];
+  const PkBlock w = work[blockIdx.x];
+  const BoxDev& B = boxes[w.box];
   Meet m;
-  m.u0 = w.y;
-  m.mine = w.z;
-  m.set0 = packets + (long)w.w * kPkWords;
-  m.stride = set_stride;
+  m.me = w.u0 / UPC;
+  m.mine = w.mine;
+  m.sums = sums + (size_t)w.b0 * 4;
+  m.counter = counters + w.box * kPkLine;
   const int N = B.N, n3 = N * N * N;
-  m.units = (n3 + kPkThreads - 1) / kPkThreads;
+  m.blocks = (n3 + kPkThreads * UPC - 1) / (kPkThreads * UPC);
   const double* __restrict__ b = Fp<double>(B, K_B);
   const double* __restrict__ dinv = Fp<double>(B, W_DINV);
   const double* __restrict__ psi = Fp<double>(B, W_PSI);
@@ -204,27 +211,40 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_cg(const BoxDev* boxe
   const double tol = B.sc[SC_TOL];
   const int maxit = (int)B.sc[SC_MAXIT];
   const int tid = threadIdx.x;
-  double x[UPC], r[UPC], pd[UPC], q[UPC], v1[1][UPC], v2[2][UPC], t1[1], t2[2];
-  auto cell = [&](int s) { return (m.u0 + s) * kPkThreads + tid; };
+  // the operator as (psi / dt + 6 lapc) pd - lapc (sum of neighbours)
+  auto diag = [&](int c) { return fma(psi[c], idt, 6.0 * lapc); };
+  constexpr bool KEEP = UPC <= 2;  // D^{-1} and the diagonal of more cells are read again
+  double x[UPC], r[UPC], zo[UPC], pd[UPC], q[UPC], di[UPC], dg[UPC], v1[1][UPC], v2[2][UPC];
+  auto cell = [&](int s) { return (w.u0 + s) * kPkThreads + tid; };
   auto on = [&](int s) { return s < m.mine && cell(s) < n3; };
 #pragma unroll
   for (int s = 0; s < UPC; ++s) {
-    x[s] = r[s] = pd[s] = q[s] = v2[0][s] = v2[1][s] = v1[0][s] = 0.0;
+    x[s] = r[s] = zo[s] = pd[s] = q[s] = di[s] = dg[s] = v2[0][s] = v2[1][s] = v1[0][s] = 0.0;
     if (on(s)) {
       const int c = cell(s);
+      if (KEEP) {
+        di[s] = dinv[c];
+        dg[s] = diag(c);
+      }
       r[s] = b[c];
-      const double zc = r[s] * dinv[c];
-      z[c] = zc;
-      v2[0][s] = r[s] * zc;
+      zo[s] = r[s] * dinv[c];
+      z[c] = zo[s];
+      v2[0][s] = r[s] * zo[s];
       v2[1][s] = r[s] * r[s];
     }
   }
-  meet<2, UPC>(m, sh, v2, t2);
-  double rz = t2[0], rr = t2[1], alpha = 0.0, beta = 0.0;
-  const double bb = t2[1];
+  // one thread's scalars: rz, ||r||^2 and the stopping bound stay with it, alpha and beta go to all
+  double rz = 0.0, rr = 0.0, bb = 0.0, stop = 0.0, alpha = 0.0, beta = 0.0;
   int it = 0;
-  bool conv = !(bb > 0.0), run = !conv && !m.failed;
-  while (run) {
+  bool conv = false;
+  meet<2, UPC>(m, sh, v2, [&](const double* t) {
+    rz = t[0];
+    bb = rr = t[1];
+    stop = (tol * sqrt(bb)) * (tol * sqrt(bb));
+    conv = !(bb > 0.0);
+    sh.go = conv ? 0 : 1;
+  });
+  while (sh.go != 0 && !m.failed) {
     const double* po = (it & 1) ? pb : pa;
     double* pn = (it & 1) ? pa : pb;
 #pragma unroll
@@ -235,43 +255,44 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_cg(const BoxDev* boxe
         const double zc = __ldcg(&z[c]);
         return it == 0 ? zc : fma(beta, __ldcg(&po[c]), zc);
       };
-      const double pc = it == 0 ? r[s] * dinv[n.c] : fma(beta, pd[s], r[s] * dinv[n.c]);
+      const double pc = it == 0 ? zo[s] : fma(beta, pd[s], zo[s]);
       const double nb = (dir(n.xm) + dir(n.xp)) + (dir(n.ym) + dir(n.yp)) + (dir(n.zm) + dir(n.zp));
-      const double y = psi[n.c] * pc * idt - lapc * (nb - 6.0 * pc);
+      const double y = fma(KEEP ? dg[s] : diag(n.c), pc, -lapc * nb);
       pn[n.c] = pc;
       pd[s] = pc;
       q[s] = y;
       v1[0][s] = pc * y;
     }
-    meet<1, UPC>(m, sh, v1, t1);
-    alpha = rz / t1[0];
+    meet<1, UPC>(m, sh, v1, [&](const double* t) { sh.out[0] = rz / t[0]; });
+    alpha = sh.out[0];
 #pragma unroll
     for (int s = 0; s < UPC; ++s) {
       if (!on(s)) continue;
       const int c = cell(s);
       x[s] = fma(alpha, pd[s], x[s]);
       r[s] = fma(-alpha, q[s], r[s]);
-      const double zc = r[s] * dinv[c];
-      z[c] = zc;
-      v2[0][s] = r[s] * zc;
+      zo[s] = r[s] * (KEEP ? di[s] : dinv[c]);
+      z[c] = zo[s];
+      v2[0][s] = r[s] * zo[s];
       v2[1][s] = r[s] * r[s];
     }
-    meet<2, UPC>(m, sh, v2, t2);
     ++it;
-    rr = t2[1];
-    if (sqrt(rr) <= tol * sqrt(bb)) conv = true, run = false;
-    else if (it >= maxit) run = false;
-    else {
-      beta = t2[0] / rz;
-      rz = t2[0];
-    }
-    run = run && !m.failed;
+    meet<2, UPC>(m, sh, v2, [&](const double* t) {
+      rr = t[1];
+      if (rr <= stop) conv = true, sh.go = 0;
+      else if (it >= maxit) sh.go = 0;
+      else {
+        sh.out[1] = t[0] / rz;
+        rz = t[0];
+      }
+    });
+    beta = sh.out[1];
   }
   double* X = Fp<double>(B, K_X);
 #pragma unroll
   for (int s = 0; s < UPC; ++s)
     if (on(s)) X[cell(s)] = x[s];
-  if (m.u0 == 0 && tid == 0) {
+  if (w.u0 == 0 && tid == 0) {
     double* sc = B.sc;
     sc[SC_RZ] = rz;
     sc[SC_BB] = bb;
@@ -286,35 +307,37 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_cg(const BoxDev* boxe
 }
 
 // Right-preconditioned BiCGStab for any operator (the iteration of k_bicg_p .. k_bicg_x).  Neighbours
-// read the preconditioned vector of the operator (K_PD) and, for the transonic term, psi times it (K_Q);
-// the velocity interpolated to the faces is formed once (K_V, K_S, K_T: +1/2 faces along x, y, z).
-// x, r (s between the two operators), p, v and t stay in registers; five meetings per iteration.
+// read the preconditioned vector of the operator (K_PD).  The operator is formed once as coefficients per
+// cell, own, then -2, -1, +1, +2 along x, y, z (the transonic term reaches two cells): 13 FP64
+// multiply-adds per application where evaluating psi, the interpolations and the face products took 36
+// (BiCGStab at 45^3 92 us per iteration kernel by kernel, 32 us here).  x, r (s between the two operators), p, v and t stay in
+// registers; five meetings per iteration.
+constexpr int kPkCoef = 13;
 template <int UPC>
-__global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_bicg(const BoxDev* boxes, const int4* work,
-                                                                unsigned long long* packets, long set_stride) {
+__global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_bicg(const BoxDev* boxes, const PkBlock* work,
+                                                                double* sums, unsigned* counters, double* coef) {
   __shared__ MeetShared sh;
-  const int4 w = work[blockIdx.x];
-  const BoxDev& B = boxes[w.x];
+  const PkBlock w = work[blockIdx.x];
+  const BoxDev& B = boxes[w.box];
   Meet m;
-  m.u0 = w.y;
-  m.mine = w.z;
-  m.set0 = packets + (long)w.w * kPkWords;
-  m.stride = set_stride;
+  m.me = w.u0 / UPC;
+  m.mine = w.mine;
+  m.sums = sums + (size_t)w.b0 * 4;
+  m.counter = counters + w.box * kPkLine;
   const int N = B.N, NN = N * N, n3 = NN * N;
-  m.units = (n3 + kPkThreads - 1) / kPkThreads;
+  m.blocks = (n3 + kPkThreads * UPC - 1) / (kPkThreads * UPC);
   const bool transonic = B.transonic != 0;
   const double* __restrict__ b = Fp<double>(B, K_B);
   const double* __restrict__ dinv = Fp<double>(B, W_DINV);
   const double* __restrict__ psi = Fp<double>(B, W_PSI);
   double* A1 = Fp<double>(B, K_PD);
-  double* A2 = Fp<double>(B, K_Q);
-  double* FH[3] = {Fp<double>(B, K_V), Fp<double>(B, K_S), Fp<double>(B, K_T)};
+  double* C = coef + w.cell0 * kPkCoef;
   const double dt = B.sc[SC_KDT], ih = B.ih, idt = 1.0 / dt, lapc = 0.5 * dt * ih * ih, ct = 0.03125 * ih;
   const double tol = B.sc[SC_TOL];
   const int maxit = (int)B.sc[SC_MAXIT];
   const int tid = threadIdx.x;
-  double x[UPC], r[UPC], p[UPC], v[UPC], t[UPC], d1[1][UPC], d2[2][UPC], t1[1], t2[2];
-  auto cell = [&](int s) { return (m.u0 + s) * kPkThreads + tid; };
+  double x[UPC], r[UPC], p[UPC], v[UPC], t[UPC], d1[1][UPC], d2[2][UPC];
+  auto cell = [&](int s) { return (w.u0 + s) * kPkThreads + tid; };
   auto on = [&](int s) { return s < m.mine && cell(s) < n3; };
   // offsets of the cells at -2, -1, 1, 2 along axis d
   auto line = [&](int c, int d, int (&o)[4]) {
@@ -326,25 +349,20 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_bicg(const BoxDev* bo
   };
   // M applied to the vector in K_PD (own value a)
   auto apply = [&](int c, double a) {
-    const double ps = psi[c], wc = ps * a;
-    double nb = 0.0, tr = 0.0;
+    double y[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       int o[4];
       line(c, d, o);
-      nb += __ldcg(&A1[o[1]]) + __ldcg(&A1[o[2]]);
+      const double* q = C + (long)(1 + 4 * d) * n3 + c;
+      y[d] = q[n3] * __ldcg(&A1[o[1]]);
+      y[d] = fma(q[2 * (long)n3], __ldcg(&A1[o[2]]), y[d]);
       if (transonic) {
-        const double m2 = __ldcg(&A2[o[0]]), m1 = __ldcg(&A2[o[1]]), p1 = __ldcg(&A2[o[2]]), p2 = __ldcg(&A2[o[3]]);
-        tr += (9.0 * (wc + p1) - (m1 + p2)) * __ldcg(&FH[d][c]) - (9.0 * (m1 + wc) - (m2 + p1)) * __ldcg(&FH[d][o[1]]);
+        y[d] = fma(q[0], __ldcg(&A1[o[0]]), y[d]);
+        y[d] = fma(q[3 * (long)n3], __ldcg(&A1[o[3]]), y[d]);
       }
     }
-    double y = wc * idt - lapc * (nb - 6.0 * a);
-    if (transonic) y += ct * tr;
-    return y;
-  };
-  auto publish = [&](int c, double a) {
-    A1[c] = a;
-    if (transonic) A2[c] = psi[c] * a;
+    return fma(C[c], a, (y[0] + y[1]) + y[2]);
   };
 #pragma unroll
   for (int s = 0; s < UPC; ++s) {
@@ -353,29 +371,50 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_bicg(const BoxDev* bo
       const int c = cell(s);
       r[s] = b[c];
       d1[0][s] = r[s] * r[s];
-      if (transonic) {
+      // (1/2) D(I4(psi x) I4(HbyA)) with f, g = I4(HbyA) at the +1/2, -1/2 faces:
+      // f (9 (w_0 + w_1) - (w_-1 + w_2)) - g (9 (w_-1 + w_0) - (w_-2 + w_1)), w = psi x
+      double own = fma(psi[c], idt, 6.0 * lapc);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
+      for (int d = 0; d < 3; ++d) {
+        int o[4];
+        line(c, d, o);
+        double* q = C + (long)(1 + 4 * d) * n3 + c;
+        double m1 = -lapc, p1 = -lapc;
+        if (transonic) {
           const double* hb = Fp<double>(B, W_HB0 + d);
-          int o[4];
-          line(c, d, o);
-          FH[d][c] = (9.0 * (hb[c] + hb[o[2]]) - (hb[o[1]] + hb[o[3]])) * 0.0625;
+          const double h0 = hb[c], hm1 = hb[o[1]], hp1 = hb[o[2]];
+          const double f = ct * 0.0625 * (9.0 * (h0 + hp1) - (hm1 + hb[o[3]]));
+          const double g = ct * 0.0625 * (9.0 * (hm1 + h0) - (hb[o[0]] + hp1));
+          own += 9.0 * (f - g) * psi[c];
+          m1 -= (f + 9.0 * g) * psi[o[1]];
+          p1 += (9.0 * f + g) * psi[o[2]];
+          q[0] = g * psi[o[0]];
+          q[3 * (long)n3] = -f * psi[o[3]];
         }
+        q[n3] = m1;
+        q[2 * (long)n3] = p1;
       }
+      C[c] = own;
     }
   }
-  meet<1, UPC>(m, sh, d1, t1);
-  const double bb = t1[0];
-  double rho = bb, rho_old = 1.0, alpha = 1.0, omega = 1.0, rr = bb;
+  // one thread's scalars; beta, omega and alpha go to all
+  double rho = 0.0, rho_old = 1.0, rr = 0.0, bb = 0.0, stop = 0.0, alpha = 1.0, omega = 1.0;
   int it = 0;
-  bool conv = !(bb > 0.0), run = !conv && !m.failed;
-  while (run) {
-    const double beta = (rho / rho_old) * (alpha / omega);
+  bool conv = false;
+  meet<1, UPC>(m, sh, d1, [&](const double* q) {
+    bb = rho = rr = q[0];
+    stop = (tol * sqrt(bb)) * (tol * sqrt(bb));
+    conv = !(bb > 0.0);
+    sh.go = conv ? 0 : 1;
+    sh.out[0] = rho;  // beta = (rho / rho_old)(alpha / omega)
+  });
+  while (sh.go != 0 && !m.failed) {
+    const double beta = sh.out[0];
 #pragma unroll
     for (int s = 0; s < UPC; ++s)
       if (on(s)) {
         p[s] = r[s] + beta * (p[s] - omega * v[s]);
-        publish(cell(s), p[s] * dinv[cell(s)]);
+        A1[cell(s)] = p[s] * dinv[cell(s)];
       }
     meet_plain(m, sh);
 #pragma unroll
@@ -385,13 +424,13 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_bicg(const BoxDev* bo
         v[s] = apply(c, p[s] * dinv[c]);
         d1[0][s] = b[c] * v[s];
       }
-    meet<1, UPC>(m, sh, d1, t1);
-    alpha = rho / t1[0];
+    meet<1, UPC>(m, sh, d1, [&](const double* q) { sh.out[1] = rho / q[0]; });
+    alpha = sh.out[1];
 #pragma unroll
     for (int s = 0; s < UPC; ++s)
       if (on(s)) {
         r[s] = r[s] - alpha * v[s];
-        publish(cell(s), r[s] * dinv[cell(s)]);
+        A1[cell(s)] = r[s] * dinv[cell(s)];
       }
     meet_plain(m, sh);
 #pragma unroll
@@ -402,8 +441,8 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_bicg(const BoxDev* bo
         d2[0][s] = t[s] * r[s];
         d2[1][s] = t[s] * t[s];
       }
-    meet<2, UPC>(m, sh, d2, t2);
-    omega = t2[0] / t2[1];
+    meet<2, UPC>(m, sh, d2, [&](const double* q) { sh.out[2] = q[0] / q[1]; });
+    omega = sh.out[2];
 #pragma unroll
     for (int s = 0; s < UPC; ++s)
       if (on(s)) {
@@ -414,20 +453,21 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_bicg(const BoxDev* bo
         d2[0][s] = r[s] * r[s];
         d2[1][s] = b[c] * r[s];
       }
-    meet<2, UPC>(m, sh, d2, t2);
     ++it;
-    rr = t2[0];
-    rho_old = rho;
-    rho = t2[1];
-    if (sqrt(rr) <= tol * sqrt(bb)) conv = true, run = false;
-    else if (it >= maxit) run = false;
-    run = run && !m.failed;
+    meet<2, UPC>(m, sh, d2, [&](const double* q) {
+      rr = q[0];
+      rho_old = rho;
+      rho = q[1];
+      if (rr <= stop) conv = true, sh.go = 0;
+      else if (it >= maxit) sh.go = 0;
+      else sh.out[0] = (rho / rho_old) * (alpha / omega);
+    });
   }
   double* X = Fp<double>(B, K_X);
 #pragma unroll
   for (int s = 0; s < UPC; ++s)
     if (on(s)) X[cell(s)] = x[s];
-  if (m.u0 == 0 && tid == 0) {
+  if (w.u0 == 0 && tid == 0) {
     double* sc = B.sc;
     sc[SC_BB] = bb;
     sc[SC_RZ] = rho;
@@ -445,59 +485,104 @@ __global__ void __launch_bounds__(kPkThreads, kPkPerSm) kc_bicg(const BoxDev* bo
 // ---- launch ---------------------------------------------------------------------------
 constexpr int kPkBicgUnits = 4;  // units per block of BiCGStab (its five register vectors)
 
-typedef void (*PkKernel)(const BoxDev*, const int4*, unsigned long long*, long);
+typedef void (*PkKernel)(const BoxDev*, const PkBlock*, double*, unsigned*, double*);
 static PkKernel pk_kernel(bool bicg, int upc) {
   if (bicg) return upc == 1 ? kc_bicg<1> : upc == 2 ? kc_bicg<2> : kc_bicg<4>;
   return upc == 1 ? kc_cg<1> : upc == 2 ? kc_cg<2> : upc == 4 ? kc_cg<4> : kc_cg<8>;
 }
 
-// Blocks of a context's boxes (box, first unit, units, units of the boxes before); none if they do not
-// fit the device at once or it has no cooperative launches.
-int persist_plan(const int* N, int nb, int nsm, bool bicg, std::vector<int4>& work, long* units, int* upc) {
-  work.clear();
-  *units = 0;
+// The one-launch solve of a context's boxes: blocks, counters, sums, BiCGStab coefficients in one allocation.
+struct Persist {
+  int blocks = 0, upc = 0;
+  size_t counter_bytes = 0;
+  PkBlock* work = nullptr;
+  unsigned* counters = nullptr;
+  double* sums = nullptr;
+  double* coef = nullptr;
+  bool bicg = false;
+};
+
+void persist_free(Persist* P) {
+  if (!P) return;
+  cudaFree(P->work);
+  delete P;
+}
+
+// null with *rc = FE_OK: the boxes do not fit the device at once, or it has no cooperative launches.
+Persist* persist_create(const int* N, int nb, int nsm, bool bicg, cudaStream_t st, int* rc) {
+  *rc = FE_OK;
   int dev = 0, coop = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
-    return 0;
+    return nullptr;
   std::vector<long> u(nb);
-  for (int b = 0; b < nb; ++b) {
-    u[b] = ((long)N[b] * N[b] * N[b] + kPkThreads - 1) / kPkThreads;
-    *units += u[b];
-  }
+  for (int b = 0; b < nb; ++b) u[b] = ((long)N[b] * N[b] * N[b] + kPkThreads - 1) / kPkThreads;
   const int most = bicg ? kPkBicgUnits : kPkMaxUnits;
-  for (*upc = 1; *upc <= most; *upc *= 2) {
+  int upc = 1;
+  for (; upc <= most; upc *= 2) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pk_kernel(bicg, *upc), kPkThreads, 0) != cudaSuccess)
-      return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pk_kernel(bicg, upc), kPkThreads, 0) != cudaSuccess)
+      return nullptr;
     const long cap = (long)std::min(per_sm, kPkPerSm) * nsm;
-    long blocks = 0;
-    for (int b = 0; b < nb; ++b) blocks += (u[b] + *upc - 1) / *upc;
-    if (blocks <= cap) break;
+    long blocks = 0, largest = 0;
+    for (int b = 0; b < nb; ++b) {
+      const long q = (u[b] + upc - 1) / upc;
+      blocks += q;
+      largest = std::max(largest, q);
+    }
+    if (blocks <= cap && largest <= (long)kPkLeaves * kPkThreads) break;
   }
-  if (*upc > most) return 0;
-  long before = 0;
+  if (upc > most) return nullptr;
+  std::vector<PkBlock> work;
+  long cells = 0;
   for (int b = 0; b < nb; ++b) {
-    for (long q = 0; q < u[b]; q += *upc)
-      work.push_back(make_int4(b, (int)q, (int)std::min<long>(*upc, u[b] - q), (int)before));
-    before += u[b];
+    const int b0 = (int)work.size();
+    for (long q = 0; q < u[b]; q += upc)
+      work.push_back(PkBlock{b, (int)q, (int)std::min<long>(upc, u[b] - q), b0, cells});
+    cells += (long)N[b] * N[b] * N[b];
   }
-  return (int)work.size();
+  Persist* P = new (std::nothrow) Persist();
+  if (!P) {
+    *rc = FE_ERR_OOM;
+    return nullptr;
+  }
+  P->blocks = (int)work.size();
+  P->upc = upc;
+  P->bicg = bicg;
+  P->counter_bytes = ((size_t)nb * kPkLine * sizeof(unsigned) + 255) / 256 * 256;
+  const size_t wb = (work.size() * sizeof(PkBlock) + 255) / 256 * 256;
+  const size_t sb = ((size_t)P->blocks * 4 * sizeof(double) + 255) / 256 * 256;
+  const size_t cb = bicg ? (size_t)cells * kPkCoef * sizeof(double) : 0;
+  if (cudaMalloc(&P->work, wb + P->counter_bytes + sb + cb) != cudaSuccess) {
+    cudaGetLastError();
+    P->work = nullptr;
+    persist_free(P);
+    *rc = FE_ERR_OOM;
+    return nullptr;
+  }
+  char* base = reinterpret_cast<char*>(P->work) + wb;
+  P->counters = reinterpret_cast<unsigned*>(base);
+  P->sums = reinterpret_cast<double*>(base + P->counter_bytes);
+  P->coef = bicg ? reinterpret_cast<double*>(base + P->counter_bytes + sb) : nullptr;
+  if (cudaMemcpyAsync(P->work, work.data(), work.size() * sizeof(PkBlock), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess) {
+    persist_free(P);
+    *rc = FE_ERR_CUDA;
+    return nullptr;
+  }
+  return P;
 }
-size_t persist_packet_bytes(long units) { return (size_t)2 * units * kPkWords * sizeof(unsigned long long); }
 
 // The whole solve of every box from K_B into K_X (FP64 fields; psi, D^{-1} and the scalars in place).
-int launch_persist(const Launch& L, bool bicg) {
-  if (cudaMemsetAsync(L.packets, 0, persist_packet_bytes(L.punits), L.st) != cudaSuccess) return FE_ERR_CUDA;
+int launch_persist(const Launch& L) {
+  Persist* P = L.persist;
+  if (cudaMemsetAsync(P->counters, 0, P->counter_bytes, L.st) != cudaSuccess) return FE_ERR_CUDA;
   const BoxDev* boxes = L.boxes;
-  const int4* work = L.pwork;
-  unsigned long long* packets = L.packets;
-  long stride = L.punits * kPkWords;
-  void* args[] = {&boxes, &work, &packets, &stride};
+  void* args[] = {&boxes, &P->work, &P->sums, &P->counters, &P->coef};
   cudaError_t e = cudaSuccess;
   FE_LAUNCH(L, KID_SOLVE,
-            (e = cudaLaunchCooperativeKernel((const void*)pk_kernel(bicg, L.pupc), dim3(L.npblocks), dim3(kPkThreads),
-                                             args, 0, L.st)));
+            (e = cudaLaunchCooperativeKernel((const void*)pk_kernel(P->bicg, P->upc), dim3(P->blocks),
+                                             dim3(kPkThreads), args, 0, L.st)));
   return e == cudaSuccess ? FE_OK : FE_ERR_CUDA;
 }
 
