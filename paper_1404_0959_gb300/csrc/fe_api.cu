@@ -113,7 +113,7 @@ struct fe_ctx {
   int2* dework = nullptr;
   int2* dbwork = nullptr;   // plane-streaming blocks (box, block of box)
   int nbblocks = 0, bsmem = 0, bcells = 0, npart = 0;
-  int ring_ok = 0;          // all N multiples of the 16-byte chunk of the ring kernels
+  int ring_ok = 0;          // ring kernels: 2 all N multiples of the 16-byte chunk, 1 all N even, 0 unusable
   bool use_bulk = true;     // streamed CG kernel where the boxes allow it
   int unet_tc = 1;          // U-Net stride-1 layers on tcgen05 (1) or warp-level MMA (0)
   int neblocks = 0;
@@ -332,9 +332,9 @@ static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
     B.etile0 = (int)ework.size();
     for (int q = 0; q < B.entiles; ++q) ework.push_back(make_int2(b, q));
   }
-  c->ring_ok = 1;
+  c->ring_ok = 2;
   for (int b = 0; b < c->nb; ++b)
-    if (c->hbox[b].N % (c->fp64 ? 2 : 4)) c->ring_ok = 0;
+    c->ring_ok = std::min(c->ring_ok, c->hbox[b].N % 2 ? 0 : c->hbox[b].N % (c->fp64 ? 2 : 4) ? 1 : 2);
   // plane-streaming blocks (FP32 fields; FP64 contexts are bound by the FP64
   // pipe and keep the z-marching kernel): every box with N in {64, 128, 256,
   // 512}, a persistent grid of the resident blocks per SM x SMs shared out by cells

@@ -596,7 +596,7 @@ struct Launch {
   int fourier;    // closure of the context (selects kernel variants)
   int transonic;  // transonic pressure operator
   int nd;         // dust classes
-  int ring_ok;        // every box's N is a multiple of the 16-byte chunk (ring kernels usable)
+  int ring_ok;        // ring kernels: 2 every box's N a multiple of the 16-byte chunk, 1 even, 0 unusable
   const int2* bwork;  // plane-streaming blocks (box, block of box); null: z-marching kernels
   int nbblocks;
   int bsmem;          // dynamic shared memory of the streamed CG kernel

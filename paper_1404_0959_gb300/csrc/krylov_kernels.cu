@@ -1954,7 +1954,7 @@ template <typename T> void launch_refine_start(const Launch& L, int* outer_activ
   launch_cg_start<T>(L);
 }
 template <typename T> void launch_refine(const Launch& L, int* outer_active) {
-  if (L.ring_ok)  // every box's N a multiple of the 16-byte chunk, so even: column pairs
+  if (L.ring_ok)  // every box's N even: column pairs
     FE_LAUNCH(L, KID_REFINE,
               (kp_refine<T><<<L.nkblocks, dim3(RTX, TY), 0, L.st>>>(L.kboxes, L.kwork, L.part, outer_active, L.active,
                                                                      L.poly)));

@@ -88,7 +88,7 @@ struct Unparen<void(P)> {
 #define RING_PROLOGUE(P)                                   \
   const TileXYZ t = tile_xyz(boxes, work);                 \
   const BoxDev& B = boxes[t.box];                          \
-  const RGeom<T> G(t.x0, t.y0, B.N);                       \
+  const RGeom<T, WIDE> G(t.x0, t.y0, B.N);                       \
   const int tid = threadIdx.x + RTX * threadIdx.y;         \
   extern __shared__ __align__(16) unsigned char rsm[];     \
   typename Unparen<void(P)>::type R;                       \
@@ -98,14 +98,14 @@ struct Unparen<void(P)> {
 // p^k = p^{k-1} + x staged as the sum of two rings; fluxes phi^k = phi* - dt G2 x,
 // u^k = HbyA - dt/rho^{k-1} Gc p^k, rho^k = rho^n - dt/2 (div phi^n + D phi^k);
 // FP64 path: ||b - M x||^2 for the reported residual.
-template <typename T, bool MIXED>
-using CorrPlan = RingPlan<T, kA, 2, 3, MIXED ? 6 : 8>;  // p^{k-1}, x | phi* | rho^n, rho^{k-1}, HbyA0..2, D phi^n [, psi, b]
+template <typename T, bool MIXED, bool WIDE = true>
+using CorrPlan = RingPlan<T, kA, 2, 3, MIXED ? 6 : 8, WIDE>;  // p^{k-1}, x | phi* | rho^n, rho^{k-1}, HbyA0..2, D phi^n [, psi, b]
 
-template <typename T, bool MIXED>
+template <typename T, bool MIXED, bool WIDE>
 __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_corr(const BoxDev* boxes, const int2* work, double* part, int s, int rhop,
                                                 int pp, int pnew, int kset, int kidx, int xslot) {
   constexpr int NC = MIXED ? 6 : 8;
-  RING_PROLOGUE((CorrPlan<T, MIXED>));
+  RING_PROLOGUE((CorrPlan<T, MIXED, WIDE>));
   R.gs[0] = Fr<T>(B, pp);
   R.gs[1] = Fr<T>(B, xslot);  // the pressure correction (FP32 solution, or the high parts of its pairs)
 #pragma unroll
@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_corr(const BoxDev* boxes
 // u_m per axis and one of div along m: the convection from the unscaled 16 I4 at both faces, the compact
 // Laplacian as (28 S1 - 162 u - S2) / 24 (S1, S2: the six neighbours at distance 1 and 2), Gc unscaled;
 // cl = mu / (24 h^2), cd = mu / (48 h), cc = 1 / (16 h).
-template <typename T, typename Plan>
-__device__ __forceinline__ void ring_L(const Plan& R, int k, const RGeom<T>& G, const T (&php)[3][2],
+template <typename T, bool WIDE, typename Plan>
+__device__ __forceinline__ void ring_L(const Plan& R, int k, const RGeom<T, WIDE>& G, const T (&php)[3][2],
                                        const T (&phm)[3][2], T cl, T cd, T cc, T (&L)[3][2], T (&visc)[3][2]) {
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
@@ -223,12 +223,12 @@ __device__ __forceinline__ void ring_L(const Plan& R, int k, const RGeom<T>& G, 
 
 // two-way: Ysum as a second centre field with one plane of lookahead, so that three blocks per
 // multiprocessor still fit in FP32
-template <typename T, bool TW = false>
-using PredPlan = RingPlan<T, TW ? kA1 : kA, 5, 3, TW ? 2 : 1>;  // u0..2, div, p | phi | rho [, Ysum]
+template <typename T, bool TW = false, bool WIDE = true>
+using PredPlan = RingPlan<T, TW ? kA1 : kA, 5, 3, TW ? 2 : 1, WIDE>;  // u0..2, div, p | phi | rho [, Ysum]
 // TW: two-way coupling (a with the inertia rho (1 + Ysum), R^n with the reaction -(rho Ysum) a)
-template <typename T, bool TW>
+template <typename T, bool TW, bool WIDE>
 __global__ void __launch_bounds__(RNT, sizeof(T) == 4 ? FE_RING_MINB_PRED : FE_RING_MINB) kr_pred(const BoxDev* boxes, const int2* work, int s, int kset, int ysl) {
-  RING_PROLOGUE((PredPlan<T, TW>));
+  RING_PROLOGUE((PredPlan<T, TW, WIDE>));
 #pragma unroll
   for (int m = 0; m < 3; ++m) R.gs[m] = Fr<T>(B, S(s, F_U0 + m));
   R.gs[3] = Fr<T>(B, W_DIV);
@@ -314,15 +314,15 @@ __global__ void __launch_bounds__(RNT, sizeof(T) == 4 ? FE_RING_MINB_PRED : FE_R
 }
 
 // ---- corrector assembly ------------------------------------------------------------------------------
-template <typename T, bool TW = false>
-using AsmPlan = RingPlan<T, kA1, 4, 3, TW ? 12 : 8>;  // u0..2 (level k-1), div | phi | rho, un0..2, rho', Rn0..2
+template <typename T, bool TW = false, bool WIDE = true>
+using AsmPlan = RingPlan<T, kA1, 4, 3, TW ? 12 : 8, WIDE>;  // u0..2 (level k-1), div | phi | rho, un0..2, rho', Rn0..2
                                                        // [, Ysum, a0..2]
 // TW: two-way coupling, L^{k-1} - (rho^{k-1} Ysum) a with a the latest Du/Dt (read per cell pair)
-template <typename T, bool TW>
+template <typename T, bool TW, bool WIDE>
 __global__ void __launch_bounds__(RNT, sizeof(T) == 4 && TW ? 3 : FE_RING_MINB) kr_asm(const BoxDev* boxes, const int2* work,
                                                                                    int s, int up0, int php0, int rhop,
                                                                                    int ysl) {
-  RING_PROLOGUE((AsmPlan<T, TW>));
+  RING_PROLOGUE((AsmPlan<T, TW, WIDE>));
 #pragma unroll
   for (int m = 0; m < 3; ++m) R.gs[m] = Fr<T>(B, up0 + m);
   R.gs[3] = Fr<T>(B, W_DIV);
@@ -376,13 +376,13 @@ __global__ void __launch_bounds__(RNT, sizeof(T) == 4 && TW ? 3 : FE_RING_MINB) 
 }
 
 // ---- Du/Dt at level k -----------------------------------------------------------------------------------
-template <typename T, bool TW = false>
-using AccelPlan = RingPlan<T, kA, 5, 0, TW ? 2 : 1>;  // u0..2, div, p | | rho [, Ysum]
+template <typename T, bool TW = false, bool WIDE = true>
+using AccelPlan = RingPlan<T, kA, 5, 0, TW ? 2 : 1, WIDE>;  // u0..2, div, p | | rho [, Ysum]
 // TW: two-way coupling, inertia rho (1 + Ysum) with Ysum from slot ysl (a centre field of the ring)
-template <typename T, bool TW>
+template <typename T, bool TW, bool WIDE>
 __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_accel(const BoxDev* boxes, const int2* work, int kset, int pk,
                                                               int ysl) {
-  RING_PROLOGUE((AccelPlan<T, TW>));
+  RING_PROLOGUE((AccelPlan<T, TW, WIDE>));
 #pragma unroll
   for (int m = 0; m < 3; ++m) R.gs[m] = Fr<T>(B, S(kset, F_U0 + m));
   R.gs[3] = Fr<T>(B, W_DIV);
@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_accel(const BoxDev* boxe
 // h D(phi_p I4 Y_j) for both cells of the pair and every class: phi_p = phi - tau_j I4(rho) I4(a_d) at each
 // face (rho, a0..2, Y_j: stencil fields 0, 1..3, 4 + j of the plan; phi: face arrays 0..2).  Lines of rho
 // and a_d along d, and of Y_j along d, each read once; 16 I4 evaluated unscaled, the factors folded.
-template <typename T, int ND, typename Plan>
-__device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, const RGeom<T>& G, const T (&taup)[ND],
+template <typename T, int ND, bool WIDE, typename Plan>
+__device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, const RGeom<T, WIDE>& G, const T (&taup)[ND],
                                                    T (&fl)[ND][2]) {
   T php[3][2], phm[3][2];
   R.faces2(0, k, G, php, phm);
@@ -474,11 +474,11 @@ __device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, const R
   for (int j = 0; j < ND; ++j) fl[j][0] *= T(0.0625), fl[j][1] *= T(0.0625);
 }
 
-template <typename T, int ND>
-using FluxPlan = RingPlan<T, kA, 4 + ND, 3, 0>;  // rho, a0..2, Y_j | phi (two planes ahead: measured)
-template <typename T, int ND>
+template <typename T, int ND, bool WIDE = true>
+using FluxPlan = RingPlan<T, kA, 4 + ND, 3, 0, WIDE>;  // rho, a0..2, Y_j | phi (two planes ahead: measured)
+template <typename T, int ND, bool WIDE>
 __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fluxn(const BoxDev* boxes, const int2* work, int s) {
-  RING_PROLOGUE((FluxPlan<T, ND>));
+  RING_PROLOGUE((FluxPlan<T, ND, WIDE>));
   (void)tid;  // no centre fields
   R.gs[0] = Fr<T>(B, S(s, F_RHO));
 #pragma unroll
@@ -513,13 +513,13 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fluxn(const BoxDev* boxe
 // FR: Fourier closure -- also E^k = (rho^n E^n - dt/2 (D F_E^n + D F_E^k)) / rho^k (E^n, D F_E^n and
 // D F_E^k as centre fields, k_fe_cell / k_fe_div), and on the last corrector T = (E - |u|^2/2) / c_v,
 // p = rho R T and the total energy sum rho E (the general k_dust<T, true>'s expressions)
-template <typename T, int ND, bool FR = false>
-using DustPlan = RingPlan<T, kA1, 4 + ND, 3, 4 + 2 * ND + (FR ? 3 : 0)>;  // rho^k, a0..2, Y_j^{k-1} | phi^k |
+template <typename T, int ND, bool FR = false, bool WIDE = true>
+using DustPlan = RingPlan<T, kA1, 4 + ND, 3, 4 + 2 * ND + (FR ? 3 : 0), WIDE>;  // rho^k, a0..2, Y_j^{k-1} | phi^k |
                                                                          // rho^n, Y^n, FYN, [E^n, DFE^n, DFE^k,] u0..2
-template <typename T, int ND, bool FR>
+template <typename T, int ND, bool FR, bool WIDE>
 __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_dust(const BoxDev* boxes, const int2* work, double* part, int s, int kset,
                                                 int yp0, int yn0, int last, int enew) {
-  RING_PROLOGUE((DustPlan<T, ND, FR>));
+  RING_PROLOGUE((DustPlan<T, ND, FR, WIDE>));
   constexpr int EB = 1 + 2 * ND, UB = EB + (FR ? 3 : 0);  // centre indices of E^n (FR) and of u^k
   R.gs[0] = Fr<T>(B, S(kset, F_RHO));
 #pragma unroll
@@ -640,12 +640,12 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_dust(const BoxDev* boxes
 // (the fields the energy face fluxes k_fe_face read; k_fe_cell's expressions).  es >= 0: E from slot es
 // (tmode 1); es < 0: the level-n energy E^n = c_v T^n + |u^n|^2 / 2 from T^n and u^n, also stored in W_EN.
 // tmode 0: T = T^n, 1: T = p / (rho R).  The gradients from line loads of u_l along m, both cells.
-template <typename T>
-using FeCellPlan = RingPlan<T, kA, 3, 0, 6>;  // u0..2 | | rho, p, E or T^n, u^n_0..2
-template <typename T>
+template <typename T, bool WIDE = true>
+using FeCellPlan = RingPlan<T, kA, 3, 0, 6, WIDE>;  // u0..2 | | rho, p, E or T^n, u^n_0..2
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fe_cell(const BoxDev* boxes, const int2* work, int s, int u0,
                                                                 int rhos, int ps, int es, int tmode) {
-  RING_PROLOGUE(FeCellPlan<T>);
+  RING_PROLOGUE((FeCellPlan<T, WIDE>));
 #pragma unroll
   for (int m = 0; m < 3; ++m) R.gs[m] = Fr<T>(B, u0 + m);
   R.gc[0] = Fr<T>(B, rhos);
@@ -696,11 +696,11 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fe_cell(const BoxDev* bo
 // The three +1/2 face fluxes F_E = phi I4(H) - sum_m tau_dm I4(u_m) - kappa G4(T) of every cell
 // (k_fe_face's expressions): lines of H, T, u0..2 and div along each axis from the ring, the gradient
 // fields h Gc_m u_d (needed only along d, at offsets -1..2) by pair loads through the read-only path.
-template <typename T>
-using FeFacePlan = RingPlan<T, kA1, 6, 0, 3>;  // H, T, u0..2, div | | phi0..2
-template <typename T>
+template <typename T, bool WIDE = true>
+using FeFacePlan = RingPlan<T, kA1, 6, 0, 3, WIDE>;  // H, T, u0..2, div | | phi0..2
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fe_face(const BoxDev* boxes, const int2* work, int u0, int phi0) {
-  RING_PROLOGUE(FeFacePlan<T>);
+  RING_PROLOGUE((FeFacePlan<T, WIDE>));
   R.gs[0] = Fr<T>(B, W_FEH);
   R.gs[1] = Fr<T>(B, W_FET);
 #pragma unroll
@@ -774,14 +774,14 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fe_face(const BoxDev* bo
 }
 
 // ---- velocity divergence div = sum_m Gc_m(u_m) --------------------------------------------------------
-template <typename T>
-using DivPlan = RingPlan<T, kAdiv, 3, 0, 0>;  // u0..2
+template <typename T, bool WIDE = true>
+using DivPlan = RingPlan<T, kAdiv, 3, 0, 0, WIDE>;  // u0..2
 // with_dt: also max_i sum_d |u_d| over the box and the adaptive time step
 // from it (the first divergence of a step reads u^n, the field k_dt reads).
-template <typename T>
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_div(const BoxDev* boxes, const int2* work, int u0,
                                                             double* part, int with_dt) {
-  RING_PROLOGUE(DivPlan<T>);
+  RING_PROLOGUE((DivPlan<T, WIDE>));
   (void)tid;  // no centre fields
 #pragma unroll
   for (int m = 0; m < 3; ++m) R.gs[m] = Fr<T>(B, u0 + m);
@@ -815,12 +815,12 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_div(const BoxDev* boxes,
 // copy (K_AUX) and to the first inner right-hand side (K_R), and the kernel
 // starts the refined solve: ||b||^2 and <b, D^{-1} b> into the refinement and
 // CG scalars (the solution pairs start as zero by the outer-step count).
-template <typename T>
-using RhsPlan = RingPlan<T, kArhs, 5, 0, 3>;  // rho', HbyA0..2, p | | rho^n, D phi^n [, D^{-1}]
-template <typename T>
+template <typename T, bool WIDE = true>
+using RhsPlan = RingPlan<T, kArhs, 5, 0, 3, WIDE>;  // rho', HbyA0..2, p | | rho^n, D phi^n [, D^{-1}]
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_rhs(const BoxDev* boxes, const int2* work, int s, int rhop,
                                                             int pp, double* part, int* rstart, int* active, int poly) {
-  RING_PROLOGUE(RhsPlan<T>);
+  RING_PROLOGUE((RhsPlan<T, WIDE>));
   R.gs[0] = Fr<T>(B, rhop);
 #pragma unroll
   for (int d = 0; d < 3; ++d) R.gs[1 + d] = Fr<T>(B, W_HB0 + d);
@@ -888,16 +888,21 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_rhs(const BoxDev* boxes,
 }
 
 // ---- launchers (0: the ring kernel could not be prepared) --------------------------------------
+// boxes with even N but not all multiples of the 16-byte chunk: the kernels with 8-byte chunks
+template <typename T>
+static bool narrow(const Launch& L) {
+  return sizeof(T) == 4 && L.ring_ok == 1;
+}
 #define RGRID(bytes) L.nblocks, dim3(RTX, TY), (bytes), L.st
 template <typename T>
 int rlaunch_corr(const Launch& L, int s, int rhop, int pp, int pnew, int kset, int kidx, int mixed) {
   if (!L.ring_ok || !ring_ready<T>(mixed ? RK_CORR_M : RK_CORR_F)) return 0;
   constexpr int bm = CorrPlan<T, true>::bytes, bf = CorrPlan<T, false>::bytes;
   if (mixed)
-    FE_LAUNCH(L, KID_CORR, (kr_corr<T, true><<<RGRID(bm)>>>(L.boxes, L.work, L.part, s, rhop, pp, pnew, kset, kidx,
+    FE_LAUNCH(L, KID_CORR, ((narrow<T>(L) ? kr_corr<T, true, sizeof(T) != 4> : kr_corr<T, true, true>)<<<RGRID(bm)>>>(L.boxes, L.work, L.part, s, rhop, pp, pnew, kset, kidx,
                                                              mixed == 2 ? K_XH : K_X)));
   else
-    FE_LAUNCH(L, KID_CORR, (kr_corr<T, false><<<RGRID(bf)>>>(L.boxes, L.work, L.part, s, rhop, pp, pnew, kset, kidx,
+    FE_LAUNCH(L, KID_CORR, ((narrow<T>(L) ? kr_corr<T, false, sizeof(T) != 4> : kr_corr<T, false, true>)<<<RGRID(bf)>>>(L.boxes, L.work, L.part, s, rhop, pp, pnew, kset, kidx,
                                                               K_X)));
   return 1;
 }
@@ -907,9 +912,9 @@ int rlaunch_pred(const Launch& L, int s, int kset) {
   const bool tw = L.ysum >= 0;
   if (!L.ring_ok || !ring_ready<T>(tw ? RK_PRED_TW : RK_PRED)) return 0;
   if (tw)
-    FE_LAUNCH(L, KID_PRED, (kr_pred<T, true><<<RGRID((PredPlan<T, true>::bytes))>>>(L.boxes, L.work, s, kset, L.ysum)));
+    FE_LAUNCH(L, KID_PRED, ((narrow<T>(L) ? kr_pred<T, true, sizeof(T) != 4> : kr_pred<T, true, true>)<<<RGRID((PredPlan<T, true>::bytes))>>>(L.boxes, L.work, s, kset, L.ysum)));
   else
-    FE_LAUNCH(L, KID_PRED, (kr_pred<T, false><<<RGRID(PredPlan<T>::bytes)>>>(L.boxes, L.work, s, kset, -1)));
+    FE_LAUNCH(L, KID_PRED, ((narrow<T>(L) ? kr_pred<T, false, sizeof(T) != 4> : kr_pred<T, false, true>)<<<RGRID(PredPlan<T>::bytes)>>>(L.boxes, L.work, s, kset, -1)));
   return 1;
 }
 template <typename T>
@@ -918,9 +923,9 @@ int rlaunch_asm(const Launch& L, int s, int up0, int php0, int rhop) {
   if (!L.ring_ok || !ring_ready<T>(tw ? RK_ASM_TW : RK_ASM)) return 0;
   if (tw)
     FE_LAUNCH(L, KID_ASM,
-              (kr_asm<T, true><<<RGRID((AsmPlan<T, true>::bytes))>>>(L.boxes, L.work, s, up0, php0, rhop, L.ysum)));
+              ((narrow<T>(L) ? kr_asm<T, true, sizeof(T) != 4> : kr_asm<T, true, true>)<<<RGRID((AsmPlan<T, true>::bytes))>>>(L.boxes, L.work, s, up0, php0, rhop, L.ysum)));
   else
-    FE_LAUNCH(L, KID_ASM, (kr_asm<T, false><<<RGRID(AsmPlan<T>::bytes)>>>(L.boxes, L.work, s, up0, php0, rhop, -1)));
+    FE_LAUNCH(L, KID_ASM, ((narrow<T>(L) ? kr_asm<T, false, sizeof(T) != 4> : kr_asm<T, false, true>)<<<RGRID(AsmPlan<T>::bytes)>>>(L.boxes, L.work, s, up0, php0, rhop, -1)));
   return 1;
 }
 template <typename T>
@@ -928,18 +933,18 @@ int rlaunch_accel(const Launch& L, int kset, int pk) {
   const bool tw = L.ysum >= 0;
   if (!L.ring_ok || !ring_ready<T>(tw ? RK_ACCEL_TW : RK_ACCEL)) return 0;
   if (tw)
-    FE_LAUNCH(L, KID_ACCEL, (kr_accel<T, true><<<RGRID((AccelPlan<T, true>::bytes))>>>(L.boxes, L.work, kset, pk, L.ysum)));
+    FE_LAUNCH(L, KID_ACCEL, ((narrow<T>(L) ? kr_accel<T, true, sizeof(T) != 4> : kr_accel<T, true, true>)<<<RGRID((AccelPlan<T, true>::bytes))>>>(L.boxes, L.work, kset, pk, L.ysum)));
   else
-    FE_LAUNCH(L, KID_ACCEL, (kr_accel<T, false><<<RGRID(AccelPlan<T>::bytes)>>>(L.boxes, L.work, kset, pk, -1)));
+    FE_LAUNCH(L, KID_ACCEL, ((narrow<T>(L) ? kr_accel<T, false, sizeof(T) != 4> : kr_accel<T, false, true>)<<<RGRID(AccelPlan<T>::bytes)>>>(L.boxes, L.work, kset, pk, -1)));
   return 1;
 }
 template <typename T>
 int rlaunch_fluxn(const Launch& L, int s, int nd) {
   if (nd < 1 || nd > 3 || !L.ring_ok || !ring_ready<T>(RK_FLUX1 + nd - 1)) return 0;
   switch (nd) {
-    case 1: FE_LAUNCH(L, KID_FLUXN, (kr_fluxn<T, 1><<<RGRID((FluxPlan<T, 1>::bytes))>>>(L.boxes, L.work, s))); break;
-    case 2: FE_LAUNCH(L, KID_FLUXN, (kr_fluxn<T, 2><<<RGRID((FluxPlan<T, 2>::bytes))>>>(L.boxes, L.work, s))); break;
-    case 3: FE_LAUNCH(L, KID_FLUXN, (kr_fluxn<T, 3><<<RGRID((FluxPlan<T, 3>::bytes))>>>(L.boxes, L.work, s))); break;
+    case 1: FE_LAUNCH(L, KID_FLUXN, ((narrow<T>(L) ? kr_fluxn<T, 1, sizeof(T) != 4> : kr_fluxn<T, 1, true>)<<<RGRID((FluxPlan<T, 1>::bytes))>>>(L.boxes, L.work, s))); break;
+    case 2: FE_LAUNCH(L, KID_FLUXN, ((narrow<T>(L) ? kr_fluxn<T, 2, sizeof(T) != 4> : kr_fluxn<T, 2, true>)<<<RGRID((FluxPlan<T, 2>::bytes))>>>(L.boxes, L.work, s))); break;
+    case 3: FE_LAUNCH(L, KID_FLUXN, ((narrow<T>(L) ? kr_fluxn<T, 3, sizeof(T) != 4> : kr_fluxn<T, 3, true>)<<<RGRID((FluxPlan<T, 3>::bytes))>>>(L.boxes, L.work, s))); break;
     default: return 0;
   }
   return 1;
@@ -949,15 +954,15 @@ static int rlaunch_dust_any(const Launch& L, int s, int kset, int yp0, int yn0, 
   if (nd < 1 || nd > 3 || !L.ring_ok || !ring_ready<T>((FR ? RK_DUST1F : RK_DUST1) + nd - 1)) return 0;
   switch (nd) {
     case 1:
-      FE_LAUNCH(L, KID_DUST, (kr_dust<T, 1, FR><<<RGRID((DustPlan<T, 1, FR>::bytes))>>>(L.boxes, L.work, L.part, s, kset,
+      FE_LAUNCH(L, KID_DUST, ((narrow<T>(L) ? kr_dust<T, 1, FR, sizeof(T) != 4> : kr_dust<T, 1, FR, true>)<<<RGRID((DustPlan<T, 1, FR>::bytes))>>>(L.boxes, L.work, L.part, s, kset,
                                                                                          yp0, yn0, last, enew)));
       break;
     case 2:
-      FE_LAUNCH(L, KID_DUST, (kr_dust<T, 2, FR><<<RGRID((DustPlan<T, 2, FR>::bytes))>>>(L.boxes, L.work, L.part, s, kset,
+      FE_LAUNCH(L, KID_DUST, ((narrow<T>(L) ? kr_dust<T, 2, FR, sizeof(T) != 4> : kr_dust<T, 2, FR, true>)<<<RGRID((DustPlan<T, 2, FR>::bytes))>>>(L.boxes, L.work, L.part, s, kset,
                                                                                          yp0, yn0, last, enew)));
       break;
     case 3:
-      FE_LAUNCH(L, KID_DUST, (kr_dust<T, 3, FR><<<RGRID((DustPlan<T, 3, FR>::bytes))>>>(L.boxes, L.work, L.part, s, kset,
+      FE_LAUNCH(L, KID_DUST, ((narrow<T>(L) ? kr_dust<T, 3, FR, sizeof(T) != 4> : kr_dust<T, 3, FR, true>)<<<RGRID((DustPlan<T, 3, FR>::bytes))>>>(L.boxes, L.work, L.part, s, kset,
                                                                                          yp0, yn0, last, enew)));
       break;
     default: return 0;
@@ -976,27 +981,27 @@ int rlaunch_dust_fourier(const Launch& L, int s, int kset, int yp0, int yn0, int
 template <typename T>
 int rlaunch_div(const Launch& L, int u0, int with_dt) {
   if (!L.ring_ok || !ring_ready<T>(RK_DIV)) return 0;
-  FE_LAUNCH(L, KID_DIV, (kr_div<T><<<RGRID(DivPlan<T>::bytes)>>>(L.boxes, L.work, u0, L.part, with_dt)));
+  FE_LAUNCH(L, KID_DIV, ((narrow<T>(L) ? kr_div<T, sizeof(T) != 4> : kr_div<T, true>)<<<RGRID(DivPlan<T>::bytes)>>>(L.boxes, L.work, u0, L.part, with_dt)));
   return 1;
 }
 template <typename T>
 int rlaunch_fe_cell(const Launch& L, int s, int u0, int rhos, int ps, int es, int tmode) {
   if (!L.ring_ok || !ring_ready<T>(RK_FECELL)) return 0;
-  FE_LAUNCH(L, KID_FE_CELL, (kr_fe_cell<T><<<RGRID(FeCellPlan<T>::bytes)>>>(L.boxes, L.work, s, u0, rhos, ps, es,
+  FE_LAUNCH(L, KID_FE_CELL, ((narrow<T>(L) ? kr_fe_cell<T, sizeof(T) != 4> : kr_fe_cell<T, true>)<<<RGRID(FeCellPlan<T>::bytes)>>>(L.boxes, L.work, s, u0, rhos, ps, es,
                                                                              tmode)));
   return 1;
 }
 template <typename T>
 int rlaunch_fe_face(const Launch& L, int u0, int phi0) {
   if (!L.ring_ok || !ring_ready<T>(RK_FEFACE)) return 0;
-  FE_LAUNCH(L, KID_FE_FACE, (kr_fe_face<T><<<RGRID(FeFacePlan<T>::bytes)>>>(L.boxes, L.work, u0, phi0)));
+  FE_LAUNCH(L, KID_FE_FACE, ((narrow<T>(L) ? kr_fe_face<T, sizeof(T) != 4> : kr_fe_face<T, true>)<<<RGRID(FeFacePlan<T>::bytes)>>>(L.boxes, L.work, u0, phi0)));
   return 1;
 }
 template <typename T>
 int rlaunch_rhs(const Launch& L, int s, int rhop, int pp) {
   if (!L.ring_ok || !ring_ready<T>(RK_RHS)) return 0;
   FE_LAUNCH(L, KID_RHS,
-            (kr_rhs<T><<<RGRID(RhsPlan<T>::bytes)>>>(L.boxes, L.work, s, rhop, pp, L.part, L.rstart, L.active,
+            ((narrow<T>(L) ? kr_rhs<T, sizeof(T) != 4> : kr_rhs<T, true>)<<<RGRID(RhsPlan<T>::bytes)>>>(L.boxes, L.work, s, rhop, pp, L.part, L.rstart, L.active,
                                                      L.poly)));
   return 1;
 }
@@ -1007,27 +1012,28 @@ int rprepare() {
   if (dev < 0) return 0;
   unsigned ok = 0;
   auto set = [&](int bit, bool accepted) { ok |= accepted ? 1u << bit : 0u; };
-  set(RK_CORR_M, set_smem(kr_corr<T, true>, CorrPlan<T, true>::bytes));
-  set(RK_CORR_F, set_smem(kr_corr<T, false>, CorrPlan<T, false>::bytes));
-  set(RK_PRED, set_smem(kr_pred<T, false>, PredPlan<T>::bytes));
-  set(RK_ASM, set_smem(kr_asm<T, false>, AsmPlan<T>::bytes));
-  set(RK_ACCEL, set_smem(kr_accel<T, false>, AccelPlan<T>::bytes));
-  set(RK_PRED_TW, set_smem(kr_pred<T, true>, PredPlan<T, true>::bytes));
-  set(RK_ASM_TW, set_smem(kr_asm<T, true>, AsmPlan<T, true>::bytes));
-  set(RK_ACCEL_TW, set_smem(kr_accel<T, true>, AccelPlan<T, true>::bytes));
-  set(RK_FLUX1, set_smem(kr_fluxn<T, 1>, FluxPlan<T, 1>::bytes));
-  set(RK_FLUX2, set_smem(kr_fluxn<T, 2>, FluxPlan<T, 2>::bytes));
-  set(RK_FLUX3, set_smem(kr_fluxn<T, 3>, FluxPlan<T, 3>::bytes));
-  set(RK_DUST1, set_smem(kr_dust<T, 1, false>, DustPlan<T, 1>::bytes));
-  set(RK_DUST2, set_smem(kr_dust<T, 2, false>, DustPlan<T, 2>::bytes));
-  set(RK_DUST3, set_smem(kr_dust<T, 3, false>, DustPlan<T, 3>::bytes));
-  set(RK_DUST1F, set_smem(kr_dust<T, 1, true>, DustPlan<T, 1, true>::bytes));
-  set(RK_DUST2F, set_smem(kr_dust<T, 2, true>, DustPlan<T, 2, true>::bytes));
-  set(RK_DUST3F, set_smem(kr_dust<T, 3, true>, DustPlan<T, 3, true>::bytes));
-  set(RK_DIV, set_smem(kr_div<T>, DivPlan<T>::bytes));
-  set(RK_RHS, set_smem(kr_rhs<T>, RhsPlan<T>::bytes));
-  set(RK_FECELL, set_smem(kr_fe_cell<T>, FeCellPlan<T>::bytes));
-  set(RK_FEFACE, set_smem(kr_fe_face<T>, FeFacePlan<T>::bytes));
+  auto both = [](auto wide, auto narrow, int bytes) { return set_smem(wide, bytes) && set_smem(narrow, bytes); };
+  set(RK_CORR_M, both(kr_corr<T, true, true>, kr_corr<T, true, sizeof(T) != 4>, CorrPlan<T, true>::bytes));
+  set(RK_CORR_F, both(kr_corr<T, false, true>, kr_corr<T, false, sizeof(T) != 4>, CorrPlan<T, false>::bytes));
+  set(RK_PRED, both(kr_pred<T, false, true>, kr_pred<T, false, sizeof(T) != 4>, PredPlan<T>::bytes));
+  set(RK_ASM, both(kr_asm<T, false, true>, kr_asm<T, false, sizeof(T) != 4>, AsmPlan<T>::bytes));
+  set(RK_ACCEL, both(kr_accel<T, false, true>, kr_accel<T, false, sizeof(T) != 4>, AccelPlan<T>::bytes));
+  set(RK_PRED_TW, both(kr_pred<T, true, true>, kr_pred<T, true, sizeof(T) != 4>, PredPlan<T, true>::bytes));
+  set(RK_ASM_TW, both(kr_asm<T, true, true>, kr_asm<T, true, sizeof(T) != 4>, AsmPlan<T, true>::bytes));
+  set(RK_ACCEL_TW, both(kr_accel<T, true, true>, kr_accel<T, true, sizeof(T) != 4>, AccelPlan<T, true>::bytes));
+  set(RK_FLUX1, both(kr_fluxn<T, 1, true>, kr_fluxn<T, 1, sizeof(T) != 4>, FluxPlan<T, 1>::bytes));
+  set(RK_FLUX2, both(kr_fluxn<T, 2, true>, kr_fluxn<T, 2, sizeof(T) != 4>, FluxPlan<T, 2>::bytes));
+  set(RK_FLUX3, both(kr_fluxn<T, 3, true>, kr_fluxn<T, 3, sizeof(T) != 4>, FluxPlan<T, 3>::bytes));
+  set(RK_DUST1, both(kr_dust<T, 1, false, true>, kr_dust<T, 1, false, sizeof(T) != 4>, DustPlan<T, 1>::bytes));
+  set(RK_DUST2, both(kr_dust<T, 2, false, true>, kr_dust<T, 2, false, sizeof(T) != 4>, DustPlan<T, 2>::bytes));
+  set(RK_DUST3, both(kr_dust<T, 3, false, true>, kr_dust<T, 3, false, sizeof(T) != 4>, DustPlan<T, 3>::bytes));
+  set(RK_DUST1F, both(kr_dust<T, 1, true, true>, kr_dust<T, 1, true, sizeof(T) != 4>, DustPlan<T, 1, true>::bytes));
+  set(RK_DUST2F, both(kr_dust<T, 2, true, true>, kr_dust<T, 2, true, sizeof(T) != 4>, DustPlan<T, 2, true>::bytes));
+  set(RK_DUST3F, both(kr_dust<T, 3, true, true>, kr_dust<T, 3, true, sizeof(T) != 4>, DustPlan<T, 3, true>::bytes));
+  set(RK_DIV, both(kr_div<T, true>, kr_div<T, sizeof(T) != 4>, DivPlan<T>::bytes));
+  set(RK_RHS, both(kr_rhs<T, true>, kr_rhs<T, sizeof(T) != 4>, RhsPlan<T>::bytes));
+  set(RK_FECELL, both(kr_fe_cell<T, true>, kr_fe_cell<T, sizeof(T) != 4>, FeCellPlan<T>::bytes));
+  set(RK_FEFACE, both(kr_fe_face<T, true>, kr_fe_face<T, sizeof(T) != 4>, FeFacePlan<T>::bytes));
   cudaGetLastError();  // a refused limit is not an error of the context
   ok &= ~(unsigned)(FE_RING_OFF);
   RingReady<T>::ok[dev] = ok;

@@ -12,7 +12,7 @@
 //   sigma = sigma^n - dt/2 [D(F^n) + D(F*)], m likewise;
 //   backward-Euler drag after each stage: V = u^{n+1} + (m/sigma - u^{n+1}) tau/(tau + dt),
 //   Y = sigma / rho^{n+1}.
-// Two forms: the ring kernels (every box's N a multiple of the 16-byte chunk;
+// Two forms: the ring kernels (every box's N even;
 // one class per launch, its planes and the gas planes arriving in shared-memory
 // rings by asynchronous copies, zring.cuh) and the general kernels (one thread
 // walks the z-planes of a column; neighbours through the read-only cache with
@@ -212,21 +212,21 @@ __device__ __forceinline__ void tfr_div(const RP& R, const GT& G, int k, T ih, T
   }
 }
 
-#define TF_RING_PROLOGUE(P)                              \
+#define TF_RING_PROLOGUE(...)                            \
   const TileXYZ t = tile_xyz(boxes, work);               \
   const BoxDev& B = boxes[t.box];                        \
-  const RGeom<T> G(t.x0, t.y0, B.N);                     \
+  const RGeom<T, WIDE> G(t.x0, t.y0, B.N);               \
   const int tid = threadIdx.x + RTX * threadIdx.y;       \
   extern __shared__ __align__(16) unsigned char rsm[];   \
-  P R;                                                   \
+  __VA_ARGS__ R;                                         \
   R.init(rsm, t.k0, t.kend)
 
 // predictor: rho^n, u^n (3), Y^n_j, V^n_j (3) | phi^n | rho^{n+1}, u^{n+1} (3)
-template <typename T>
-using TfPredPlan = RingPlan<T, 1, 8, 3, 4>;
-template <typename T>
+template <typename T, bool WIDE = true>
+using TfPredPlan = RingPlan<T, 1, 8, 3, 4, WIDE>;
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(RNT) kr_tf_pred(const BoxDev* boxes, const int2* work, int s, int ks, int j) {
-  TF_RING_PROLOGUE(TfPredPlan<T>);
+  TF_RING_PROLOGUE(TfPredPlan<T, WIDE>);
   R.gs[0] = TF<T>(B, S(s, F_RHO));
 #pragma unroll
   for (int m = 0; m < 3; ++m) R.gs[1 + m] = TF<T>(B, S(s, F_U0 + m));
@@ -284,12 +284,12 @@ __global__ void __launch_bounds__(RNT) kr_tf_pred(const BoxDev* boxes, const int
 }
 
 // corrector: rho^{n+1}, u^{n+1} (3), Y*_j, V*_j (3) | phi^{n+1} | rho^n, Y^n_j, D(F^n), D(G^n) (3), V^n_j (3)
-template <typename T>
-using TfCorrPlan = RingPlan<T, 1, 8, 3, 9>;
-template <typename T>
+template <typename T, bool WIDE = true>
+using TfCorrPlan = RingPlan<T, 1, 8, 3, 9, WIDE>;
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(RNT) kr_tf_corr(const BoxDev* boxes, const int2* work, double* part, int s, int ks,
                                                   int j) {
-  TF_RING_PROLOGUE(TfCorrPlan<T>);
+  TF_RING_PROLOGUE(TfCorrPlan<T, WIDE>);
   R.gs[0] = TF<T>(B, S(ks, F_RHO));
 #pragma unroll
   for (int m = 0; m < 3; ++m) R.gs[1 + m] = TF<T>(B, S(ks, F_U0 + m));
@@ -370,10 +370,11 @@ template <typename T>
 int tfprepare() {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kTfMaxDev) return 0;
-  const bool a = cudaFuncSetAttribute(kr_tf_pred<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      TfPredPlan<T>::bytes) == cudaSuccess;
-  const bool b = cudaFuncSetAttribute(kr_tf_corr<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      TfCorrPlan<T>::bytes) == cudaSuccess;
+  auto set = [](auto kernel, int bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+  };
+  const bool a = set(kr_tf_pred<T, true>, TfPredPlan<T>::bytes) && set(kr_tf_pred<T, sizeof(T) != 4>, TfPredPlan<T>::bytes);
+  const bool b = set(kr_tf_corr<T, true>, TfCorrPlan<T>::bytes) && set(kr_tf_corr<T, sizeof(T) != 4>, TfCorrPlan<T>::bytes);
   cudaGetLastError();  // a refused limit is not an error of the context
   TfReady<T>::ok[dev] = a && b ? 1 : -1;
   return a && b;
@@ -402,11 +403,12 @@ __global__ void __launch_bounds__(NTHR) k_tf_init(const BoxDev* boxes, const int
 template <typename T>
 void launch_two_fluid(const Launch& L, int s, int ks) {
   if (L.ring_ok && tf_ring_ready<T>()) {  // one class per launch; predictor of every class first
+    const bool nw = sizeof(T) == 4 && L.ring_ok == 1;  // 8-byte chunks
     for (int j = 0; j < L.nd; ++j)
       FE_LAUNCH(L, KID_TF_PRED,
-                (kr_tf_pred<T><<<L.nblocks, dim3(RTX, TY), TfPredPlan<T>::bytes, L.st>>>(L.boxes, L.work, s, ks, j)));
+                ((nw ? kr_tf_pred<T, sizeof(T) != 4> : kr_tf_pred<T, true>)<<<L.nblocks, dim3(RTX, TY), TfPredPlan<T>::bytes, L.st>>>(L.boxes, L.work, s, ks, j)));
     for (int j = 0; j < L.nd; ++j)
-      FE_LAUNCH(L, KID_TF_CORR, (kr_tf_corr<T><<<L.nblocks, dim3(RTX, TY), TfCorrPlan<T>::bytes, L.st>>>(
+      FE_LAUNCH(L, KID_TF_CORR, ((nw ? kr_tf_corr<T, sizeof(T) != 4> : kr_tf_corr<T, true>)<<<L.nblocks, dim3(RTX, TY), TfCorrPlan<T>::bytes, L.st>>>(
                                     L.boxes, L.work, L.part, s, ks, j)));
     return;
   }

@@ -37,6 +37,9 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
@@ -78,48 +81,51 @@ __device__ __forceinline__ void stp(T* p, T a, T b) {
   *reinterpret_cast<P2<T>*>(p) = v;
 }
 
+// chunks of ce cells of a tile-with-halo plane (x-halo xh) and of a centre plane
+__host__ __device__ constexpr int ring_nch(int ce, int xh) { return TY * ((TX + 2 * xh) / ce) + 4 * (TX / ce); }
+__host__ __device__ constexpr int ring_ncc(int ce) { return TX * TY / ce; }
+
 // Tile geometry of the ring kernels: 32 x 8 columns, y-halo 2, x-halo XH (2
 // cells rounded up to one 16-byte chunk), copied in 16-byte chunks: at most
 // two chunks per thread and field for the tile with its star halo (corners
-// are not needed), at most one per thread for a centre-only plane.  Needs
-// N % CE == 0 so no chunk straddles the periodic seam (and N even, so a
-// column pair is inside the box or outside it as a whole); wrapped columns
-// beyond a ragged box edge hold the periodic continuation as in ZGeom.
-template <typename T>
+// are not needed), at most one per thread for a centre-only plane.  Chunks
+// must not straddle the periodic seam, so 16-byte chunks need N % CE == 0;
+// FP32 boxes with other even N run the kernels with WIDE = false: 8-byte
+// chunks (column pairs) into the same slots, x-halo 2.  Twice the copies,
+// still ahead of the z-marching kernels they ran on before (step of 250^3
+// cells 10.8 -> 9.2 ms, of 150^3 3.24 -> 2.90 ms).  A kernel that chose the
+// chunk at run time was 1 % slower on the wide grids.  N must be even (a column pair is inside the box or
+// outside it as a whole); wrapped columns beyond a ragged box edge hold the
+// periodic continuation as in ZGeom.
+template <typename T, bool WIDE = true>
 struct RGeom {
-  static constexpr int CE = 16 / (int)sizeof(T);  // cells per chunk
+  static constexpr int CE = 16 / (int)sizeof(T);  // cells per 16-byte chunk
   static constexpr int XH = CE > 2 ? CE : 2;      // x-halo
   static constexpr int W = TX + 2 * XH, H = TY + 4, HW = H * W;
-  static constexpr int ROWC = W / CE, MIDC = TX / CE;
-  static constexpr int NCH = TY * ROWC + 4 * MIDC;  // chunks of a tile-with-halo plane
-  static constexpr int NCC = TX * TY / CE;          // chunks of a centre plane
-  static_assert(NCH <= 2 * RNT && NCC <= RNT, "two halo chunks and one centre chunk per thread");
+  static_assert(ring_nch(CE, XH) <= 2 * RNT && ring_ncc(CE) <= RNT && ring_nch(2, 2) <= 2 * RNT && ring_ncc(2) <= RNT,
+                "two halo chunks and one centre chunk per thread");
   int N, NN, col, csm;
   bool active;
   int ch_g[2], ch_s[2];  // this thread's halo-plane chunks: global column (-1: none), shared offset
   int cc_g, cc_s;        // this thread's centre-plane chunk
   __device__ __forceinline__ static int wrap(int v, int n) { return ((v % n) + n) % n; }
-  __device__ __forceinline__ RGeom(int x0, int y0, int N_) {
-    N = N_;
-    NN = N * N;
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + RTX * ty;
-    active = (x0 + 2 * tx < N) && (y0 + ty < N);
-    col = wrap(x0 + 2 * tx, N) + N * wrap(y0 + ty, N);
-    csm = (ty + 2) * W + 2 * tx + XH;
+  template <int ce, int xh>
+  __device__ __forceinline__ void chunks(int x0, int y0, int tid) {
+    constexpr int rowc = (TX + 2 * xh) / ce, midc = TX / ce;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int ch = tid + j * RNT;
       ch_g[j] = -1;
       ch_s[j] = 0;
-      if (ch < NCH) {
+      if (ch < ring_nch(ce, xh)) {
         int lx, ly;
-        if (ch < TY * ROWC) {
-          ly = ch / ROWC;
-          lx = (ch % ROWC) * CE - XH;
+        if (ch < TY * rowc) {
+          ly = ch / rowc;
+          lx = (ch % rowc) * ce - xh;
         } else {
-          const int h = ch - TY * ROWC, hr = h / MIDC;
+          const int h = ch - TY * rowc, hr = h / midc;
           ly = hr < 2 ? hr - 2 : TY + hr - 2;
-          lx = (h % MIDC) * CE;
+          lx = (h % midc) * ce;
         }
         ch_g[j] = wrap(x0 + lx, N) + N * wrap(y0 + ly, N);
         ch_s[j] = (ly + 2) * W + lx + XH;
@@ -127,26 +133,40 @@ struct RGeom {
     }
     cc_g = -1;
     cc_s = 0;
-    if (tid < NCC) {
-      const int row = tid / (TX / CE), x = (tid % (TX / CE)) * CE;
+    if (tid < ring_ncc(ce)) {
+      const int row = tid / midc, x = (tid % midc) * ce;
       cc_g = wrap(x0 + x, N) + N * wrap(y0 + row, N);
       cc_s = row * TX + x;
     }
+  }
+  __device__ __forceinline__ RGeom(int x0, int y0, int N_) {
+    N = N_;
+    NN = N * N;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + RTX * ty;
+    active = (x0 + 2 * tx < N) && (y0 + ty < N);
+    col = wrap(x0 + 2 * tx, N) + N * wrap(y0 + ty, N);
+    csm = (ty + 2) * W + 2 * tx + XH;
+    chunks<WIDE ? CE : 2, WIDE ? XH : 2>(x0, y0, tid);
   }
   __device__ __forceinline__ int plane(int k) const { return NN * k; }
   __device__ __forceinline__ int wrapz(int k) const { return k < 0 ? k + N : (k >= N ? k - N : k); }
 };
 
 // Plane m of a tile-with-halo field / of a centre-only field into a ring slot.
-template <typename T>
-__device__ __forceinline__ void zr_issue_halo(const RGeom<T>& G, const T* g, T* slot, int m) {
+template <bool WIDE>
+__device__ __forceinline__ void zr_copy(void* dst, const void* src) {
+  if (WIDE) cp_async16(dst, src);
+  else cp_async8(dst, src);
+}
+template <typename T, bool WIDE>
+__device__ __forceinline__ void zr_issue_halo(const RGeom<T, WIDE>& G, const T* g, T* slot, int m) {
 #pragma unroll
   for (int j = 0; j < 2; ++j)
-    if (G.ch_g[j] >= 0) cp_async16(slot + G.ch_s[j], g + G.ch_g[j] + G.plane(m));
+    if (G.ch_g[j] >= 0) zr_copy<WIDE>(slot + G.ch_s[j], g + G.ch_g[j] + G.plane(m));
 }
-template <typename T>
-__device__ __forceinline__ void zr_issue_centre(const RGeom<T>& G, const T* g, T* slot, int m) {
-  if (G.cc_g >= 0) cp_async16(slot + G.cc_s, g + G.cc_g + G.plane(m));
+template <typename T, bool WIDE>
+__device__ __forceinline__ void zr_issue_centre(const RGeom<T, WIDE>& G, const T* g, T* slot, int m) {
+  if (G.cc_g >= 0) zr_copy<WIDE>(slot + G.cc_s, g + G.cc_g + G.plane(m));
 }
 
 // Stencil view of one field at plane k for cell r (0: x, 1: x+1) of the
@@ -160,7 +180,7 @@ struct ZView {
   template <typename GT>
   __device__ __forceinline__ T at(const GT&, int d, int s) const {
     if (d == 2) return pc<T>(z[2 + s], r);
-    if (d == 1) return pc<T>(ldp(p + csm + s * RGeom<T>::W), r);
+    if (d == 1) return pc<T>(ldp(p + csm + s * RGeom<T>::W), r);  // one layout for both chunk widths
     const int o = r + s;  // -2 .. 3: pair (o >> 1), component (o & 1)
     return pc<T>(ldp(p + csm + 2 * (o >> 1)), o & 1);
   }
@@ -189,10 +209,10 @@ struct ZSlots {
 // Ring plan of one kernel: NSF stencil fields, NFF face arrays, NCF centre
 // fields, A planes of lookahead.  Global pointers are set by the kernel
 // (gs/gf/gc); smem is carved from the dynamic shared allocation.
-template <typename T, int A, int NSF, int NFF, int NCF>
+template <typename T, int A, int NSF, int NFF, int NCF, bool WIDE = true>
 struct RingPlan {
   using SL = ZSlots<A>;
-  using G_ = RGeom<T>;
+  using G_ = RGeom<T, WIDE>;
   static constexpr int HW = G_::HW;
   static constexpr int elems = NSF * SL::NS * HW + NFF * SL::NF * HW + NCF * SL::NC * NTHR;
   static constexpr int bytes = (elems > 0 ? elems : 1) * (int)sizeof(T);
@@ -332,8 +352,8 @@ template <typename T>
 struct Line2 {
   T m2[2], m1[2], p1[2], p2[2];
 };
-template <typename T, typename Plan>
-__device__ __forceinline__ Line2<T> ring_line(const Plan& R, int f, int k, const RGeom<T>& G, int d) {
+template <typename T, bool WIDE, typename Plan>
+__device__ __forceinline__ Line2<T> ring_line(const Plan& R, int f, int k, const RGeom<T, WIDE>& G, int d) {
   Line2<T> L;
   const P2<T> c = R.zq[f][2];
   if (d == 2) {
@@ -356,8 +376,8 @@ __device__ __forceinline__ Line2<T> ring_line(const Plan& R, int f, int k, const
   return L;
 }
 // Only the neighbours at distance 1 (m1, p1; m2, p2 left unset): two reads along x, two along y.
-template <typename T, typename Plan>
-__device__ __forceinline__ Line2<T> ring_line1(const Plan& R, int f, int k, const RGeom<T>& G, int d) {
+template <typename T, bool WIDE, typename Plan>
+__device__ __forceinline__ Line2<T> ring_line1(const Plan& R, int f, int k, const RGeom<T, WIDE>& G, int d) {
   Line2<T> L;
   const P2<T> c = R.zq[f][2];
   if (d == 2) {

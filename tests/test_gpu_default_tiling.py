@@ -79,3 +79,35 @@ def test_one_launch_solves(fe, N, transonic):
     code, x, info = s.solve_pressure(0, torch.zeros_like(bd), dt, 1e-12, 50)
     assert code == fe.FE_OK and info.iters == 0 and not x.any()
     s.close()
+
+
+@pytest.mark.parametrize("N", [10, 22, 30, 34, 66])
+@pytest.mark.parametrize("kind", ["barotropic", "fourier", "two-way", "two-fluid"])
+def test_rings_on_grids_of_8_byte_chunks(fe, N, kind):
+    """FP32 steps on even N that are no multiple of four (ring kernels with 8-byte copies: tiles narrower than
+    the box, ragged, wrapping more than once) against the oracle at the mixed-precision bar."""
+    from oracle import piso
+    nd = 2
+    rho, u, Y, T = random_fields(N, nd, kind == "fourier", seed=N, mach=0.2, noise=0.01)
+    f32 = lambda a: np.asarray(a, dtype=np.float32).astype(np.float64)  # noqa: E731
+    rho, u, Y = f32(rho), [f32(c) for c in u], [f32(y) for y in Y]
+    T = f32(T) if T is not None else None
+    kw = dict(closure=1 if kind == "fourier" else 0, coupling=1 if kind == "two-way" else 0,
+              dust_model=1 if kind == "two-fluid" else 0)
+    prm = piso.Params(N=N, nu=0.005, tau_p=[0.05, 0.1], Y0=[0.01, 0.02], p_tol=1e-10, **kw)
+    ref, _ = piso.step(prm, piso.make_state(prm, rho, u, Y, T))
+    s = fe.Solver([dict(N=N, nu=0.005, tau_p=[0.05, 0.1], Y0=[0.01, 0.02])], precision=fe.FE_FP32_MIXED, p_tol=1e-8,
+                  solver=fe.FE_PCG_POLY, **kw)
+    s.set_state(0, rho, u, Y, T)
+    code, _ = s.step(1)
+    assert code == fe.FE_OK
+    got = s.get_state(0)
+    pairs = [(got["rho"], ref["rho"]), (got["p"], ref["p"])] + list(zip(got["u"] + got["phi"] + got["Y"],
+                                                                         ref["u"] + ref["phi"] + ref["Y"]))
+    if kind == "fourier":
+        pairs.append((got["T"], ref["T"]))
+    if kind == "two-fluid":
+        pairs += [(a, b) for j in range(nd) for a, b in zip(got["V"][j], ref["V"][j])]
+    for a, b in pairs:
+        assert np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(b)
+    s.close()
