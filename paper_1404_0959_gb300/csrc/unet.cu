@@ -213,6 +213,203 @@ __global__ void __launch_bounds__(CONV_WARPS * 32) k_conv(ConvArgs a) {
     }
 }
 
+// ---- staged gather convolution ---------------------------------------------------------------
+// k_conv with its operands staged: a CTA of 8 warps computes a tile of 16 x 4 x 4 (MT = 2), 16 x 8 x 4
+// (4) or 32 x 8 x 4 (8) output voxels, MT 16-voxel m-tiles per warp.  The input voxels that the tile
+// touches are copied into shared memory once, all channels, [channel octet][voxel][8 channels] (an
+// upsampled source at its own resolution), the weights, [tap][channel octet][output channel][8 channels],
+// all at once where they fit, else in groups of taps one group ahead (tap by tap their latency set the
+// pace: 218 us for a 16-channel layer of 128^3 voxels, 174 us with all taps staged); both fragments come
+// by ldmatrix, eight voxels or channels being 128 contiguous bytes.  k_conv gathers every fragment from
+// global memory, the input 27 times and the weights once per 32 voxels (the half-grid layers of a 128^3
+// network: 311 us each, 70 TFLOP/s, against 68 to 147 us).  The order of the matrix instructions of an
+// output (tap, source, channel slice) is k_conv's, so the results are its bits.
+// Modes: same grid, nearest upsampling, stride 2, and the data gradient of stride 1 (negated taps).
+constexpr int kStThreads = 256;
+
+__device__ __forceinline__ unsigned st_smem(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void st_cp16(unsigned dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Staged box of one source: voxels per axis for an output tile of w voxels along the axis.
+__host__ __device__ constexpr int st_extent(int mode, int w) {
+  return mode == G_UP ? w / 2 + 2 : (mode == G_DOWN ? 2 * w + 1 : w + 2);
+}
+constexpr int st_tx(int mt) { return mt == 8 ? 32 : 16; }
+constexpr int st_ty(int mt) { return mt == 2 ? 4 : 8; }
+constexpr int kStTz = 4;
+
+static int st_src_bytes(const Src& s, int mt) {
+  return s.C * 2 * st_extent(s.mode, st_tx(mt)) * st_extent(s.mode, st_ty(mt)) * st_extent(s.mode, kStTz);
+}
+// with the weights in groups of `taps` (27: one buffer, else two)
+static int st_bytes(const ConvArgs& a, int mt, int taps) {
+  return st_src_bytes(a.s0, mt) + (a.s1.C ? st_src_bytes(a.s1, mt) : 0) +
+         (taps == 27 ? 27 : 2 * taps) * a.Cin * a.Cout * 2;
+}
+
+template <int NT, int MT>
+__global__ void __launch_bounds__(kStThreads, NT * MT <= 16 ? 2 : 1) k_conv_st(ConvArgs a, int taps) {
+  constexpr int TXO = MT == 8 ? 32 : 16, TYO = MT == 2 ? 4 : 8, COUT = 8 * NT;
+  extern __shared__ __align__(128) unsigned char st_sm[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, tig = lane & 3;
+  const int ntx = (a.No + TXO - 1) / TXO, nty = (a.No + TYO - 1) / TYO;
+  const int x0 = TXO * (blockIdx.x % ntx), y0 = TYO * ((blockIdx.x / ntx) % nty), z0 = kStTz * (blockIdx.x / (ntx * nty));
+  // staged boxes: extents, voxels, shared base
+  int ex[2], ey[2], nv[2];
+  unsigned sb[2];
+  unsigned base = st_smem(st_sm);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const Src& s = q == 0 ? a.s0 : a.s1;
+    ex[q] = st_extent(s.mode, TXO);
+    ey[q] = st_extent(s.mode, TYO);
+    nv[q] = s.C ? ex[q] * ey[q] * st_extent(s.mode, kStTz) : 0;
+    sb[q] = base;
+    base += nv[q] * s.C * 2;
+  }
+  const unsigned wbuf = base, wtap = (unsigned)(a.Cin * COUT * 2);
+  auto stage_weights = [&](int group) {  // taps group * taps .. + taps - 1
+    const int octs = a.Cin / 8, per = COUT * octs;
+    const bf16* w = a.W + (long)group * taps * COUT * a.Cin;
+    const unsigned dst = wbuf + (group & 1) * taps * wtap;
+    for (int q = tid; q < taps * per; q += kStThreads) {
+      const int c8 = q % octs, r = q / octs, co = r % COUT, t = r / COUT;
+      st_cp16(dst + t * wtap + (unsigned)(c8 * COUT + co) * 16, w + (long)r * a.Cin + 8 * c8);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto wrapv = [](int v, int n) {
+    v += v < 0 ? n : 0;
+    while (v >= n) v -= n;
+    return v;
+  };
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const Src& s = q == 0 ? a.s0 : a.s1;
+    if (s.C == 0) continue;
+    const int lo = __ffs(s.C / 8) - 1;  // log2 of the channel octets (16, 32 or 64 channels)
+    // first voxel of the box on the source's grid; a warp copies rows of voxels
+    const int ox = s.mode == G_UP ? x0 / 2 - 1 : (s.mode == G_DOWN ? 2 * x0 - 1 : x0 - 1);
+    const int oy = s.mode == G_UP ? y0 / 2 - 1 : (s.mode == G_DOWN ? 2 * y0 - 1 : y0 - 1);
+    const int oz = s.mode == G_UP ? z0 / 2 - 1 : (s.mode == G_DOWN ? 2 * z0 - 1 : z0 - 1);
+    const int rows = nv[q] / ex[q];
+    for (int r = warp; r < rows; r += kStThreads / 32) {
+      const int lz = r / ey[q], ly = r - lz * ey[q];
+      const bf16* src = s.ptr + (long)s.n * (wrapv(oy + ly, s.n) + (long)s.n * wrapv(oz + lz, s.n)) * s.C;
+      for (int c = lane; c < ex[q] << lo; c += 32) {
+        const int c8 = c & ((1 << lo) - 1), lx = c >> lo;
+        st_cp16(sb[q] + (unsigned)(c8 * nv[q] + r * ex[q] + lx) * 16, src + wrapv(ox + lx, s.n) * s.C + 8 * c8);
+      }
+    }
+  }
+  stage_weights(0);  // one group with the input
+  float acc[MT][NT][4];
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
+  // this lane's row of an m-tile and channel half for ldmatrix; the warp's m-tiles: one z, MT (x, y) rows
+  const int row = (lane & 7) + (lane & 8), half = lane >> 4;
+  const int zt = warp >> 1, yt = (warp & 1) * (TYO / 2);
+  const int sgn = a.s0.mode == G_SAME_T ? -1 : 1;
+  const int brow = (lane & 7) + ((lane >> 4) << 3), bhalf = (lane >> 3) & 1;
+  for (int t = 0; t < 27; ++t) {
+    const int group = t / taps;
+    if (t == group * taps) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      if (t + taps < 27) stage_weights(group + 1);
+    }
+    const int dz = sgn * (t / 9 - 1), dy = sgn * ((t / 3) % 3 - 1), dx = sgn * (t % 3 - 1);
+    const unsigned wb = wbuf + ((group & 1) * taps + t - group * taps) * wtap + (unsigned)(bhalf * COUT + brow) * 16;
+    int oct = 0;  // channel octet among both sources
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const Src& s = q == 0 ? a.s0 : a.s1;
+      if (s.C == 0) continue;
+      unsigned va[MT];  // shared address of this lane's voxel, per m-tile
+#pragma unroll
+      for (int m = 0; m < MT; ++m) {
+        const int xb = (MT == 8 ? 16 * (m & 1) : 0) + row, yb = yt + (MT == 8 ? m >> 1 : m);
+        int lx, ly, lz;
+        if (s.mode == G_UP) {
+          lx = (xb + 2 + dx) >> 1;
+          ly = (yb + 2 + dy) >> 1;
+          lz = (zt + 2 + dz) >> 1;
+        } else if (s.mode == G_DOWN) {
+          lx = 2 * xb + 1 + dx;
+          ly = 2 * yb + 1 + dy;
+          lz = 2 * zt + 1 + dz;
+        } else {
+          lx = xb + 1 + dx;
+          ly = yb + 1 + dy;
+          lz = zt + 1 + dz;
+        }
+        va[m] = sb[q] + (unsigned)(half * nv[q] + (lz * ey[q] + ly) * ex[q] + lx) * 16;
+      }
+      for (int c = 0; c < s.C / 16; ++c, oct += 2) {
+        uint32_t af[MT][4];
+#pragma unroll
+        for (int m = 0; m < MT; ++m) ldsm4(af[m], va[m] + (unsigned)(2 * c * nv[q]) * 16);
+#pragma unroll
+        for (int n = 0; n < NT; n += 2) {
+          uint32_t bf[4];
+          ldsm4(bf, wb + (unsigned)(oct * COUT + 8 * n) * 16);
+          const uint32_t b0[2] = {bf[0], bf[1]}, b1[2] = {bf[2], bf[3]};
+#pragma unroll
+          for (int m = 0; m < MT; ++m) {
+            mma_bf16(acc[m][n], af[m], b0);
+            mma_bf16(acc[m][n + 1], af[m], b1);
+          }
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < MT; ++m) {
+    const int yo = y0 + yt + (MT == 8 ? m >> 1 : m), zo = z0 + zt;
+    if (yo >= a.No || zo >= a.No) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int xo = x0 + (MT == 8 ? 16 * (m & 1) : 0) + g + 8 * h;
+      if (xo >= a.No) continue;
+      const long v = xo + (long)a.No * (yo + (long)a.No * zo);
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        const int co = 8 * n + 2 * tig;
+        float v0 = acc[m][n][2 * h], v1 = acc[m][n][2 * h + 1];
+        if (a.bias) {
+          v0 += a.bias[co];
+          v1 += a.bias[co + 1];
+        }
+        if (a.relu) {
+          v0 = fmaxf(v0, 0.f);
+          v1 = fmaxf(v1, 0.f);
+        }
+        if (a.out) *reinterpret_cast<__nv_bfloat162*>(a.out + v * COUT + co) = __floats2bfloat162_rn(v0, v1);
+        if (a.out32) {
+          if (a.out32_ch == 1) {
+            if (co == 0) a.out32[v] = v0;
+          } else {
+            *reinterpret_cast<float2*>(a.out32 + v * COUT + co) = make_float2(v0, v1);
+          }
+        }
+      }
+    }
+  }
+}
+
 // Weight gradient: dW[t][co][ci] += sum_v dpre(v)[co] * in(v, t)[ci] over a
 // chunk of voxels, for one tap, one 16-wide co block and one 32-wide ci
 // block per CTA; the 4 warps split the chunk and are reduced in shared
@@ -604,6 +801,54 @@ static int ew(long n) {
   return (int)(g < 152L * 8 ? g : 152L * 8);
 }
 
+// min_taps: the smallest group of weights worth running this tile with
+template <int NT, int MT>
+static bool conv_st(const ConvArgs& a, int min_taps, cudaStream_t st) {
+  const int limit = (NT * MT <= 16 ? 113 : 227) * 1024;  // the resident blocks its registers allow
+  int taps = 27;
+  while (taps > min_taps && st_bytes(a, MT, taps) > limit) taps /= 3;
+  const int bytes = st_bytes(a, MT, taps);
+  if (bytes > limit) return false;
+  if (cudaFuncSetAttribute(k_conv_st<NT, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const int nx = (a.No + st_tx(MT) - 1) / st_tx(MT), ny = (a.No + st_ty(MT) - 1) / st_ty(MT),
+            nz = (a.No + kStTz - 1) / kStTz;
+  k_conv_st<NT, MT><<<nx * ny * nz, kStThreads, bytes, st>>>(a, taps);
+  return true;
+}
+
+// The staged kernel where its modes fit; the largest tile (least staging per voxel, most reuse of the
+// weights) whose accumulators and staged input leave room for two blocks per SM, if the grid still gives
+// every SM one.  The tile counts for more than the group of weights it leaves room for: 48 input
+// channels at 128^3 369 us tap by tap on 32 x 8 x 4, 416 us with all taps staged on 16 x 8 x 4; 96 at 64^3
+// 147 us on 16 x 8 x 4, 161 us in threes on 16 x 4 x 4.
+static bool launch_conv_st(const UNet& U, const ConvArgs& a, cudaStream_t st) {
+  auto fits = [&](const Src& s) {
+    if (s.C == 0) return true;
+    if (s.C != 16 && s.C != 32 && s.C != 64) return false;
+    if (s.mode == G_SAME || s.mode == G_SAME_T) return s.n == a.No;
+    if (s.mode == G_UP) return 2 * s.n == a.No;
+    return s.mode == G_DOWN && s.n == 2 * a.No;
+  };
+  if (a.accumulate || !fits(a.s0) || !fits(a.s1)) return false;
+  if (a.s1.C && (a.s0.mode == G_SAME_T || a.s1.mode == G_SAME_T)) return false;
+  auto blocks = [&](int mt) {
+    return (long)((a.No + st_tx(mt) - 1) / st_tx(mt)) * ((a.No + st_ty(mt) - 1) / st_ty(mt)) *
+           ((a.No + kStTz - 1) / kStTz);
+  };
+  const bool big = blocks(8) >= U.nsm, mid = blocks(4) >= U.nsm;
+  switch (a.Cout / 8) {
+    case 2: return (big && conv_st<2, 8>(a, 1, st)) || (mid && conv_st<2, 4>(a, 1, st)) || conv_st<2, 2>(a, 1, st);
+    case 4: return (mid && conv_st<4, 4>(a, 1, st)) || conv_st<4, 2>(a, 1, st);
+    case 6: return (mid && conv_st<6, 4>(a, 1, st)) || conv_st<6, 2>(a, 1, st);
+    case 8: return conv_st<8, 2>(a, 1, st) || conv_st<8, 4>(a, 1, st);
+    case 12: return conv_st<12, 2>(a, 1, st);
+  }
+  return false;
+}
+
 static void launch_conv(const UNet& U, const ConvArgs& a, cudaStream_t st) {
   // stride-1 gathers (same grid, nearest upsampling) go to the tensor-memory kernel when it fits
   auto tc_mode = [&](const Src& s, int& m) {
@@ -618,6 +863,7 @@ static void launch_conv(const UNet& U, const ConvArgs& a, cudaStream_t st) {
     TcConvArgs t{a.s0.ptr, a.s1.ptr, a.s0.C, a.s1.C, m0, m1, a.No, a.W, a.bias, a.out, a.out32, a.relu, U.err};
     if (conv_tc(t, a.Cout, U.nsm, st)) return;
   }
+  if (launch_conv_st(U, a, st)) return;
   const long nvox = cube(a.No);
   const int grid = (int)((nvox + 16 * CONV_MT * CONV_WARPS - 1) / (16 * CONV_MT * CONV_WARPS));
   switch (a.Cout / 8) {
