@@ -44,6 +44,12 @@ constexpr int kA = FE_RING_A, kA1 = FE_RING_A_LIGHT;
 // 256^3: divergence 0.277 -> 0.248 ms, right-hand side 0.360 -> 0.346 ms per step; four planes for the
 // divergence 0.255).
 constexpr int kArhs = FE_RING_A_RHS, kAdiv = FE_RING_A_DIV;
+// FP64 kernels take the value of a lower z face over from the plane below, where it was the upper one (a
+// sixth of the face operations: 128^3 predictor 867 -> 798 us, assembly 667 -> 599, right-hand side 329 -> 293,
+// dust 620 -> 574, flux divergence 343 -> 299).  FP32 kernels, which are not bound by their arithmetic, form
+// it again: carrying it cost the predictor 2 % in registers.
+template <typename T>
+constexpr bool kCarryZ = sizeof(T) == 8;
 
 template <typename T>
 __device__ __forceinline__ T* Fr(const BoxDev& B, int slot) {
@@ -191,9 +197,19 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_corr(const BoxDev* boxes
 // u_m per axis and one of div along m: the convection from the unscaled 16 I4 at both faces, the compact
 // Laplacian as (28 S1 - 162 u - S2) / 24 (S1, S2: the six neighbours at distance 1 and 2), Gc unscaled;
 // cl = mu / (24 h^2), cd = mu / (48 h), cc = 1 / (16 h).
+// zf (FP64): 16 I4 of u_m at the lower z faces, taken over from the plane below (formed on a tile's first).
 template <typename T, bool WIDE, typename Plan>
-__device__ __forceinline__ void ring_L(const Plan& R, int k, const RGeom<T, WIDE>& G, const T (&php)[3][2],
-                                       const T (&phm)[3][2], T cl, T cd, T cc, T (&L)[3][2], T (&visc)[3][2]) {
+__device__ __forceinline__ void ring_L(const Plan& R, int k, bool first, const RGeom<T, WIDE>& G, const T (&php)[3][2],
+                                       const T (&phm)[3][2], T cl, T cd, T cc, T (&zf)[3][2], T (&L)[3][2],
+                                       T (&visc)[3][2]) {
+  if (kCarryZ<T> && first) {
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const Line2<T> lz = ring_line(R, m, k, G, 2);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) zf[m][r] = i4m16(lz, pc<T>(R.zq[m][2], r), r);
+    }
+  }
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
     T conv[2], lap[2];
@@ -205,7 +221,12 @@ __device__ __forceinline__ void ring_L(const Plan& R, int k, const RGeom<T, WIDE
         const T u = pc<T>(uc, r);
         T cv = T(0);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) cv += php[d][r] * i4p16(l[d], u, r) - phm[d][r] * i4m16(l[d], u, r);
+        for (int d = 0; d < 3; ++d) {
+          const T fp = i4p16(l[d], u, r), fm = kCarryZ<T> && d == 2 ? zf[m][r] : i4m16(l[d], u, r);
+          if (kCarryZ<T> && d == 2) zf[m][r] = fp;
+          cv = fma(php[d][r], fp, cv);
+          cv = fma(-phm[d][r], fm, cv);
+        }
         conv[r] = cv;
         const T s1 = (l[0].m1[r] + l[0].p1[r]) + (l[1].m1[r] + l[1].p1[r]) + (l[2].m1[r] + l[2].p1[r]);
         const T s2 = (l[0].m2[r] + l[0].p2[r]) + (l[1].m2[r] + l[1].p2[r]) + (l[2].m2[r] + l[2].p2[r]);
@@ -247,6 +268,7 @@ __global__ void __launch_bounds__(RNT, sizeof(T) == 4 ? FE_RING_MINB_PRED : FE_R
   const T ih = (T)B.ih, mu = (T)B.mu, dt = (T)B.sc[SC_DT], gam = (T)B.gamma;
   const T cl = mu * ih * ih * T(1.0 / 24.0), cd = mu * ih * T(1.0 / 48.0), cc = ih * T(0.0625);
   const JacobiDiag<T> jd(B.sc[SC_DT], B.ih);
+  T zf[3][2];
   R.prologue(G);
   for (int i = 0; i < t.kend - t.k0; ++i) {
     const int k = t.k0 + i;
@@ -260,7 +282,7 @@ __global__ void __launch_bounds__(RNT, sizeof(T) == 4 ? FE_RING_MINB_PRED : FE_R
     T php[3][2], phm[3][2];
     R.faces2(0, k, G, php, phm);
     T L[3][2], visc[3][2];
-    ring_L(R, k, G, php, phm, cl, cd, cc, L, visc);
+    ring_L(R, k, i == 0, G, php, phm, cl, cd, cc, zf, L, visc);
     T gp[3][2];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
@@ -342,6 +364,7 @@ __global__ void __launch_bounds__(RNT, sizeof(T) == 4 && TW ? 3 : FE_RING_MINB) 
   T* __restrict__ hb[3] = {Fr<T>(B, W_HB0), Fr<T>(B, W_HB1), Fr<T>(B, W_HB2)};
   const T ih = (T)B.ih, mu = (T)B.mu, dt = (T)B.sc[SC_DT];
   const T cl = mu * ih * ih * T(1.0 / 24.0), cd = mu * ih * T(1.0 / 48.0), cc = ih * T(0.0625);
+  T zf[3][2];
   R.prologue(G);
   for (int i = 0; i < t.kend - t.k0; ++i) {
     const int k = t.k0 + i;
@@ -353,7 +376,7 @@ __global__ void __launch_bounds__(RNT, sizeof(T) == 4 && TW ? 3 : FE_RING_MINB) 
     T php[3][2], phm[3][2];
     R.faces2(0, k, G, php, phm);
     T L[3][2], visc[3][2];
-    ring_L(R, k, G, php, phm, cl, cd, cc, L, visc);
+    ring_L(R, k, i == 0, G, php, phm, cl, cd, cc, zf, L, visc);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const T rc = pc<T>(crho, r);
@@ -439,12 +462,25 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_accel(const BoxDev* boxe
 // h D(phi_p I4 Y_j) for both cells of the pair and every class: phi_p = phi - tau_j I4(rho) I4(a_d) at each
 // face (rho, a0..2, Y_j: stencil fields 0, 1..3, 4 + j of the plan; phi: face arrays 0..2).  Lines of rho
 // and a_d along d, and of Y_j along d, each read once; 16 I4 evaluated unscaled, the factors folded.
+// zf (FP64): 16 x the class fluxes of the lower z faces, taken over from the plane below (formed on a tile's
+// first).
 template <typename T, int ND, bool WIDE, typename Plan>
-__device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, const RGeom<T, WIDE>& G, const T (&taup)[ND],
-                                                   T (&fl)[ND][2]) {
+__device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, bool first, const RGeom<T, WIDE>& G,
+                                                   const T (&taup)[ND], T (&zf)[ND][2], T (&fl)[ND][2]) {
   T php[3][2], phm[3][2];
   R.faces2(0, k, G, php, phm);
   const P2<T> rc = R.zq[0][2];
+  if (kCarryZ<T> && first) {
+    const Line2<T> lr = ring_line(R, 0, k, G, 2), la = ring_line(R, 3, k, G, 2);
+#pragma unroll
+    for (int j = 0; j < ND; ++j) {
+      const Line2<T> ly = ring_line(R, 4 + j, k, G, 2);
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+        zf[j][r] = fma(-taup[j] * T(1.0 / 256.0), i4m16(lr, pc<T>(rc, r), r) * i4m16(la, pc<T>(R.zq[3][2], r), r),
+                       phm[2][r]) * i4m16(ly, pc<T>(R.zq[4 + j][2], r), r);
+    }
+  }
 #pragma unroll
   for (int j = 0; j < ND; ++j) fl[j][0] = fl[j][1] = T(0);
 #pragma unroll
@@ -456,7 +492,7 @@ __device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, const R
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         rap[r] = i4p16(lr, pc<T>(rc, r), r) * i4p16(la, pc<T>(ac, r), r);
-        ram[r] = i4m16(lr, pc<T>(rc, r), r) * i4m16(la, pc<T>(ac, r), r);
+        if (!kCarryZ<T> || d < 2) ram[r] = i4m16(lr, pc<T>(rc, r), r) * i4m16(la, pc<T>(ac, r), r);
       }
     }
 #pragma unroll
@@ -465,9 +501,17 @@ __device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, const R
       const Line2<T> ly = ring_line(R, 4 + j, k, G, d);
       const P2<T> yc = R.zq[4 + j][2];
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
-        fl[j][r] += fma(-tq, rap[r], php[d][r]) * i4p16(ly, pc<T>(yc, r), r) -
-                    fma(-tq, ram[r], phm[d][r]) * i4m16(ly, pc<T>(yc, r), r);
+      for (int r = 0; r < 2; ++r) {
+        const T cp = fma(-tq, rap[r], php[d][r]), yp = i4p16(ly, pc<T>(yc, r), r);
+        if (!kCarryZ<T> || d < 2) {
+          fl[j][r] = fma(cp, yp, fl[j][r]);
+          fl[j][r] = fma(-fma(-tq, ram[r], phm[d][r]), i4m16(ly, pc<T>(yc, r), r), fl[j][r]);
+        } else {
+          const T f = cp * yp;
+          fl[j][r] += f - zf[j][r];
+          zf[j][r] = f;
+        }
+      }
     }
   }
 #pragma unroll
@@ -495,6 +539,7 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fluxn(const BoxDev* boxe
     taup[j] = (T)B.tau_p[j];
     fyn[j] = Fr<T>(B, W_FYN0 + j);
   }
+  T zf[ND][2];
   R.prologue(G);
   for (int i = 0; i < t.kend - t.k0; ++i) {
     const int k = t.k0 + i;
@@ -502,7 +547,7 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fluxn(const BoxDev* boxe
     if (!G.active) continue;
     const int c = G.col + G.plane(k);
     T fl[ND][2];
-    ring_particle_flux<T, ND>(R, k, G, taup, fl);
+    ring_particle_flux<T, ND>(R, k, i == 0, G, taup, zf, fl);
 #pragma unroll
     for (int j = 0; j < ND; ++j) stp(fyn[j] + c, fl[j][0] * ih, fl[j][1] * ih);
   }
@@ -555,6 +600,7 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_dust(const BoxDev* boxes
   T* __restrict__ pout = Fr<T>(B, S(kset, F_P));
   SumAcc<T> amass, abad;
   DotAcc<T> aen, ady[ND];
+  T zf[ND][2];
   R.prologue(G);
   for (int i = 0; i < t.kend - t.k0; ++i) {
     const int k = t.k0 + i;
@@ -564,7 +610,7 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_dust(const BoxDev* boxes
     const P2<T> crn = R.cen(0, k, tid);
     T oy[ND][2], op[2], oe[2], ot[2];
     T flx[ND][2];
-    ring_particle_flux<T, ND>(R, k, G, taup, flx);
+    ring_particle_flux<T, ND>(R, k, i == 0, G, taup, zf, flx);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const T rk = pc<T>(R.zq[0][2], r);
@@ -848,6 +894,7 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_rhs(const BoxDev* boxes,
   T* __restrict__ r0 = Fr<T>(B, K_R);
   const T ih = (T)B.ih, dt = (T)B.sc[SC_DT], idt = T(1) / dt, dih = dt * ih;
   DotAcc<T> abb, abz;
+  T zf[2];
   R.prologue(G);
   for (int i = 0; i < t.kend - t.k0; ++i) {
     const int k = t.k0 + i;
@@ -867,9 +914,16 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_rhs(const BoxDev* boxes,
       for (int r = 0; r < 2; ++r) {
         const T rc = pc<T>(rpc, r), h = pc<T>(hc, r), p = pc<T>(pcc, r);
         const T fp = i4p16(lr, rc, r) * i4p16(lh, h, r) * T(1.0 / 256.0) - dih * (lp.p1[r] - p);
-        const T fm = i4m16(lr, rc, r) * i4m16(lh, h, r) * T(1.0 / 256.0) - dih * (p - lp.m1[r]);
+        if (!kCarryZ<T> || d < 2 || i == 0) {
+          const T fm = i4m16(lr, rc, r) * i4m16(lh, h, r) * T(1.0 / 256.0) - dih * (p - lp.m1[r]);
+          if (kCarryZ<T> && d == 2) zf[r] = fm;
+          else dsum[r] += fp - fm;
+        }
         ops[d][r] = fp;
-        dsum[r] += fp - fm;
+        if (kCarryZ<T> && d == 2) {
+          dsum[r] += fp - zf[r];
+          zf[r] = fp;
+        }
       }
     }
 #pragma unroll
