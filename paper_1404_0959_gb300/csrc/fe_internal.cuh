@@ -476,27 +476,30 @@ __device__ bool sum_partials_last(const BoxDev& B, double* part, double* res, in
 // whether this is the box's last block; if so `res` (shared) holds the box
 // totals (partials added in block order).  Must be called by all threads.
 // tile0/ntiles: the box's block range in the work list of this launch.
+// An FP64 instruction costs a warp 16 clocks however many of its lanes are wanted: each warp stops
+// at four lanes, and one warp per value adds what is left (few values; many: one lane, for the room).
 template <int K>
 __device__ bool block_sum_last(double (&v)[K], const BoxDev& B, double* part, double* res, int tile0, int ntiles) {
-  __shared__ double red[K][kMaxWarps];
+  constexpr int LEFT = K <= 3 ? 4 : 1;
+  __shared__ double red[K][kMaxWarps * LEFT];
   const int tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
-  const int lane = tid & 31, warp = tid >> 5;
+  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
 #pragma unroll
   for (int q = 0; q < K; ++q) {
     double s = v[q];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) red[q][warp] = s;
+    for (int o = 16; o >= LEFT; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane < LEFT) red[q][warp * LEFT + lane] = s;
   }
   __syncthreads();
-  if (tid == 0) {
+  for (int q = warp; q < K; q += nw) {
+    double s = 0.0;
+    for (int w = lane; w < LEFT * nw; w += 32) s += red[q][w];
 #pragma unroll
-    for (int q = 0; q < K; ++q) {
-      double s = 0.0;
-      for (int w = 0; w < nt / 32; ++w) s += red[q][w];
-      part[(size_t)blockIdx.x * MAXP + q] = s;
-    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) part[(size_t)blockIdx.x * MAXP + q] = s;
   }
+  __syncthreads();
   return sum_partials_last<K>(B, part, res, tile0, ntiles);
 }
 // Float-pair values: the warp and block trees add pairs on the FP32 pipe.

@@ -118,7 +118,8 @@ __device__ __forceinline__ void chunk_loop(const Chunk& ch, int tid, F4 f4, F1 f
   }
 }
 
-// r = b, x = 0, pd = z = b / diag; rz = <r, z>, bb = <b, b>.
+// r = b, x = 0, pd = z = b / diag; rz = <r, z>, bb = <b, b>.  FP64 fields: z also to K_AUX, from which the
+// fused iteration takes it (see k_cg_rupdate).
 template <typename T>
 __global__ void __launch_bounds__(NTHR) k_cg_init(const BoxDev* boxes, const int2* work, double* part, int* active) {
   const Chunk ch = chunk_of(boxes, work);
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(NTHR) k_cg_init(const BoxDev* boxes, const int
   T* __restrict__ r = F<T>(B, K_R);
   T* __restrict__ x = F<T>(B, K_X);
   T* __restrict__ pd = F<T>(B, K_PD);
+  T* __restrict__ zs = sizeof(T) == 8 ? F<T>(B, K_AUX) : nullptr;
   const T keep = B.sc[SC_ODONE] != 0.0 ? T(0) : T(1);  // refinement already converged for this box
   DotAcc<T> a0, a1;
   chunk_loop(
@@ -145,6 +147,7 @@ __global__ void __launch_bounds__(NTHR) k_cg_init(const BoxDev* boxes, const int
         st4(r + q0, bv);
         st4(x + q0, zero);
         st4(pd + q0, zv);
+        if (sizeof(T) == 8) st4(zs + q0, zv);
       },
       [&](int c) {
         T bc = b[c] * keep;
@@ -152,6 +155,7 @@ __global__ void __launch_bounds__(NTHR) k_cg_init(const BoxDev* boxes, const int
         r[c] = bc;
         x[c] = T(0);
         pd[c] = z;
+        if (sizeof(T) == 8) zs[c] = z;
         a0.add(bc, z);
         a1.add(bc, bc);
       });
@@ -299,9 +303,12 @@ __global__ void __launch_bounds__(NTHR) kz_cg_matvec(const BoxDev* boxes, const 
 // the iteration counter (neighbouring tiles still read pd_old as halo).  At
 // iteration 0 alpha = beta = 0 (set by k_cg_init) and pd_new = D^{-1} b.
 // POLY: pd_new = z + beta pd_old with z = P r from kz_cg_rpoly (the first-order Neumann
-// polynomial preconditioner), z read in place of r and D^{-1}.
+// polynomial preconditioner), z read in place of r and D^{-1}.  FP64 fields run this form with
+// z = D^{-1} r from k_cg_rupdate: one FP64 operation per cell and halo cell instead of two, and with the
+// lighter loads three blocks fit an SM (128^3: 99 us per launch; 90 with z, 72 with three blocks; four
+// blocks or one plane of lookahead less 72, tiles of 16 planes 76).
 template <typename T, bool POLY>
-__global__ void __launch_bounds__(NTHR, sizeof(T) == 4 ? FE_DM_MINB : 2) kz_cg_dirmatvec(const BoxDev* boxes, const int2* work, double* part) {
+__global__ void __launch_bounds__(NTHR, sizeof(T) == 4 ? FE_DM_MINB : 3) kz_cg_dirmatvec(const BoxDev* boxes, const int2* work, double* part) {
   const TileXYZ t = tile_xyz(boxes, work);
   const BoxDev& B = boxes[t.box];
   if (box_done(B)) return;
@@ -310,13 +317,13 @@ __global__ void __launch_bounds__(NTHR, sizeof(T) == 4 ? FE_DM_MINB : 2) kz_cg_d
   const int odd = ((int)B.sc[SC_ITERS]) & 1;
   const T* __restrict__ po = F<T>(B, odd ? K_PP : K_PD);
   T* __restrict__ pn = F<T>(B, odd ? K_PD : K_PP);
-  const T* __restrict__ r = F<T>(B, POLY ? K_Z : K_R);  // POLY: z
+  const T* __restrict__ r = F<T>(B, POLY ? (sizeof(T) == 8 ? K_AUX : K_Z) : K_R);  // POLY: z
   const T* __restrict__ dinv = F<T>(B, W_DINV);
   T* __restrict__ x = F<T>(B, K_X);
   T* __restrict__ q = F<T>(B, K_Q);
   const T alpha = (T)B.sc[SC_ALPHA], beta = (T)B.sc[SC_BETA];
   const T dt = (T)B.sc[SC_KDT], ih = (T)B.ih, idt = T(1) / dt;
-  const T lapc = T(0.5) * dt * ih * ih;
+  const T lapc = T(0.5) * dt * ih * ih, lap6 = T(6) * lapc;
   // first iteration of a solve: pd_new = D^{-1} r (POLY: z) and x = 0 whatever pd_old and x hold
   const bool first = B.sc[SC_ITERS] == 0.0;
   auto dir = [&](T rv, T dv, T pv) {
@@ -383,7 +390,8 @@ __global__ void __launch_bounds__(NTHR, sizeof(T) == 4 ? FE_DM_MINB : 2) kz_cg_d
       const int c = G.col + G.plane(k);
       const T* s = sm + G.csm;
       const T nb = (s[-1] + s[1]) + (s[-ZGeom<1>::W] + s[ZGeom<1>::W]) + (zm + zp);
-      const T y = ps * zc * idt - lapc * (nb - T(6) * zc);
+      // FP64: the diagonal psi/dt + 6 lapc in one multiply-add
+      const T y = sizeof(T) == 8 ? fma(fma(ps, idt, lap6), zc, -lapc * nb) : ps * zc * idt - lapc * (nb - T(6) * zc);
       q[c] = y;
       pn[c] = zc;
       x[c] = first ? T(0) : xv + alpha * oc;
@@ -658,7 +666,8 @@ __device__ void cg_update_scalars(const BoxDev& B, double rz, double rr, int* ac
 }
 
 // r -= alpha q; rz = <r, D^{-1} r>; convergence test on ||r|| (the update of
-// the fused iteration: x is advanced by kz_cg_dirmatvec).
+// the fused iteration: x is advanced by kz_cg_dirmatvec).  FP64 fields: z = D^{-1} r is stored for the next
+// direction (K_AUX), which then does not form it again on its cells and their halo.
 template <typename T>
 __global__ void __launch_bounds__(NTHR) k_cg_rupdate(const BoxDev* boxes, const int2* work, double* part, int* active) {
   const Chunk ch = chunk_of(boxes, work);
@@ -668,6 +677,7 @@ __global__ void __launch_bounds__(NTHR) k_cg_rupdate(const BoxDev* boxes, const 
   const T* __restrict__ qv = F<T>(B, K_Q);
   const T* __restrict__ dinv = F<T>(B, W_DINV);
   T* __restrict__ r = F<T>(B, K_R);
+  T* __restrict__ zs = sizeof(T) == 8 ? F<T>(B, K_AUX) : nullptr;
   const T alpha = (T)B.sc[SC_ALPHA];
   DotAcc<T> a0, a1;
   chunk_loop(
@@ -677,15 +687,18 @@ __global__ void __launch_bounds__(NTHR) k_cg_rupdate(const BoxDev* boxes, const 
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           rv.v[e] -= alpha * qq.v[e];
-          a0.add(rv.v[e], rv.v[e] * dv.v[e]);
+          dv.v[e] *= rv.v[e];
+          a0.add(rv.v[e], dv.v[e]);
           a1.add(rv.v[e], rv.v[e]);
         }
         st4(r + q0, rv);
+        if (sizeof(T) == 8) st4(zs + q0, dv);
       },
       [&](int c) {
-        T rc = r[c] - alpha * qv[c];
+        const T rc = r[c] - alpha * qv[c], zc = rc * dinv[c];
         r[c] = rc;
-        a0.add(rc, rc * dinv[c]);
+        if (sizeof(T) == 8) zs[c] = zc;
+        a0.add(rc, zc);
         a1.add(rc, rc);
       });
   Red<T> v[2] = {a0.red(), a1.red()};
@@ -1895,7 +1908,7 @@ template <typename T> void launch_cg_fused(const Launch& L) {
     FE_LAUNCH(L, KID_CG_DIRMATVEC, (kb_cg_dirmatvec<T, false, kBulkCells><<<L.nbblocks, kBulkThreads, L.bsmem, L.st>>>(
                                        L.boxes, L.bwork, L.part)));
   else
-    FE_LAUNCH(L, KID_CG_DIRMATVEC, (kz_cg_dirmatvec<T, false><<<GRID>>>(L.kboxes, L.kwork, L.part)));
+    FE_LAUNCH(L, KID_CG_DIRMATVEC, (kz_cg_dirmatvec<T, sizeof(T) == 8><<<GRID>>>(L.kboxes, L.kwork, L.part)));
   FE_LAUNCH(L, KID_CG_RUPDATE, (k_cg_rupdate<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
 }
 // First polynomial-preconditioned residual z = P r of an inner solve and <r, z> (nothing without it)
