@@ -410,113 +410,6 @@ __global__ void __launch_bounds__(kStThreads, NT * MT <= 16 ? 2 : 1) k_conv_st(C
   }
 }
 
-// Weight gradient: dW[t][co][ci] += sum_v dpre(v)[co] * in(v, t)[ci] over a
-// chunk of voxels, for one tap, one 16-wide co block and one 32-wide ci
-// block per CTA; the 4 warps split the chunk and are reduced in shared
-// memory before one FP32 atomic add per weight.
-struct WgradArgs {
-  Src s0, s1;
-  int Cin, Cout, No;
-  const bf16* dpre;  // [No^3][Cout]
-  float* dW;         // [27][Cout][Cin]
-  long chunk;        // voxels per CTA
-};
-
-__device__ __forceinline__ uint32_t pack2(bf16 lo, bf16 hi) {
-  return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
-
-__global__ void __launch_bounds__(CONV_WARPS * 32) k_wgrad(WgradArgs a) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int g = lane >> 2, tig = lane & 3;
-  const int t = blockIdx.y;
-  const int co0 = 16 * (blockIdx.z % (a.Cout / 16 > 0 ? a.Cout / 16 : 1));
-  const int ci0 = 32 * (blockIdx.z / (a.Cout / 16 > 0 ? a.Cout / 16 : 1));
-  const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-  const long nvox = (long)a.No * a.No * a.No;
-  const long v0 = (long)blockIdx.x * a.chunk;
-  const long v1 = v0 + a.chunk < nvox ? v0 + a.chunk : nvox;
-  const int ncb = a.Cin - ci0 < 32 ? (a.Cin - ci0) / 8 : 4;  // n-tiles in this ci block
-  const bool row0 = co0 + g < a.Cout, row1 = co0 + g + 8 < a.Cout;
-  float acc[4][4];
-#pragma unroll
-  for (int n = 0; n < 4; ++n)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
-  // warp w takes k-steps w, w + 4, ...
-  for (long kb = v0 + 16 * warp; kb < v1; kb += 16 * CONV_WARPS) {
-    // this thread's 4 voxels: kb + 2 tig + {0, 1, 8, 9}
-    long vv[4] = {kb + 2 * tig, kb + 2 * tig + 1, kb + 2 * tig + 8, kb + 2 * tig + 9};
-    bf16 dp[2][4];  // rows co0 + g, co0 + g + 8
-    int gi0[4], gi1[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const bool ok = vv[q] < v1;
-      const long v = ok ? vv[q] : v0;
-      const int x = (int)(v % a.No), y = (int)((v / a.No) % a.No), z = (int)(v / ((long)a.No * a.No));
-      gi0[q] = ok ? gather_index(a.s0, x, y, z, dx, dy, dz, a.No) : -1;
-      gi1[q] = ok && a.s1.C ? gather_index(a.s1, x, y, z, dx, dy, dz, a.No) : -1;
-      const bf16 zero = __float2bfloat16(0.f);
-      dp[0][q] = ok && row0 ? a.dpre[v * a.Cout + co0 + g] : zero;
-      dp[1][q] = ok && row1 ? a.dpre[v * a.Cout + co0 + g + 8] : zero;
-    }
-    // A (16 co x 16 voxels): a0 = (g, 2tig..+1), a1 = (g+8, ..), a2 = (g, 2tig+8..+9), a3 = (g+8, ..)
-    uint32_t af[4] = {pack2(dp[0][0], dp[0][1]), pack2(dp[1][0], dp[1][1]), pack2(dp[0][2], dp[0][3]),
-                      pack2(dp[1][2], dp[1][3])};
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-      if (n >= ncb) break;
-      const int ci = ci0 + 8 * n + g;
-      const bool in0 = ci < a.s0.C;
-      bf16 b[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int id = in0 ? gi0[q] : gi1[q];
-        const Src& s = in0 ? a.s0 : a.s1;
-        const int cc = in0 ? ci : ci - a.s0.C;
-        b[q] = id < 0 ? __float2bfloat16(0.f) : s.ptr[(long)id * s.C + cc];
-      }
-      uint32_t bfr[2] = {pack2(b[0], b[1]), pack2(b[2], b[3])};
-      mma_bf16(acc[n], af, bfr);
-    }
-  }
-  // reduce the 4 warps in shared memory, then one atomic per weight
-  __shared__ float red[CONV_WARPS][16][32];
-#pragma unroll
-  for (int n = 0; n < 4; ++n) {
-    const int col = 8 * n + 2 * tig;
-    red[warp][g][col] = acc[n][0];
-    red[warp][g][col + 1] = acc[n][1];
-    red[warp][g + 8][col] = acc[n][2];
-    red[warp][g + 8][col + 1] = acc[n][3];
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < 16 * 32; e += CONV_WARPS * 32) {
-    const int r = e / 32, col = e % 32;
-    if (col >= 8 * ncb || co0 + r >= a.Cout) continue;
-    const float s = red[0][r][col] + red[1][r][col] + red[2][r][col] + red[3][r][col];
-    atomicAdd(&a.dW[((long)t * a.Cout + co0 + r) * a.Cin + ci0 + col], s);
-  }
-}
-
-// bias gradient: db[co] += sum_v dpre(v)[co] (one block per chunk)
-__global__ void k_bgrad(const bf16* dpre, long nvox, int Cout, float* db) {
-  __shared__ float red[256];
-  for (int co = 0; co < Cout; ++co) {
-    float s = 0.f;
-    for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < nvox; v += (long)gridDim.x * blockDim.x)
-      s += __bfloat162float(dpre[v * Cout + co]);
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(&db[co], red[0]);
-    __syncthreads();
-  }
-}
-
 // dpre = bf16(d * (act > 0))  (act null: no mask), optional second addend
 __global__ void k_mask(const float* d, const float* d2, const bf16* act, long n, bf16* out) {
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
@@ -802,6 +695,182 @@ static int ew(long n) {
 }
 
 // min_taps: the smallest group of weights worth running this tile with
+// ---- weight and bias gradients ---------------------------------------------------------------
+// dW[t][co][ci] += sum_v dpre(v)[co] in(v, t)[ci].
+// A CTA has a chunk of consecutive voxels (64 per layer), the three taps of one (dz, dy), one slice of 16 input
+// channels and up to 32 output channels.  It walks over the chunk in batches of 256 voxels (128 at stride 2): the
+// input row of every row that a batch touches and the batch's dpre are copied into shared memory, [channel octet]
+// [voxel][8 channels], the next batch's behind the current one's products, and both fragments come by ldmatrix
+// with transposition, sixteen consecutive voxels being one K step; each lane finds its voxel's row, so a step may
+// straddle rows and planes.  A warp holds 3 taps x 16 x 16 sums in registers and reads its dpre fragment once for
+// the three (nine taps of one dz per warp: a third of the dpre copies, but 192 CTAs of four warps for a 16-channel
+// layer leave the chip idle: 637 us a 64^3 step; the same with the three dy in twelve warps: 629).  The order of
+// the sums is fixed: four chains of K steps per chunk (step j to chain j mod 4), added in order, then one atomic
+// per weight and chunk -- a gradient near zero decides the sign of a first Adam step, so sums must not move by more
+// than the order of the 64 atomics moves them.
+// With one tap per CTA and every fragment element gathered from global memory (2 bytes a load) the input was
+// read 27 times: 4.1 ms of the 6.3 ms of a 64^3 training step, 0.50 ms now.
+struct WgradArgs {
+  Src s0, s1;
+  int Cin, Cout, No;
+  const bf16* dpre;  // [No^3][Cout]
+  float* dW;         // [27][Cout][Cin]
+  long chunk;        // voxels per chunk, a multiple of 16
+};
+
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+// batch length, staged row length and most rows of a batch on an output grid of side N
+__host__ __device__ constexpr int wg_run(int mode) { return mode == G_DOWN ? 128 : 256; }
+__host__ __device__ constexpr int wg_pitch(int mode, int N) {
+  const int w = N < wg_run(mode) ? N : wg_run(mode);
+  return mode == G_UP ? w / 2 + 2 : (mode == G_DOWN ? 2 * w + 1 : w + 2);
+}
+__host__ __device__ constexpr int wg_rows(int mode, int N) { return (N + wg_run(mode) - 2) / N + 1; }
+// one buffer: two channel octets of the input rows, the batch's dpre
+static int wg_stage_bytes(int mode, int N, int cout) {
+  return wg_rows(mode, N) * wg_pitch(mode, N) * 32 + wg_run(mode) * cout * 2;
+}
+
+__global__ void __launch_bounds__(256) k_wgrad(WgradArgs a) {
+  extern __shared__ __align__(128) unsigned char st_sm[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
+  const int g = lane >> 2, tig = lane & 3;
+  const int slices = a.Cin / 16, slice = blockIdx.z % slices, co0 = 32 * (blockIdx.z / slices);
+  const bool first = 16 * slice < a.s0.C;
+  const Src s = first ? a.s0 : a.s1;
+  const bf16* in = s.ptr + 16 * slice - (first ? 0 : a.s0.C);
+  const int mode = s.mode, No = a.No, dz = (int)blockIdx.y / 3 - 1, dy = (int)blockIdx.y % 3 - 1;
+  const int V = wg_run(mode), P = wg_pitch(mode, No), np = wg_rows(mode, No) * P;
+  const int ncb = nwarp / 4, lco = ncb;  // blocks of 16 output channels; log2 of their octets (1 -> 2, 2 -> 4)
+  const unsigned base = st_smem(st_sm), stage = (unsigned)(np * 32 + V * ncb * 32);
+  const long nvox = (long)No * No * No, vc = (long)blockIdx.x * a.chunk;
+  const long v1 = vc + a.chunk < nvox ? vc + a.chunk : nvox;
+  const int chain = warp & 3, cob = warp >> 2;
+  auto wrapv = [](int v, int n) {
+    v += v < 0 ? n : 0;
+    while (v >= n) v -= n;
+    return v;
+  };
+  // first source voxel of a staged row, relative to the row: of the batch's first row (which begins at x0) or a later one
+  auto row_origin = [&](bool head, int x0) {
+    return !head ? -1 : (mode == G_UP ? (x0 - 1) >> 1 : (mode == G_DOWN ? 2 * x0 - 1 : x0 - 1));
+  };
+  auto along = [&](int v, int d) {  // source coordinate, not wrapped
+    return mode == G_UP ? (v + d) >> 1 : (mode == G_DOWN ? 2 * v + d : v + d);
+  };
+  auto across = [&](int v, int d) {
+    return mode == G_UP ? wrapn(v + d, No) >> 1 : wrapn(mode == G_DOWN ? 2 * v + d : v + d, s.n);
+  };
+  auto copy = [&](long v0, unsigned dst) {
+    const long vend = v0 + V < v1 ? v0 + V : v1;
+    const int R0 = (int)(v0 / No), x0 = (int)(v0 - (long)R0 * No), nr = (int)((vend - 1) / No) - R0 + 1;
+    for (int lr = warp; lr < nr; lr += nwarp) {
+      const int R = R0 + lr, z = R / No, y = R - z * No;
+      const bf16* src = in + (long)s.n * (across(y, dy) + (long)s.n * across(z, dz)) * s.C;
+      const int xo = row_origin(lr == 0, x0);
+      for (int c = lane; c < 2 * P; c += 32) {
+        const int c8 = c & 1, lx = c >> 1;
+        st_cp16(dst + (unsigned)(c8 * np + lr * P + lx) * 16, src + wrapv(xo + lx, s.n) * s.C + 8 * c8);
+      }
+    }
+    const unsigned dd = dst + np * 32;
+    for (int q = tid; q < V << lco; q += blockDim.x) {
+      const int c8 = q & ((1 << lco) - 1), v = q >> lco;
+      const unsigned d = dd + (unsigned)(c8 * V + v) * 16;
+      if (v0 + v < v1)
+        st_cp16(d, a.dpre + (v0 + v) * a.Cout + co0 + 8 * c8);
+      else
+        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0) : "memory");
+    }
+  };
+  float acc[3][2][4];
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[t][n][e] = 0.f;
+  // ldmatrix rows of this lane: voxel and octet of the dpre fragment and of the input fragment
+  const int ak = (lane & 7) + ((lane >> 4) << 3), aoct = 2 * cob + ((lane >> 3) & 1);
+  const int bk = lane & 15, boct = lane >> 4;
+  int cur = 0;
+  copy(vc, base);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (long v0 = vc; v0 < v1; v0 += V, cur ^= 1) {
+    if (v0 + V < v1) copy(v0 + V, base + (cur ^ 1) * stage);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    const int R0 = (int)(v0 / No), x0 = (int)(v0 - (long)R0 * No), left = (int)(v1 - v0 < V ? v1 - v0 : V);
+    const unsigned ib = base + cur * stage + (unsigned)(boct * np) * 16;
+    const unsigned db = base + cur * stage + (unsigned)(np * 32) + (unsigned)(aoct * V + ak) * 16;
+    for (int j = 16 * chain; j < left; j += 64) {
+      uint32_t af[4];
+      ldsm4t(af, db + (unsigned)j * 16);
+      // the lane's voxel (past the end: dpre is 0 there, any staged voxel serves)
+      const int l = x0 + (j + bk < left ? j + bk : left - 1), lr = l / No, x = l - lr * No;
+      const int xo = row_origin(lr == 0, x0);
+      const unsigned row = ib + (unsigned)(lr * P) * 16;
+#pragma unroll
+      for (int tx = 0; tx < 3; ++tx) {
+        uint32_t bf[4];
+        ldsm4t(bf, row + (unsigned)(along(x, tx - 1) - xo) * 16);
+        const uint32_t b0[2] = {bf[0], bf[1]}, b1[2] = {bf[2], bf[3]};
+        mma_bf16(acc[tx][0], af, b0);
+        mma_bf16(acc[tx][1], af, b1);
+      }
+    }
+    __syncthreads();
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  float* red = reinterpret_cast<float*>(st_sm);  // [3][16 ncb][16]
+  for (int q = 0; q < 4; ++q) {
+    __syncthreads();
+    if (chain != q) continue;
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int co = 16 * cob + g + 8 * (e >> 1), ci = 8 * n + 2 * tig + (e & 1);
+          float* r = red + (t * 16 * ncb + co) * 16 + ci;
+          const float v = q > 0 ? *r + acc[t][n][e] : acc[t][n][e];
+          if (q < 3) *r = v;
+          else atomicAdd(a.dW + ((long)(3 * blockIdx.y + t) * a.Cout + co0 + co) * a.Cin + 16 * slice + ci, v);
+        }
+  }
+}
+
+// bias gradient: db[co] += sum_v dpre(v)[co]; a block takes 8 channels, 16 bytes a voxel (one channel after the
+// other, 2 bytes a load: 0.27 ms of a 64^3 training step)
+__global__ void k_bgrad(const bf16* dpre, long nvox, int Cout, float* db) {
+  __shared__ float red[8][256];
+  float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < nvox; v += (long)gridDim.x * blockDim.x) {
+    const uint4 u = *reinterpret_cast<const uint4*>(dpre + v * Cout + 8 * blockIdx.y);
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      s[2 * c] += __uint_as_float(w[c] << 16);
+      s[2 * c + 1] += __uint_as_float(w[c] & 0xFFFF0000u);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c) red[c][threadIdx.x] = s[c];
+  __syncthreads();
+  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    for (int q = threadIdx.x; q < 8 * o; q += blockDim.x) red[q / o][q % o] += red[q / o][q % o + o];
+    __syncthreads();
+  }
+  if (threadIdx.x < 8) atomicAdd(&db[8 * blockIdx.y + threadIdx.x], red[threadIdx.x][0]);
+}
+
 template <int NT, int MT>
 static bool conv_st(const ConvArgs& a, int min_taps, cudaStream_t st) {
   const int limit = (NT * MT <= 16 ? 113 : 227) * 1024;  // the resident blocks its registers allow
@@ -931,24 +1000,16 @@ static void bwd_data(UNet& U, int l, int n_in, float* dIn, cudaStream_t st) {
 
 static void wgrad(UNet& U, int l, Src s0, Src s1, cudaStream_t st) {
   Layer& y = U.L[l];
-  WgradArgs a;
-  a.s0 = s0;
-  a.s1 = s1;
-  a.Cin = y.cin;
-  a.Cout = y.cout;
-  a.No = U.N >> y.level_out;
-  a.dpre = U.dpre;
-  a.dW = y.gw;
+  WgradArgs a{s0, s1, y.cin, y.cout, U.N >> y.level_out, U.dpre, y.gw, 0};
   const long nvox = cube(a.No);
-  const int coblocks = y.cout >= 16 ? y.cout / 16 : 1;
-  const int ciblocks = (y.cin + 31) / 32;
-  long nchunk = 64;
-  a.chunk = (nvox + nchunk - 1) / nchunk;
-  a.chunk = (a.chunk + 15) / 16 * 16;
-  nchunk = (nvox + a.chunk - 1) / a.chunk;
-  dim3 grid((unsigned)nchunk, 27, coblocks * ciblocks);
-  k_wgrad<<<grid, CONV_WARPS * 32, 0, st>>>(a);
-  k_bgrad<<<64, 256, 0, st>>>(U.dpre, nvox, y.cout, y.gb);
+  a.chunk = ((nvox + 63) / 64 + 15) / 16 * 16;
+  const int co = y.cout < 32 ? y.cout : 32;
+  int bytes = wg_stage_bytes(s0.mode, a.No, co);
+  if (s1.C) bytes = std::max(bytes, wg_stage_bytes(s1.mode, a.No, co));
+  bytes = std::max(2 * bytes, 3 * co * 16 * 4);
+  cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  k_wgrad<<<dim3((unsigned)((nvox + a.chunk - 1) / a.chunk), 9, y.cin / 16 * (y.cout / co)), 8 * co, bytes, st>>>(a);
+  k_bgrad<<<dim3(64, y.cout / 8), 256, 0, st>>>(U.dpre, nvox, y.cout, y.gb);
 }
 
 }  // namespace fe

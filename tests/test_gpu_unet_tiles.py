@@ -60,3 +60,11 @@ def test_gradients_on_ragged_tiles(fe, N):  # noqa: F811
     errs = {n + k: base.rel(g[n + k], G[n + k]) for n in base.NAMES for k in (".W", ".b")}
     assert max(errs.values()) < 3e-2, errs
     s.close()
+
+
+@pytest.mark.parametrize("N", [16, 28, 44, 52])
+def test_weight_gradients_on_staged_tiles(fe, N):  # noqa: F811
+    """The staged weight gradients where a grid is smaller than the 16 x 4 x 4 (stride 2: 16 x 4 x 2) voxel tile,
+    of odd size (28: 14 and 7; 44: 22 and 11), or leaves remainders along every axis; accumulation in FP32 of the
+    same BF16 products, so the bars of the gradients above hold."""
+    test_gradients_on_ragged_tiles(fe, N)
