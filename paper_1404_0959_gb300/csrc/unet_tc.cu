@@ -365,17 +365,22 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_conv_tc(TcConvArgs a) {
 // 4.4 us per (tile, slice) at 128^3.  Here one ring of units -- unit = the R + 2 rows of one z plane and one
 // 16-channel slice -- holds the planes z-1 .. z+1 of all slices plus what is staged ahead, so a tile needs one
 // new plane (a third of the copies and of the L2 reads), the copies run two units ahead behind their own warps,
-// and the epilogue has warps of its own.  What bounds it then is the issue of the MMAs: with the operands formed
-// by the issuing lane alone 107 clocks each, computed by the whole warp in converged code (uniform registers,
-// one 32-bit addition per operand) 85.  16 -> 16 channels at 128^3: 121 us streamed, 85, 69 us; 48 -> 16 (two
-// rows a tile): 302, 332, 252 us; 32 -> 32 at 128^3 of a 256^3 network: 245, 229, 191 us.
+// and the epilogue has warps of its own.  What bounds it then is the issue of the MMAs (47 clocks each when
+// nothing else holds them up): 107 clocks with the operands formed by the issuing lane alone, 85 with the whole
+// warp computing them in converged code, 58 with four warps issuing for a tile each.  16 -> 16 channels at 128^3:
+// 121 us streamed, then 85, 69, 56; 48 -> 16 (two rows a tile): 302, then 332, 252, 180; 32 -> 32 at 128^3 of a
+// 256^3 network: 245, then 229, 191, 135.
 // The MMAs are issued in the order of the streamed form, so the results are the same bits.
-// Warps 0-3: epilogue (warp % 4 selects the tensor memory lanes); warp 4: MMA; warps 5 ..: producers, one per row.
+// Warps 0-3: epilogue (warp % 4 selects the tensor memory lanes); the next `issuers` warps issue the MMAs of every
+// issuers-th tile into an accumulator of their own; then the producers, one warp per row of a unit.  A unit is free
+// when the three tiles that read it have committed (`empty` counts three; tiles at the ends of a run of planes
+// commit for the missing ones).
 template <int COUT, int R>
 struct TcRing {
   static constexpr int rows = R + 2, unit = rows * tc::kRowBytes;
-  static constexpr int threads = 32 * (5 + rows), ahead = 2;  // copy groups in flight per producer thread
-  static constexpr int wslice = 27 * COUT * 32, zbytes = R * COUT * 32, head = 256, max_units = 12;
+  static constexpr int issuers = 4;
+  static constexpr int threads = 32 * (4 + issuers + rows), ahead = 2;  // copy groups in flight per producer thread
+  static constexpr int wslice = 27 * COUT * 32, zbytes = R * COUT * 32, head = 384, max_units = 12;
   static constexpr int room = 227 * 1024;
   // units of the ring for nsl slices: all that fit (at most max_units); 0: fewer than three planes and `ahead` units
   static __host__ __device__ int units(int nsl) {
@@ -392,12 +397,13 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
   extern __shared__ __align__(1024) unsigned char sm[];
   uint64_t* full = reinterpret_cast<uint64_t*>(sm);  // max_units
   uint64_t* empty = full + P::max_units;             // max_units
-  uint64_t* acc_full = empty + P::max_units;         // 2
-  uint64_t* acc_empty = acc_full + 2;                // 2
-  uint64_t* done = acc_empty + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  constexpr int NB = P::issuers;
+  uint64_t* acc_full = empty + P::max_units;         // NB
+  uint64_t* acc_empty = acc_full + NB;               // NB
+  uint64_t* done = acc_empty + NB;                   // NB
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + NB);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  static_assert((2 * P::max_units + 5) * 8 + 8 <= P::head, "barriers fit");
+  static_assert((2 * P::max_units + 3 * NB) * 8 + 8 <= P::head, "barriers fit");
   const int nsl = (a.c0 + a.c1) / 16, NU = P::units(nsl);
   unsigned char* zb = sm + P::head;
   unsigned char* wres = zb + P::zbytes;
@@ -406,7 +412,7 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
   const int No = a.No, nseg = No / 128;
   const long ntiles = (long)nseg * (No / R) * No;
   const long t0 = ntiles * blockIdx.x / gridDim.x, t1 = ntiles * (blockIdx.x + 1) / gridDim.x;
-  constexpr int TCOLS = 2 * R * COUT;  // two tiles x R rows x COUT fp32 columns (a power of two)
+  constexpr int TCOLS = NB * R * COUT;  // NB tiles x R rows x COUT fp32 columns (a power of two)
   static_assert((TCOLS & (TCOLS - 1)) == 0 && TCOLS >= 32 && TCOLS <= 512, "tensor memory columns");
 
   if (warp == 4) {
@@ -418,13 +424,13 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
   if (tid == 0) {
     for (int q = 0; q < NU; ++q) {
       mbar_init(full + q, P::rows);
-      mbar_init(empty + q, 1);
+      mbar_init(empty + q, 3);
     }
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < NB; ++q) {
       mbar_init(acc_full + q, 1);
       mbar_init(acc_empty + q, 4);
+      mbar_init(done + q, 1);
     }
-    mbar_init(done, 1);
     *abort_flag = 0;
     mbar_fence_init();
   }
@@ -446,11 +452,13 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
     return (int)((t1 - t) < (long)(No - zs) ? (t1 - t) : (long)(No - zs));
   };
 
-  if (warp == 4) {
-    // ---------------- MMA issuer: the warp waits and computes the operands together, one lane issues ----------
+  if (warp >= 4 && warp < 4 + NB) {
+    // ---------------- MMA issuers: the warp waits and computes the operands together, one lane issues ----------
     constexpr uint32_t id1 = tc::idesc(128, COUT), id2 = tc::idesc(128, 2 * COUT), id3 = tc::idesc(128, 3 * COUT),
                        idz = tc::idesc(128, R * COUT);
+    const int me = warp - 4;
     const uint32_t leader = tc::elect();
+    const uint32_t d0 = tmem + (uint32_t)(me * R * COUT);
     const uint64_t da = tc::desc(smem_u32(unit0), tc::kRowVox * 16, 128);
     const uint32_t hi = (uint32_t)(da >> 32), a0 = (uint32_t)da;
     const uint32_t b0 = (uint32_t)tc::desc(smem_u32(wres), 3 * COUT * 16, 128);
@@ -463,7 +471,8 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
       int x0, y0, zs;
       const int n = run_of(t, x0, y0, zs);
       for (int j = 0; j < n && ok; ++j, ++i, ub += nsl) {
-        bool w = i < 2 || mbar_wait(acc_empty + (i & 1), (unsigned)(((i - 2) >> 1) & 1));
+        if (i % NB != me) continue;
+        bool w = i < NB || mbar_wait(acc_empty + me, (unsigned)((i / NB - 1) & 1));
         for (int sl = 0; sl < nsl && ok; ++sl) {
           unsigned slot[3];
 #pragma unroll
@@ -478,7 +487,7 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
           uint32_t ab[3];
 #pragma unroll
           for (int zz = 0; zz < 3; ++zz) ab[zz] = a0 + slot[zz] * ustep;
-          const uint32_t bb = b0 + (uint32_t)(sl * (P::wslice >> 4)), d0 = tmem + (uint32_t)((i & 1) * R * COUT);
+          const uint32_t bb = b0 + (uint32_t)(sl * (P::wslice >> 4));
           if (sl == 0) tc::mma_by(leader, d0, ab[0], z0, hi, idz, 0);  // D = 0
 #pragma unroll
           for (int yy = 0; yy < R + 2; ++yy)
@@ -493,12 +502,11 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
                            bb + (uint32_t)(((zz * 3 + dx) * (3 * COUT * 32) + dyi0 * COUT * 16) >> 4), hi,
                            nj == 3 ? id3 : (nj == 2 ? id2 : id1), 1);
               }
-          tc::commit_by(leader, empty + slot[0]);  // the lower plane is done with
-          if (j == n - 1) {                        // and at the end of a run the other two
-            tc::commit_by(leader, empty + slot[1]);
-            tc::commit_by(leader, empty + slot[2]);
-          }
-          if (sl == nsl - 1) tc::commit_by(leader, acc_full + (i & 1));
+          const int uses[3] = {j == 0 ? 3 : 1, 1 + (j == 0) + (j == n - 1), j == n - 1 ? 3 : 1};
+#pragma unroll
+          for (int zz = 0; zz < 3; ++zz)
+            for (int q = 0; q < uses[zz]; ++q) tc::commit_by(leader, empty + slot[zz]);
+          if (sl == nsl - 1) tc::commit_by(leader, acc_full + me);
           __syncwarp();
         }
       }
@@ -507,13 +515,13 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
     }
     if (!ok && lane == 0) fail();
     // every MMA issued has completed before the accumulator memory is released
-    tc::commit_by(leader, done);
+    tc::commit_by(leader, done + me);
     __syncwarp();
-    mbar_wait(done, 0);
-  } else if (warp >= 5) {
-    // ---------------- producers: warp 5 + r copies row r of each unit ----------------
-    const int r = warp - 5;
-    for (int q = tid - 160; q < nsl * 27 * COUT * 2; q += 32 * P::rows) {  // weights, part of the first group
+    mbar_wait(done + me, 0);
+  } else if (warp >= 4 + NB) {
+    // ---------------- producers: warp 4 + NB + r copies row r of each unit ----------------
+    const int r = warp - 4 - NB;
+    for (int q = tid - 32 * (4 + NB); q < nsl * 27 * COUT * 2; q += 32 * P::rows) {  // weights, part of the first group
       const int h = q & 1, co = (q >> 1) % COUT, r2 = (q >> 1) / COUT, t = r2 % 27, sl = r2 / 27;
       tc::cp16(wres + sl * P::wslice + wofs<COUT>(t, co, h),
                a.W + ((long)t * COUT + co) * (a.c0 + a.c1) + 16 * sl + 8 * h);
@@ -583,10 +591,10 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
       const int n = run_of(t, x0, y0, zs);
       const int x = x0 + 32 * warp + lane;
       for (int j = 0; j < n; ++j, ++i) {
-        ok = __all_sync(0xffffffffu, mbar_wait(acc_full + (i & 1), (unsigned)((i >> 1) & 1)));
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_full + i % NB, (unsigned)((i / NB) & 1)));
         if (!ok) break;
         tc::fence_after();
-        const uint32_t tb = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)((i & 1) * R * COUT);
+        const uint32_t tb = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)((i % NB) * R * COUT);
 #pragma unroll 1
         for (int j0 = 0; j0 < R; j0 += JB) {
           float v[JB * COUT];
@@ -616,7 +624,7 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
         }
         tc::fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(acc_empty + (i & 1));
+        if (lane == 0) mbar_arrive(acc_empty + i % NB);
         if (aborted()) ok = false;
       }
       t += n;
