@@ -50,6 +50,12 @@ constexpr int kArhs = FE_RING_A_RHS, kAdiv = FE_RING_A_DIV;
 // it again: carrying it cost the predictor 2 % in registers.
 template <typename T>
 constexpr bool kCarryZ = sizeof(T) == 8;
+// FP32 kernels whose issue slots bind evaluate both cells of a pair with one instruction (add2, mul2, fma2; the
+// same roundings).  Before and after, ms per step at 512^3: flux divergences (three classes) 2.01 -> 1.77,
+// predictor 2.44 -> 2.21, right-hand side 2.43 -> 2.40, energy faces 10.20 -> 10.07; two-fluid at 150^3: predictor
+// 236 -> 205 us, corrector 266 -> 252.  Not the assembly (3.65 -> 3.67), the dust update (0.48 -> 0.59 at 256^3,
+// its 170 registers leave two blocks per SM; held to three blocks 0.48), Du/Dt and the per-cell energy pass
+// (equal): those wait for memory, and aligned register pairs cost them registers.
 
 template <typename T>
 __device__ __forceinline__ T* Fr(const BoxDev& B, int slot) {
@@ -198,7 +204,8 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_corr(const BoxDev* boxes
 // Laplacian as (28 S1 - 162 u - S2) / 24 (S1, S2: the six neighbours at distance 1 and 2), Gc unscaled;
 // cl = mu / (24 h^2), cd = mu / (48 h), cc = 1 / (16 h).
 // zf (FP64): 16 I4 of u_m at the lower z faces, taken over from the plane below (formed on a tile's first).
-template <typename T, bool WIDE, typename Plan>
+// PAIR: FP32, both cells per instruction.
+template <typename T, bool PAIR, bool WIDE, typename Plan>
 __device__ __forceinline__ void ring_L(const Plan& R, int k, bool first, const RGeom<T, WIDE>& G, const T (&php)[3][2],
                                        const T (&phm)[3][2], T cl, T cd, T cc, T (&zf)[3][2], T (&L)[3][2],
                                        T (&visc)[3][2]) {
@@ -209,6 +216,30 @@ __device__ __forceinline__ void ring_L(const Plan& R, int k, bool first, const R
 #pragma unroll
       for (int r = 0; r < 2; ++r) zf[m][r] = i4m16(lz, pc<T>(R.zq[m][2], r), r);
     }
+  }
+  if constexpr (PAIR) {
+    float2 np[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) np[d] = mul2(two(phm[d]), two(-1.f));
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      float2 cv, lap;
+      {
+        const Line2<T> l[3] = {ring_line(R, m, k, G, 0), ring_line(R, m, k, G, 1), ring_line(R, m, k, G, 2)};
+        const float2 u = two(R.zq[m][2]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {  // cv: -conv
+          cv = d == 0 ? mul2(two(php[0]), i4p16n(l[0], u)) : fma2(two(php[d]), i4p16n(l[d], u), cv);
+          cv = fma2(np[d], i4m16n(l[d], u), cv);
+        }
+        lap = lap24n(l[0], l[1], l[2], u);
+      }
+      const float2 v = fma2(two(-cl), lap, mul2(two(-cd), gc16n(ring_line(R, 3, k, G, m))));
+      const float2 o = fma2(two(cc), cv, v);
+      visc[m][0] = v.x, visc[m][1] = v.y;
+      L[m][0] = o.x, L[m][1] = o.y;
+    }
+    return;
   }
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
@@ -282,7 +313,7 @@ __global__ void __launch_bounds__(RNT, sizeof(T) == 4 ? FE_RING_MINB_PRED : FE_R
     T php[3][2], phm[3][2];
     R.faces2(0, k, G, php, phm);
     T L[3][2], visc[3][2];
-    ring_L(R, k, i == 0, G, php, phm, cl, cd, cc, zf, L, visc);
+    ring_L<T, sizeof(T) == 4>(R, k, i == 0, G, php, phm, cl, cd, cc, zf, L, visc);
     T gp[3][2];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
@@ -376,7 +407,7 @@ __global__ void __launch_bounds__(RNT, sizeof(T) == 4 && TW ? 3 : FE_RING_MINB) 
     T php[3][2], phm[3][2];
     R.faces2(0, k, G, php, phm);
     T L[3][2], visc[3][2];
-    ring_L(R, k, i == 0, G, php, phm, cl, cd, cc, zf, L, visc);
+    ring_L<T, false>(R, k, i == 0, G, php, phm, cl, cd, cc, zf, L, visc);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const T rc = pc<T>(crho, r);
@@ -464,7 +495,8 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_accel(const BoxDev* boxe
 // and a_d along d, and of Y_j along d, each read once; 16 I4 evaluated unscaled, the factors folded.
 // zf (FP64): 16 x the class fluxes of the lower z faces, taken over from the plane below (formed on a tile's
 // first).
-template <typename T, int ND, bool WIDE, typename Plan>
+// PAIR: FP32, both cells per instruction.
+template <typename T, int ND, bool PAIR, bool WIDE, typename Plan>
 __device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, bool first, const RGeom<T, WIDE>& G,
                                                    const T (&taup)[ND], T (&zf)[ND][2], T (&fl)[ND][2]) {
   T php[3][2], phm[3][2];
@@ -480,6 +512,33 @@ __device__ __forceinline__ void ring_particle_flux(const Plan& R, int k, bool fi
         zf[j][r] = fma(-taup[j] * T(1.0 / 256.0), i4m16(lr, pc<T>(rc, r), r) * i4m16(la, pc<T>(R.zq[3][2], r), r),
                        phm[2][r]) * i4m16(ly, pc<T>(R.zq[4 + j][2], r), r);
     }
+  }
+  if constexpr (PAIR) {
+    float2 f2[ND];
+#pragma unroll
+    for (int j = 0; j < ND; ++j) f2[j] = two(0.f);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      float2 rap, ram;
+      {
+        const Line2<T> lr = ring_line(R, 0, k, G, d), la = ring_line(R, 1 + d, k, G, d);
+        const float2 r = two(rc), a = two(R.zq[1 + d][2]);
+        rap = mul2(i4p16n(lr, r), i4p16n(la, a));
+        ram = mul2(i4m16n(lr, r), i4m16n(la, a));
+      }
+#pragma unroll
+      for (int j = 0; j < ND; ++j) {
+        const float2 tq = two(-taup[j] * (1.f / 256.f));
+        const Line2<T> ly = ring_line(R, 4 + j, k, G, d);
+        const float2 y = two(R.zq[4 + j][2]);
+        const float2 fp = mul2(fma2(tq, rap, two(php[d])), i4p16n(ly, y));  // -16 x the upper face's flux
+        f2[j] = fma2(fma2(tq, ram, two(phm[d])), i4m16n(ly, y), f2[j]);
+        f2[j] = fma2(fp, two(-1.f), f2[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < ND; ++j) fl[j][0] = f2[j].x * 0.0625f, fl[j][1] = f2[j].y * 0.0625f;
+    return;
   }
 #pragma unroll
   for (int j = 0; j < ND; ++j) fl[j][0] = fl[j][1] = T(0);
@@ -547,7 +606,7 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fluxn(const BoxDev* boxe
     if (!G.active) continue;
     const int c = G.col + G.plane(k);
     T fl[ND][2];
-    ring_particle_flux<T, ND>(R, k, i == 0, G, taup, zf, fl);
+    ring_particle_flux<T, ND, sizeof(T) == 4>(R, k, i == 0, G, taup, zf, fl);
 #pragma unroll
     for (int j = 0; j < ND; ++j) stp(fyn[j] + c, fl[j][0] * ih, fl[j][1] * ih);
   }
@@ -610,7 +669,7 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_dust(const BoxDev* boxes
     const P2<T> crn = R.cen(0, k, tid);
     T oy[ND][2], op[2], oe[2], ot[2];
     T flx[ND][2];
-    ring_particle_flux<T, ND>(R, k, i == 0, G, taup, zf, flx);
+    ring_particle_flux<T, ND, false>(R, k, i == 0, G, taup, zf, flx);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const T rk = pc<T>(R.zq[0][2], r);
@@ -787,6 +846,7 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fe_face(const BoxDev* bo
       const P2<T> hc = R.zq[0][2], tc = R.zq[1][2];
       const P2<T> ph = R.cen(d, k, tid);
       T work[2] = {T(0), T(0)}, of[2];
+      float2 nwork = make_float2(0.f, 0.f);  // FP32: -work of both cells
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
         const Line2<T> lu = ring_line(R, 2 + m, k, G, d);
@@ -807,6 +867,19 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fe_face(const BoxDev* bo
             gv[0][q] = v.x, gv[1][q] = v.y;
           }
         }
+        if constexpr (sizeof(T) == 4) {  // both cells at once, the same roundings
+          const float2 u = two(uc);
+          const float2 ig = fma2(two(-9.f), add2(make_float2(gv[0][1], gv[1][1]), make_float2(gv[0][2], gv[1][2])),
+                                 add2(make_float2(gv[0][0], gv[1][0]), make_float2(gv[0][3], gv[1][3])));
+          const float2 g4u = fma2(two(-27.f), sub2(two(lu.p1), u), sub2(two(lu.p2), two(lu.m1)));
+          float2 tau = mul2(fma2(g4u, two(-1.f / 24.f), mul2(ig, two(-0.0625f))), two(ih));
+          if (d == m) {
+            const Line2<T> ld = ring_line(R, 5, k, G, d);
+            tau = fma2(two(2.f / 3.f * 0.0625f), i4p16n(ld, two(R.zq[5][2])), tau);
+          }
+          nwork = fma2(mul2(two(mu * 0.0625f), tau), i4p16n(lu, u), nwork);
+          continue;
+        }
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           const T u = pc<T>(uc, r);
@@ -819,6 +892,13 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_fe_face(const BoxDev* bo
           }
           work[r] += (mu * tau) * (i4p16(lu, u, r) * T(0.0625));
         }
+      }
+      if constexpr (sizeof(T) == 4) {
+        const float2 g4t = fma2(two(-27.f), sub2(two(lt.p1), two(tc)), sub2(two(lt.p2), two(lt.m1)));
+        const float2 o = fma2(two(-kappa), mul2(mul2(g4t, two(-1.f / 24.f)), two(ih)),
+                              fma2(mul2(two(ph), two(-0.0625f)), i4p16n(lh, two(hc)), nwork));
+        stp(Fr<T>(B, W_FEF0 + d) + c, o.x, o.y);
+        continue;
       }
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
@@ -910,6 +990,15 @@ __global__ void __launch_bounds__(RNT, FE_RING_MINB) kr_rhs(const BoxDev* boxes,
       const Line2<T> lr = ring_line(R, 0, k, G, d), lh = ring_line(R, 1 + d, k, G, d);
       const Line2<T> lp = ring_line1(R, 4, k, G, d);
       const P2<T> hc = R.zq[1 + d][2];
+      if constexpr (sizeof(T) == 4) {  // both cells at once, the same roundings
+        const float2 r2 = two(rpc), h2 = two(hc), p2 = two(pcc), nd = two(-dih);
+        const float2 fp = fma2(nd, sub2(two(lp.p1), p2), mul2(mul2(i4p16n(lr, r2), i4p16n(lh, h2)), two(1.f / 256.f)));
+        const float2 fm = fma2(nd, sub2(p2, two(lp.m1)), mul2(mul2(i4m16n(lr, r2), i4m16n(lh, h2)), two(1.f / 256.f)));
+        const float2 ds = add2(two(dsum), sub2(fp, fm));
+        ops[d][0] = fp.x, ops[d][1] = fp.y;
+        dsum[0] = ds.x, dsum[1] = ds.y;
+        continue;
+      }
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         const T rc = pc<T>(rpc, r), h = pc<T>(hc, r), p = pc<T>(pcc, r);

@@ -186,6 +186,34 @@ __device__ __forceinline__ void tfr_div(const RP& R, const GT& G, int k, T ih, T
   T php[3][2], phm[3][2];
   R.faces2(0, k, G, php, phm);
   T dg[3][2] = {{T(0), T(0)}, {T(0), T(0)}, {T(0), T(0)}}, df[2] = {T(0), T(0)};
+  if constexpr (sizeof(T) == 4) {  // both cells at once, the same roundings
+    float2 f2 = two(0.f), g2[3] = {two(0.f), two(0.f), two(0.f)};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      float2 Fp, Fm;  // Fp negated
+      {
+        const Line2<T> lv = ring_line(R, 5 + d, k, G, d), lu = ring_line(R, 1 + d, k, G, d);
+        const float2 vc = two(R.zq[5 + d][2]), uc = two(R.zq[1 + d][2]);
+        const float2 sp = sub2(i4p16n(lv, vc), i4p16n(lu, uc)), sm = sub2(i4m16n(lv, vc), i4m16n(lu, uc));
+        const Line2<T> lr = ring_line(R, 0, k, G, d), ly = ring_line(R, 4, k, G, d);
+        const float2 rc = two(R.zq[0][2]), yc = two(R.zq[4][2]);
+        Fp = mul2(fma2(mul2(i4p16n(lr, rc), two(1.f / 256.f)), sp, two(php[d])), i4p16n(ly, yc));
+        Fm = mul2(fma2(mul2(i4m16n(lr, rc), two(1.f / 256.f)), sm, two(phm[d])), i4m16n(ly, yc));
+        f2 = add2(f2, sub2(Fm, Fp));
+        Fm = mul2(Fm, two(-1.f));
+      }
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        const Line2<T> lv = ring_line(R, 5 + m, k, G, d);
+        const float2 vc = two(R.zq[5 + m][2]);
+        g2[m] = add2(g2[m], fma2(Fp, i4p16n(lv, vc), mul2(Fm, i4m16n(lv, vc))));
+      }
+    }
+    DF[0] = f2.x * (ih * 0.0625f), DF[1] = f2.y * (ih * 0.0625f);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) DG[m][0] = g2[m].x * (ih * (1.f / 256.f)), DG[m][1] = g2[m].y * (ih * (1.f / 256.f));
+    return;
+  }
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const Line2<T> lr = ring_line(R, 0, k, G, d), ly = ring_line(R, 4, k, G, d), lu = ring_line(R, 1 + d, k, G, d);

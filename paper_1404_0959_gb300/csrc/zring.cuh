@@ -413,4 +413,30 @@ __device__ __forceinline__ T gc16(const Line2<T>& L, int r) {
   return fma(T(10), L.p1[r] - L.m1[r], -(L.p2[r] - L.m2[r]));
 }
 
+// Both cells of a pair in one instruction (FP32: add, mul and fma on two lanes of a 64-bit register pair, each
+// rounded as its scalar form; subtraction is an exact product with -1).
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 two(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 two(const float (&a)[2]) { return make_float2(a[0], a[1]); }
+__device__ __forceinline__ float2 two(const P2<float>& a) { return make_float2(a.x, a.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, two(-1.f), a); }
+// -16 h Gc, and the negative of 28 S1 - 162 u - S2 (see gc16 and the compact Laplacian), of both cells
+__device__ __forceinline__ float2 gc16n(const Line2<float>& L) {
+  return fma2(two(-10.f), sub2(two(L.p1), two(L.m1)), sub2(two(L.p2), two(L.m2)));
+}
+__device__ __forceinline__ float2 lap24n(const Line2<float>& x, const Line2<float>& y, const Line2<float>& z, float2 u) {
+  const float2 s1 = add2(add2(add2(two(x.m1), two(x.p1)), add2(two(y.m1), two(y.p1))), add2(two(z.m1), two(z.p1)));
+  const float2 s2 = add2(add2(add2(two(x.m2), two(x.p2)), add2(two(y.m2), two(y.p2))), add2(two(z.m2), two(z.p2)));
+  return fma2(two(-28.f), s1, fma2(two(162.f), u, s2));
+}
+// -16 I4 at the +1/2 and -1/2 faces of both cells (negated: no operand changes sign)
+__device__ __forceinline__ float2 i4p16n(const Line2<float>& L, float2 c) {
+  return fma2(two(-9.f), add2(c, two(L.p1)), add2(two(L.m1), two(L.p2)));
+}
+__device__ __forceinline__ float2 i4m16n(const Line2<float>& L, float2 c) {
+  return fma2(two(-9.f), add2(two(L.m1), c), add2(two(L.m2), two(L.p1)));
+}
+
 }  // namespace fe
