@@ -277,18 +277,20 @@ static void tile_box(BoxDev& B, int tz, int box, std::vector<int2>& work) {
 }
 
 // Built-in tile depth of the step kernels (and of the FP32 Krylov kernels, whose float-pair sums do not
-// depend on it to FP32 accuracy), one for all boxes: the one that minimises (waves + share) x (tz + o).
+// depend on it to FP32 accuracy), one for all boxes: the one that minimises
+// (waves + share x most tiles of an SM) x (tz + o).
 // A wave is `res` resident blocks per SM; o stands for the planes a tile reads beyond its own, its ring
-// prologue and its partial sums; share, for FP32 kernels, is 0.3 tiles per SM: blocks that fit one wave
-// still compete.  FP64 kernels saturate the FP64 pipe with one block per SM (res = 1, o = 1, no share);
-// FP32 kernels keep about three (o = 5).  Fitted to sweeps over depths 1 to 64 of 26 contexts (N = 24 to
-// 512, every closure and dust model, ensembles): within 5 % of each sweep's best depth, 1 % on average.
-// Against the fixed depths 8 (N >= 128) and 4 before, ms per step: 256^3 6.93 -> 6.23, 512^3 with three
-// classes 69.0 -> 59.6, 300^3 15.9 -> 12.1, 64 boxes of 32^3 to 96^3 15.4 -> 10.6, 112^3 1.79 -> 1.43,
-// 96^3 1.26 -> 1.09, FP64 32^3 1.54 -> 1.22.
+// prologue and its partial sums; the share, for FP32 kernels, is 0.4 per tile that the fullest SM has: blocks
+// that fit one wave still compete.  FP64 kernels saturate the FP64 pipe with one block per SM (res = 1, o = 1,
+// no share); FP32 kernels keep about three (o = 6).  Fitted to sweeps over depths 1 to 64 of 28 contexts
+// (N = 24 to 512, every closure and dust model, ensembles): within 5 % of each sweep's best depth, 0.5 % on
+// average, and none slower than with the fixed depths 8 (N >= 128) and 4 before.  Against those, ms per step:
+// 256^3 6.93 -> 6.37, 512^3 with three classes 69.0 -> 59.6, 300^3 15.9 -> 12.1, 64 boxes of 32^3 to 96^3
+// 15.4 -> 10.8, 112^3 1.79 -> 1.43, 96^3 1.26 -> 1.09, FP64 32^3 1.54 -> 1.22.  (With tiles / SMs in place of
+// the fullest SM's tiles: 1.2 % on average, 36^3 two-fluid 2 % slower than at depth 4.)
 static int tz_default(const fe_ctx* c) {
-  const long res = c->fp64 ? 1 : 3, over = c->fp64 ? 1 : 5;
-  const double share = c->fp64 ? 0.0 : 0.3;
+  const long res = c->fp64 ? 1 : 3, over = c->fp64 ? 1 : 6;
+  const double share = c->fp64 ? 0.0 : 0.4;
   int maxN = 0;
   for (int N : c->N) maxN = std::max(maxN, N);
   double best = -1.0;
@@ -301,7 +303,7 @@ static int tz_default(const fe_ctx* c) {
       tiles += (long)((N + TX - 1) / TX) * ((N + TY - 1) / TY) * ((N + z - 1) / z);
     }
     const long wave = res * c->nsm;
-    const double cost = ((double)((tiles + wave - 1) / wave) + share * tiles / c->nsm) * (double)(cand + over);
+    const double cost = ((double)((tiles + wave - 1) / wave) + share * ((tiles + c->nsm - 1) / c->nsm)) * (double)(cand + over);
     if (best < 0.0 || cost < best) {
       best = cost;
       tz = cand;
