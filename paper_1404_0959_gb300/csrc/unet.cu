@@ -591,6 +591,12 @@ static const int kDims[kNL][6] = {{16, 16, 2, 16, 0, 1},  {16, 16, 16, 16, 0, 1}
                                   {96, 32, 96, 32, 1, 1}, {48, 16, 48, 16, 0, 1}, {16, 16, 16, 1, 0, 1}};
 static const char* kNames[kNL] = {"e1a", "e1b", "d1", "e2", "d2", "e3", "u2", "u1", "out"};
 
+long unet_param_count() {
+  long n = 0;
+  for (int l = 0; l < kNL; ++l) n += 27L * kDims[l][2] * kDims[l][3] + kDims[l][3];
+  return n;
+}
+
 struct UNet {
   int N = 0;  // finest grid
   Layer L[kNL];
@@ -599,6 +605,7 @@ struct UNet {
   bf16 *in16 = nullptr, *e1a = nullptr, *e1b = nullptr, *d1 = nullptr, *e2 = nullptr, *d2 = nullptr,
        *e3 = nullptr, *u2 = nullptr, *u1 = nullptr;
   float* out32 = nullptr;  // [N^3] channel 0
+  float* xfer = nullptr;   // parameters or gradients in the host's order, on their way out
   // training buffers
   float *g0 = nullptr, *g1 = nullptr, *g2 = nullptr, *gsk0 = nullptr, *gsk1 = nullptr, *dy8 = nullptr;
   bf16* dpre = nullptr;
@@ -654,7 +661,8 @@ static int unet_alloc(UNet& U, int N, bool training) {
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && nsm > 0)
       U.nsm = nsm;
   }
-  if (!U.in16 || !U.e1a || !U.e1b || !U.d1 || !U.e2 || !U.d2 || !U.e3 || !U.u2 || !U.u1 || !U.out32 || !U.err)
+  U.xfer = (float*)A(unet_param_count() * 4);
+  if (!U.xfer || !U.in16 || !U.e1a || !U.e1b || !U.d1 || !U.e2 || !U.d2 || !U.e3 || !U.u2 || !U.u1 || !U.out32 || !U.err)
     return FE_ERR_OOM;
   size_t wtotal = 0;
   for (int l = 0; l < kNL; ++l) {
@@ -1105,12 +1113,6 @@ void unet_destroy(UNet* U) {
   delete U;
 }
 
-long unet_param_count() {
-  long n = 0;
-  for (int l = 0; l < kNL; ++l) n += 27L * kDims[l][2] * kDims[l][3] + kDims[l][3];
-  return n;
-}
-
 // host layout per layer: W[27][cin_real][cout_real] then b[cout_real]
 int unet_set_weights(UNet* U, const float* host, cudaStream_t st) {
   long off = 0;
@@ -1139,24 +1141,30 @@ int unet_set_weights(UNet* U, const float* host, cudaStream_t st) {
   return cudaGetLastError() == cudaSuccess ? FE_OK : FE_ERR_CUDA;
 }
 
-// which = 0: weights and biases, 1: their gradients
+// One layer's parameters (or gradients) from [27][cout][cin] and [cout] to the host's order, without the padding.
+__global__ void k_export(const float* __restrict__ w, const float* __restrict__ b, int cin, int cout, int cin_real,
+                         int cout_real, float* __restrict__ out) {
+  const int nw = 27 * cin_real * cout_real, n = nw + cout_real;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+    const int co = q % cout_real, r = q / cout_real, ci = r % cin_real, t = r / cin_real;
+    out[q] = q < nw ? w[((long)t * cout + co) * cin + ci] : b[q - nw];
+  }
+}
+
+// which = 0: weights and biases, 1: their gradients.  Put into the host's order on the device and copied at once
+// (a copy and a wait per layer array and the reordering on the host took 0.5 ms of the 64^3 training step's 2.4 ms
+// for each of the two).
 int unet_get_weights(UNet* U, float* host, int which, cudaStream_t st) {
   long off = 0;
   for (int l = 0; l < kNL; ++l) {
     Layer& y = U->L[l];
-    const long nw = 27L * y.cin * y.cout;
-    std::vector<float> w(nw), b(y.cout);
-    cudaMemcpyAsync(w.data(), which ? y.gw : y.w, nw * 4, cudaMemcpyDeviceToHost, st);
-    cudaMemcpyAsync(b.data(), which ? y.gb : y.b, y.cout * 4, cudaMemcpyDeviceToHost, st);
-    cudaStreamSynchronize(st);
-    for (int t = 0; t < 27; ++t)
-      for (int ci = 0; ci < y.cin_real; ++ci)
-        for (int co = 0; co < y.cout_real; ++co)
-          host[off + ((long)t * y.cin_real + ci) * y.cout_real + co] = w[((long)t * y.cout + co) * y.cin + ci];
-    off += 27L * y.cin_real * y.cout_real;
-    for (int co = 0; co < y.cout_real; ++co) host[off + co] = b[co];
-    off += y.cout_real;
+    const long n = 27L * y.cin_real * y.cout_real + y.cout_real;
+    k_export<<<ew(n), 256, 0, st>>>(which ? y.gw : y.w, which ? y.gb : y.b, y.cin, y.cout, y.cin_real, y.cout_real,
+                                    U->xfer + off);
+    off += n;
   }
+  cudaMemcpyAsync(host, U->xfer, off * 4, cudaMemcpyDeviceToHost, st);
+  cudaStreamSynchronize(st);
   return cudaGetLastError() == cudaSuccess ? FE_OK : FE_ERR_CUDA;
 }
 

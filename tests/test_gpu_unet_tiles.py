@@ -68,3 +68,14 @@ def test_weight_gradients_on_staged_tiles(fe, N):  # noqa: F811
     of odd size (28: 14 and 7; 44: 22 and 11), or leaves remainders along every axis; accumulation in FP32 of the
     same BF16 products, so the bars of the gradients above hold."""
     test_gradients_on_ragged_tiles(fe, N)
+
+
+def test_parameters_come_back_as_loaded(fe):  # noqa: F811
+    """The parameters' way out (padding of the first and last layers left behind, biases between the weights) returns
+    what was loaded, bit for bit; before a training step the gradients are zero."""
+    s, _, P, _ = problem(fe, 8)
+    w = np.random.default_rng(3).standard_normal(fe.fe_preconditioner_size()).astype(np.float32)
+    fe.fe_load_preconditioner(s.ctx, w)
+    assert np.array_equal(fe.fe_get_preconditioner(s.ctx), w)
+    assert not fe.fe_get_preconditioner(s.ctx, gradients=True).any()
+    s.close()
