@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "fe_internal.cuh"
+#include "widen.cuh"
 
 namespace fe {
 
@@ -484,8 +485,8 @@ __device__ __forceinline__ void pack_voxel(bf16* o, float c0, float c1) {
 template <typename T>
 __global__ void k_pack_input(const T* r, const T* dinv, long n, double a, double w, bf16* in16) {
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
-    const double dq = (double)dinv[q];
-    pack_voxel(in16 + q * 16, (float)((double)r[q] * dq * a), (float)(dq * w));
+    const double dq = widen(dinv[q]);
+    pack_voxel(in16 + q * 16, narrow(widen(r[q]) * dq * a), narrow(dq * w));
   }
 }
 
@@ -493,7 +494,7 @@ __global__ void k_pack_input(const T* r, const T* dinv, long n, double a, double
 template <typename T>
 __global__ void k_direction(const T* r, const T* dinv, const float* y, double scale, long n, float* z) {
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x)
-    z[q] = (float)((double)r[q] * (double)dinv[q] + scale * (double)y[q]);
+    z[q] = narrow(widen(r[q]) * widen(dinv[q]) + scale * widen(y[q]));
 }
 
 // training target t = (e - r dinv) * inv_scale into tgt; block partial sums of t^2
@@ -1051,17 +1052,27 @@ namespace fe {
 
 // Network input for the current residual of a solve: rms(r)^2 = rr / n with
 // rr read from the box scalar rr_slot, dt from SC_KDT (the solve's operator);
-// the output scale rms(r) d0 of the direction goes to SC_NSCALE.
+// the output scale rms(r) d0 of the direction goes to SC_NSCALE.  The scales, five FP64 divisions and a root, are
+// formed by one thread of a block, and the fields converted off the FP64 pipe (per thread and by the conversion
+// instruction they bound the kernel: 53 us at 128^3, 40 now).
 template <typename T>
-__global__ void k_pack_fcg(const T* r, const T* dinv, long n, double* sc, int rr_slot, double ih, bf16* in16) {
-  const double rr = sc[rr_slot], dt = sc[SC_KDT];
-  const double c3 = 3.0 * dt * ih * ih, d0 = 1.0 / (1.0 / dt + c3);
-  const double rms = rr > 0.0 ? sqrt(rr / (double)n) : 0.0;
-  const double a = rms > 0.0 ? 1.0 / (rms * d0) : 0.0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) sc[SC_NSCALE] = rms * d0;
+__global__ void __launch_bounds__(256) k_pack_fcg(const T* __restrict__ r, const T* __restrict__ dinv, long n, double* sc,
+                                                  int rr_slot, double ih, bf16* __restrict__ in16) {
+  __shared__ double sa, sc3;
+  if (threadIdx.x == 0) {
+    const double rr = sc[rr_slot], dt = sc[SC_KDT];
+    const double c3 = 3.0 * dt * ih * ih, d0 = 1.0 / (1.0 / dt + c3);
+    const double rms = rr > 0.0 ? sqrt(rr / (double)n) : 0.0;
+    sa = rms > 0.0 ? 1.0 / (rms * d0) : 0.0;
+    sc3 = c3;
+    if (blockIdx.x == 0) sc[SC_NSCALE] = rms * d0;
+  }
+  __syncthreads();
+  const double a = sa, c3 = sc3;
+#pragma unroll 4
   for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) {
-    const double dq = (double)dinv[q];
-    pack_voxel(in16 + q * 16, (float)((double)r[q] * dq * a), (float)(dq * c3));
+    const double dq = widen(dinv[q]);
+    pack_voxel(in16 + q * 16, narrow(widen(r[q]) * dq * a), narrow(dq * c3));
   }
 }
 
@@ -1173,7 +1184,8 @@ int unet_get_weights(UNet* U, float* host, int which, cudaStream_t st) {
 template <typename T>
 void unet_apply_sc(UNet* U, const T* r, const T* dinv, double* sc, int rr_slot, double ih, cudaStream_t st) {
   const long n = cube(U->N);
-  k_pack_fcg<T><<<ew(n), 256, 0, st>>>(r, dinv, n, sc, rr_slot, ih, U->in16);
+  const int blocks = ew(n) < 4 * U->nsm ? ew(n) : 4 * U->nsm;
+  k_pack_fcg<T><<<blocks, 256, 0, st>>>(r, dinv, n, sc, rr_slot, ih, U->in16);
   unet_forward(*U, st);
 }
 
