@@ -43,8 +43,10 @@ def alg_words(kernel, nd, mixed=False, poly=False):
         return {"cg_dirmatvec": 7, "cg_rupdate": 6, "cg_start": 4, "rhs": 12, "refine": 10}[kernel]
     table = {
         "dt": 3, "div": 4, "pred": 21, "fluxn": 7 + 2 * nd, "asm": 18, "rhs": 13 if mixed else 11,
-        "cg_init": 5, "cg_matvec": 3, "cg_update": 7, "cg_dir": 4,
-        "cg_dirmatvec": 8, "cg_rupdate": 4, "cg_xfinal": 3, "corr": 19 if mixed else 21, "accel": 9,
+        # FP64: the residual update stores D^{-1} r and the direction reads it in place of r and D^{-1}
+        "cg_init": 5 if mixed else 6, "cg_matvec": 3, "cg_update": 7, "cg_dir": 4,
+        "cg_dirmatvec": 8 if mixed else 7, "cg_rupdate": 4 if mixed else 5, "cg_xfinal": 3,
+        "solve": 4,  # a whole FP64 solve on chip: b, psi, D^{-1} read, x written "corr": 19 if mixed else 21, "accel": 9,
         "dust": 8 + 4 * nd + 2,  # last corrector adds u reads and p write; averaged over 2 correctors
         "bicg_p": 4, "bicg_v": 4, "bicg_s": 3, "bicg_t": 3, "bicg_x": 8, "true_res": 3,
         # refinement (field word = 4 bytes; x64 counts as two words)
@@ -326,9 +328,8 @@ def time_path(fe, box, cfg, precision, solver, args, stream, learned_every=0, we
 
 def time_les(fe, box, cfg, args, stream, m=2):
     """CUDA-event time of the a-priori LES analysis (fe_les_apriori) on the
-    workload's spectral state in FP32; roofline from its 74 algorithmic words
-    per cell (x pass 4 read + 10 written, y and z passes 10 + 10 each, Favre
-    velocity 4 + 3, statistics 13 read)."""
+    workload's spectral state in FP32; roofline from its 24 algorithmic words
+    per cell (filter pass 4 read + 10 written, statistics 10 read)."""
     import torch
     N = box["N"]
     s = fe.Solver([box], precision=fe.FE_FP32_MIXED, closure=cfg["closure"], p_tol=cfg["p_tol"],
@@ -347,8 +348,8 @@ def time_les(fe, box, cfg, args, stream, m=2):
     s.close()
     ms = ev0.elapsed_time(ev1) / K
     hbm, kind = peaks()
-    gbs = 74 * 4 * float(N) ** 3 / (ms / 1e3) / 1e9
-    return {"N": N, "m": m, "ms_per_call": ms, "alg_bytes": 74 * 4 * N ** 3, "achieved_gbs": gbs, "peak": hbm,
+    gbs = 24 * 4 * float(N) ** 3 / (ms / 1e3) / 1e9
+    return {"N": N, "m": m, "ms_per_call": ms, "alg_bytes": 24 * 4 * N ** 3, "achieved_gbs": gbs, "peak": hbm,
             "frac": gbs / hbm, "note": "includes the host read of the block partial sums", "stats": st}
 
 
