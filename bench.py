@@ -46,7 +46,8 @@ def alg_words(kernel, nd, mixed=False, poly=False):
         # FP64: the residual update stores D^{-1} r and the direction reads it in place of r and D^{-1}
         "cg_init": 5 if mixed else 6, "cg_matvec": 3, "cg_update": 7, "cg_dir": 4,
         "cg_dirmatvec": 8 if mixed else 7, "cg_rupdate": 4 if mixed else 5, "cg_xfinal": 3,
-        "solve": 4,  # a whole FP64 solve on chip: b, psi, D^{-1} read, x written "corr": 19 if mixed else 21, "accel": 9,
+        # a whole FP64 solve on chip: b, psi, D^{-1} read, x written
+        "solve": 4, "corr": 19 if mixed else 21, "accel": 9,
         "dust": 8 + 4 * nd + 2,  # last corrector adds u reads and p write; averaged over 2 correctors
         "bicg_p": 4, "bicg_v": 4, "bicg_s": 3, "bicg_t": 3, "bicg_x": 8, "true_res": 3,
         # refinement (field word = 4 bytes; x64 counts as two words)
