@@ -375,6 +375,13 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_conv_tc(TcConvArgs a) {
 // issuers-th tile into an accumulator of their own; then the producers, one warp per row of a unit.  A unit is free
 // when the three tiles that read it have committed (`empty` counts three; tiles at the ends of a run of planes
 // commit for the missing ones).
+// A wait for a unit tells its fill from the one before by the parity of the slot's turn, so an issuer may wait for
+// unit u only once it has seen some unit >= u - NU arrive: units are published in order, so the slot's earlier
+// fills are then over, and the next one needs this tile's commit.  From unit to unit of a tile, and from an
+// issuer's tile to its next, that holds (at most 4 nsl units further, 2 nsl more where a run of planes ends
+// between, against 3 nsl - 1 seen and NU >= 3 nsl + 2).  An issuer's first tile can begin beyond the first NU units, where the block's first run is
+// short (which runs a block gets follows from the number of blocks, that is of SMs): it waits for `primed` before,
+// which the producers complete once, with unit NU - 1.
 template <int COUT, int R>
 struct TcRing {
   static constexpr int rows = R + 2, unit = rows * tc::kRowBytes;
@@ -401,9 +408,10 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
   uint64_t* acc_full = empty + P::max_units;         // NB
   uint64_t* acc_empty = acc_full + NB;               // NB
   uint64_t* done = acc_empty + NB;                   // NB
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + NB);
+  uint64_t* primed = done + NB;                      // 1
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(primed + 1);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  static_assert((2 * P::max_units + 3 * NB) * 8 + 8 <= P::head, "barriers fit");
+  static_assert((2 * P::max_units + 3 * NB + 1) * 8 + 8 <= P::head, "barriers fit");
   const int nsl = (a.c0 + a.c1) / 16, NU = P::units(nsl);
   unsigned char* zb = sm + P::head;
   unsigned char* wres = zb + P::zbytes;
@@ -431,6 +439,7 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
       mbar_init(acc_empty + q, 4);
       mbar_init(done + q, 1);
     }
+    mbar_init(primed, P::rows);
     *abort_flag = 0;
     mbar_fence_init();
   }
@@ -472,7 +481,7 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
       const int n = run_of(t, x0, y0, zs);
       for (int j = 0; j < n && ok; ++j, ++i, ub += nsl) {
         if (i % NB != me) continue;
-        bool w = i < NB || mbar_wait(acc_empty + me, (unsigned)((i / NB - 1) & 1));
+        bool w = i >= NB ? mbar_wait(acc_empty + me, (unsigned)((i / NB - 1) & 1)) : (int)ub < NU || mbar_wait(primed, 0);
         for (int sl = 0; sl < nsl && ok; ++sl) {
           unsigned slot[3];
 #pragma unroll
@@ -533,6 +542,7 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
       tc::fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(full + slotp);
+      if (lane == 0 && vp == (unsigned)NU - 1) mbar_arrive(primed);
       ++vp;
       if (++slotp == (unsigned)NU) slotp = 0;
     };
