@@ -528,49 +528,33 @@ __global__ void __launch_bounds__(NTHR) k_rho_var(const T* __restrict__ rho, lon
 }
 
 // Q = (|Omega|^2 - |S|^2) / 2 = -(sum_i A_ii^2 / 2 + A_01 A_10 + A_02 A_20 + A_12 A_21), A the Gauss
-// velocity gradient.  FP64 fields: in FP64.  FP32 fields: every step in float pairs (exact
-// differences, about 46 bits after that, rounded to FP32 once), since the FP64 pipe has 1/64 of the
-// FP32 pipe's lanes: 0.3 thousand FP32 operations per cell against 70 FP64 ones.
-__device__ __forceinline__ double q_of(const double (&g)[3][3], double scale) {
-  return -scale * (0.5 * (g[0][0] * g[0][0] + g[1][1] * g[1][1] + g[2][2] * g[2][2]) + g[0][1] * g[1][0] +
-                   g[0][2] * g[2][0] + g[1][2] * g[2][1]);
-}
-__device__ __forceinline__ float q_of(const DF (&g)[3][3], double scale) {
-  DF d = df_add(df_add(df_mul(g[0][0], g[0][0]), df_mul(g[1][1], g[1][1])), df_mul(g[2][2], g[2][2]));
-  d = DF{0.5f * d.hi, 0.5f * d.lo};
-  DF o = df_add(df_add(df_mul(g[0][1], g[1][0]), df_mul(g[0][2], g[2][0])), df_mul(g[1][2], g[2][1]));
-  return df_mul(df_add(d, o), df_from_double(-scale)).hi;
-}
-__device__ __forceinline__ double grad16(const double (&v)[4]) { return 10.0 * (v[2] - v[1]) - (v[3] - v[0]); }
-__device__ __forceinline__ DF grad16(const float (&v)[4]) {
-  const DF a = df_two_sum(v[2], -v[1]), b = df_two_sum(v[3], -v[0]);
-  const float h = __fmul_rn(10.f, a.hi), l = __fmaf_rn(10.f, a.hi, -h);
-  const DF t = df_two_sum(h, -b.hi);
-  return df_fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(l, __fmaf_rn(10.f, a.lo, -b.lo))));
-}
-
+// velocity gradient; in FP64 for either field type, rounded to it once: strain and rotation may cancel.  About 36
+// FP64 operations per cell bound it, the planes staged as FP64 like k_diag's.
 template <typename T>
 __global__ void __launch_bounds__(NTHR) k_qcrit(const BoxDev* boxes, int box, int s, T* __restrict__ q) {
-  __shared__ T sh[3][kGradH][kGradW];
+  __shared__ double sh[3][kGradH][kGradW];
   const BoxDev& B = boxes[box];
   const int N = B.N;
-  GradTile<T, T> t(F<T>(B, S(s, F_U0)), F<T>(B, S(s, F_U1)), F<T>(B, S(s, F_U2)), N, sh);
+  GradTile<T, double> t(F<T>(B, S(s, F_U0)), F<T>(B, S(s, F_U1)), F<T>(B, S(s, F_U2)), N, sh);
   const double scale = B.ih * B.ih * (1.0 / 256.0);
   const int k0 = blockIdx.z * kGradTz, kend = min(k0 + kGradTz, N);
   t.start(k0);
   for (int k = k0; k < kend; ++k) {
     t.next(k);
     if (t.i >= N || t.j >= N) continue;
-    Red<T> g[3][3];
+    double g[3][3];  // g[m][l] = 16 h Gc_m u_l
 #pragma unroll
     for (int m = 0; m < 3; ++m)
 #pragma unroll
       for (int l = 0; l < 3; ++l) {
-        T v[4];
+        double v[4];
         t.line(l, m, v);
-        g[m][l] = grad16(v);
+        g[m][l] = 10.0 * (v[2] - v[1]) - (v[3] - v[0]);
       }
-    q[t.plane(k) + t.own] = q_of(g, scale);
+    const double qv = -scale * (0.5 * (g[0][0] * g[0][0] + g[1][1] * g[1][1] + g[2][2] * g[2][2]) + g[0][1] * g[1][0] +
+                                g[0][2] * g[2][0] + g[1][2] * g[2][1]);
+    if constexpr (sizeof(T) == 4) q[t.plane(k) + t.own] = narrow(qv);
+    else q[t.plane(k) + t.own] = qv;
   }
 }
 
