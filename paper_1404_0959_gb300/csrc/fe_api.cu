@@ -106,10 +106,11 @@ struct fe_ctx {
   BoxDev* dbox = nullptr;
   int2* dwork = nullptr;
   int nblocks = 0;
-  BoxDev* dkbox = nullptr;  // FP64 default tiling: the Krylov kernels' own tiles (null: the step's)
-  int2* dkwork = nullptr;
-  int nkblocks = 0;
-  Persist* persist = nullptr;  // one-launch FP64 solve (null: the boxes do not fit it)
+  BoxDev* dkbox = nullptr;  // FP64: the Krylov kernels' own tiles and chunks (null: the step's)
+  int2 *dkwork = nullptr, *dkework = nullptr;
+  int nkblocks = 0, nkeblocks = 0;
+  int nkloop = 0, nkeloop = 0;  // of these, at the front: the boxes without a one-launch solve
+  Persist* persist = nullptr;   // one-launch FP64 solves (null: no box takes one)
   int2* dework = nullptr;
   int2* dbwork = nullptr;   // plane-streaming blocks (box, block of box)
   int nbblocks = 0, bsmem = 0, bcells = 0, npart = 0;
@@ -160,7 +161,15 @@ struct fe_ctx {
     l.kboxes = dkbox ? dkbox : dbox;
     l.kwork = dkbox ? dkwork : dwork;
     l.nkblocks = dkbox ? nkblocks : nblocks;
+    l.kework = dkbox ? dkework : dework;
+    l.nkeblocks = dkbox ? nkeblocks : neblocks;
     return l;
+  }
+  // l for the Krylov kernels of the boxes without a one-launch solve; false: there are none
+  bool loop_boxes(Launch& l) const {
+    l.nkblocks = nkloop;
+    l.nkeblocks = nkeloop;
+    return nkloop > 0;
   }
 };
 
@@ -261,9 +270,25 @@ static int validate(const fe_params* p) {
 #ifndef FE_ECHUNKS
 #define FE_ECHUNKS 8  // one wave of eight 256-thread blocks per SM (measured: the residual update 57 -> 54 us at 256^3)
 #endif
-// Built-in tile depth of the FP64 Krylov kernels: a function of the box alone, so that a box's sums,
-// and with them its iterates, are the same in an ensemble as on its own.
+// FP64 solves: the built-in tile depth and the chunk of the Krylov kernels are functions of the box alone, like the
+// choice of the one-launch solve, so that for one right-hand side a box's sums, and with them its iterates, are the
+// same in an ensemble as on its own.  (With chunks set by all boxes eight of 96^3 took 27.6 ms a step, 28.2 so.)
 static int tz_krylov(int N) { return N >= 128 ? 8 : 4; }
+
+// Cells per block of the element-wise kernels on `total` cells: about one wave of FE_ECHUNKS blocks per SM, so
+// the per-block reduction tail (fence + counter) is paid rarely.
+static long chunk_for(const fe_ctx* c, long total) {
+  const long quantum = 4L * NTHR, blocks = (long)FE_ECHUNKS * c->nsm;
+  return std::max(quantum, ((total + blocks - 1) / blocks + quantum - 1) / quantum * quantum);
+}
+
+static void chunk_box(BoxDev& B, long chunk, int box, std::vector<int2>& work) {
+  const long n = (long)B.N * B.N * B.N;
+  B.echunk = (int)chunk;
+  B.entiles = (int)((n + chunk - 1) / chunk);
+  B.etile0 = (int)work.size();
+  for (int q = 0; q < B.entiles; ++q) work.push_back(make_int2(box, q));
+}
 
 static void tile_box(BoxDev& B, int tz, int box, std::vector<int2>& work) {
   const int N = B.N;
@@ -315,24 +340,14 @@ static int tz_default(const fe_ctx* c) {
 // (Re)build the work lists for the tile depths tzb (tzb[b] = 0: the built-in depth) and upload the
 // descriptors.  Grows the partial-sum buffer when needed.
 static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
-  std::vector<int2> work, ework, kwork;
+  std::vector<int2> work, ework, kwork, kework;
   std::vector<BoxDev> kbox;
   const int tz0 = tz_default(c);
-  // element-wise chunk: about two waves of 8 blocks per SM over all boxes, so
-  // the per-block reduction tail (fence + counter) is paid rarely
   long total = 0;
   for (int b = 0; b < c->nb; ++b) total += (long)c->hbox[b].N * c->hbox[b].N * c->hbox[b].N;
-  const long quantum = 4L * NTHR;
-  long chunk = (total + (long)FE_ECHUNKS * c->nsm - 1) / ((long)FE_ECHUNKS * c->nsm);
-  chunk = std::max(quantum, (chunk + quantum - 1) / quantum * quantum);
   for (int b = 0; b < c->nb; ++b) {
-    BoxDev& B = c->hbox[b];
-    tile_box(B, tzb[b] > 0 ? tzb[b] : tz0, b, work);
-    const long n = (long)B.N * B.N * B.N;
-    B.echunk = (int)chunk;
-    B.entiles = (int)((n + chunk - 1) / chunk);
-    B.etile0 = (int)ework.size();
-    for (int q = 0; q < B.entiles; ++q) ework.push_back(make_int2(b, q));
+    tile_box(c->hbox[b], tzb[b] > 0 ? tzb[b] : tz0, b, work);
+    chunk_box(c->hbox[b], chunk_for(c, total), b, ework);
   }
   c->ring_ok = 2;
   for (int b = 0; b < c->nb; ++b)
@@ -377,12 +392,21 @@ static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
     bcells = 0;
     for (int b = 0; b < c->nb; ++b) c->hbox[b].btile0 = c->hbox[b].bntiles = 0;
   }
+  int nkloop = 0, nkeloop = 0;
   if (c->fp64) {
     kbox = c->hbox;
-    for (int b = 0; b < c->nb; ++b) tile_box(kbox[b], tzb[b] > 0 ? tzb[b] : tz_krylov(kbox[b].N), b, kwork);
+    for (const bool one_launch : {false, true}) {
+      for (int b = 0; b < c->nb; ++b) {
+        const int N = kbox[b].N;
+        if (persist_takes(c->persist, b) != one_launch) continue;
+        tile_box(kbox[b], tzb[b] > 0 ? tzb[b] : tz_krylov(N), b, kwork);
+        chunk_box(kbox[b], chunk_for(c, (long)N * N * N), b, kework);
+      }
+      if (!one_launch) nkloop = (int)kwork.size(), nkeloop = (int)kework.size();
+    }
   }
   CK(cudaStreamSynchronize(c->st));
-  const int need = (int)std::max(std::max(work.size(), ework.size()), std::max(bwork.size(), kwork.size()));
+  const int need = (int)std::max({work.size(), ework.size(), bwork.size(), kwork.size(), kework.size()});
   cudaFree(c->dbwork);
   c->dbwork = nullptr;
   if (!bwork.empty() && cudaMalloc(&c->dbwork, bwork.size() * sizeof(int2)) != cudaSuccess) return FE_ERR_OOM;
@@ -392,12 +416,18 @@ static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
   c->bsmem = bsmem;
   c->bcells = bcells;
   cudaFree(c->dkwork);
-  c->dkwork = nullptr;
+  cudaFree(c->dkework);
+  c->dkwork = c->dkework = nullptr;
   if (c->fp64) {
     if ((!c->dkbox && cudaMalloc(&c->dkbox, c->nb * sizeof(BoxDev)) != cudaSuccess) ||
-        cudaMalloc(&c->dkwork, kwork.size() * sizeof(int2)) != cudaSuccess)
+        cudaMalloc(&c->dkwork, kwork.size() * sizeof(int2)) != cudaSuccess ||
+        cudaMalloc(&c->dkework, kework.size() * sizeof(int2)) != cudaSuccess)
       return FE_ERR_OOM;
     c->nkblocks = (int)kwork.size();
+    c->nkeblocks = (int)kework.size();
+    c->nkloop = nkloop;
+    c->nkeloop = nkeloop;
+    CK(cudaMemcpyAsync(c->dkework, kework.data(), kework.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync(c->dkwork, kwork.data(), kwork.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync(c->dkbox, kbox.data(), c->nb * sizeof(BoxDev), cudaMemcpyHostToDevice, c->st));
   }
@@ -569,6 +599,7 @@ extern "C" void fe_destroy(fe_ctx* c) {
   cudaFree(c->dwork);
   cudaFree(c->dkbox);
   cudaFree(c->dkwork);
+  cudaFree(c->dkework);
   persist_free(c->persist);
   cudaFree(c->dework);
   cudaFree(c->dbwork);
@@ -644,7 +675,10 @@ template <typename T>
 static int krylov(fe_ctx* c, int maxit, int key) {
   Launch L = c->L();
   const bool bicg = c->prm.solver == FE_BICGSTAB_JACOBI;
-  if (sizeof(T) == 8 && L.persist && !c->harvest_b) return launch_persist(L);
+  if (sizeof(T) == 8 && L.persist && !c->harvest_b) {
+    const int rc = launch_persist(L);
+    if (rc != FE_OK || !c->loop_boxes(L)) return rc;
+  }
   CK(cudaMemsetAsync(c->dactive, 0, sizeof(int), c->st));
   if (bicg) launch_bicg_init<T>(L);
   else launch_cg_init<T>(L, 0.0);
@@ -1039,7 +1073,10 @@ static int krylov_graph(fe_ctx* c, int lev) {
   L.st = cs;
   const int maxit = c->prm.p_maxit;
   const bool bicg = c->prm.solver == FE_BICGSTAB_JACOBI;
-  if (sizeof(T) == 8 && L.persist) return launch_persist(L);
+  if (sizeof(T) == 8 && L.persist) {
+    const int rc = launch_persist(L);
+    if (rc != FE_OK || !c->loop_boxes(L)) return rc;
+  }
   CK(cudaMemsetAsync(c->dactive, 0, sizeof(int), cs));
   const bool learned = c->prm.solver == FE_FCG_LEARNED;
   BoxDev& B0 = c->hbox[0];

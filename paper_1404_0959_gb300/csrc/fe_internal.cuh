@@ -609,7 +609,9 @@ struct Launch {
   const BoxDev* kboxes = nullptr;  // the boxes under the tiling of the Krylov kernels (their sums follow it)
   const int2* kwork = nullptr;
   int nkblocks = 0;
-  Persist* persist = nullptr;  // the one-launch FP64 solve (null: the boxes do not fit it)
+  const int2* kework = nullptr;  // and the chunks of their element-wise kernels
+  int nkeblocks = 0;
+  Persist* persist = nullptr;  // the one-launch FP64 solves (null: no box takes one)
   int bcells = 0;         // cells per block of the streamed CG kernels (kBulkCells or kBulkCellsPoly)
 };
 
@@ -678,6 +680,7 @@ template <typename V> void launch_bicg_v(const Launch& L);
 template <typename V> void launch_bicg_s(const Launch& L);
 template <typename V> void launch_bicg_x(const Launch& L);
 int launch_persist(const Launch& L);  // krylov_persist.cu: whole FP64 solves of small boxes
+bool persist_takes(const Persist* P, int box);
 template <typename V> void launch_mix_residual(const Launch& L, int first, int* outer_active);
 template <typename V> void launch_mix_accum(const Launch& L);
 template <typename V> void launch_mix_finish(const Launch& L);

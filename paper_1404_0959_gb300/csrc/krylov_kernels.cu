@@ -1875,16 +1875,16 @@ __global__ void __launch_bounds__(NTHR) k_fcg_matvec(const BoxDev* boxes, const 
 
 // ---- launchers ------------------------------------------------------------------------
 #define GRID L.nkblocks, dim3(TX, TY), 0, L.st  // tile kernels: the Krylov tiling
-#define EGRID L.neblocks, dim3(TX, TY), 0, L.st
+#define EGRID L.nkeblocks, dim3(TX, TY), 0, L.st  // element-wise kernels: the Krylov chunks
 template <typename T> void launch_cg_init(const Launch& L, double) {
-  FE_LAUNCH(L, KID_CG_INIT, (k_cg_init<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
+  FE_LAUNCH(L, KID_CG_INIT, (k_cg_init<T><<<EGRID>>>(L.kboxes, L.kework, L.part, L.active)));
 }
 template <typename T> void launch_cg_matvec(const Launch& L) {
   if (L.transonic) FE_LAUNCH(L, KID_CG_MATVEC, (k_cg_matvec<T><<<GRID>>>(L.kboxes, L.kwork, L.part)));
   else FE_LAUNCH(L, KID_CG_MATVEC, (kz_cg_matvec<T><<<GRID>>>(L.kboxes, L.kwork, L.part)));
 }
 template <typename T> void launch_cg_update(const Launch& L) {
-  FE_LAUNCH(L, KID_CG_UPDATE, (k_cg_update<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
+  FE_LAUNCH(L, KID_CG_UPDATE, (k_cg_update<T><<<EGRID>>>(L.kboxes, L.kework, L.part, L.active)));
 }
 template <typename T> void launch_cg_fused(const Launch& L) {
   if (L.poly) {  // polynomial preconditioner: direction from z, residual update forms the next z
@@ -1909,7 +1909,7 @@ template <typename T> void launch_cg_fused(const Launch& L) {
                                        L.boxes, L.bwork, L.part)));
   else
     FE_LAUNCH(L, KID_CG_DIRMATVEC, (kz_cg_dirmatvec<T, sizeof(T) == 8><<<GRID>>>(L.kboxes, L.kwork, L.part)));
-  FE_LAUNCH(L, KID_CG_RUPDATE, (k_cg_rupdate<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
+  FE_LAUNCH(L, KID_CG_RUPDATE, (k_cg_rupdate<T><<<EGRID>>>(L.kboxes, L.kework, L.part, L.active)));
 }
 // First polynomial-preconditioned residual z = P r of an inner solve and <r, z> (nothing without it)
 template <typename T> void launch_cg_start(const Launch& L) {
@@ -1924,10 +1924,10 @@ template <typename T> void launch_cg_start(const Launch& L) {
     FE_LAUNCH(L, KID_CG_START, (kz_cg_rpoly<T, true><<<GRID>>>(L.kboxes, L.kwork, L.part, L.active)));
 }
 template <typename T> void launch_cg_xfinal(const Launch& L) {
-  FE_LAUNCH(L, KID_CG_XFINAL, (k_cg_xfinal<T><<<EGRID>>>(L.boxes, L.ework)));
+  FE_LAUNCH(L, KID_CG_XFINAL, (k_cg_xfinal<T><<<EGRID>>>(L.kboxes, L.kework)));
 }
 template <typename T> void launch_cg_dir(const Launch& L) {
-  FE_LAUNCH(L, KID_CG_DIR, (k_cg_dir<T><<<EGRID>>>(L.boxes, L.ework)));
+  FE_LAUNCH(L, KID_CG_DIR, (k_cg_dir<T><<<EGRID>>>(L.kboxes, L.kework)));
 }
 template <typename T> void launch_true_res(const Launch& L, int xs) {
   FE_LAUNCH(L, KID_TRUE_RES, (k_true_res<T><<<GRID>>>(L.kboxes, L.kwork, L.part, xs)));
@@ -1949,21 +1949,21 @@ template <typename T> void launch_bicg_x(const Launch& L) {
   FE_LAUNCH(L, KID_BICG_X, (k_bicg_x<T><<<GRID>>>(L.kboxes, L.kwork, L.part, L.active)));
 }
 template <typename T> void launch_fcg(const Launch& L, const float* z) {
-  FE_LAUNCH(L, KID_FCG_DOTS, (k_fcg_dots<T><<<EGRID>>>(L.boxes, L.ework, L.part, z)));
-  FE_LAUNCH(L, KID_FCG_DIR, (k_fcg_dir<T><<<EGRID>>>(L.boxes, L.ework, z)));
+  FE_LAUNCH(L, KID_FCG_DOTS, (k_fcg_dots<T><<<EGRID>>>(L.kboxes, L.kework, L.part, z)));
+  FE_LAUNCH(L, KID_FCG_DIR, (k_fcg_dir<T><<<EGRID>>>(L.kboxes, L.kework, z)));
   FE_LAUNCH(L, KID_FCG_MATVEC, (k_fcg_matvec<T><<<GRID>>>(L.kboxes, L.kwork, L.part)));
-  FE_LAUNCH(L, KID_CG_UPDATE, (k_cg_update<T><<<EGRID>>>(L.boxes, L.ework, L.part, L.active)));
+  FE_LAUNCH(L, KID_CG_UPDATE, (k_cg_update<T><<<EGRID>>>(L.kboxes, L.kework, L.part, L.active)));
 }
 template <typename T> void launch_mix_residual(const Launch& L, int first, int* outer_active) {
   if (first)
-    FE_LAUNCH(L, KID_MIX_RES, (k_mix_first<T><<<EGRID>>>(L.boxes, L.ework, L.part, outer_active)));
+    FE_LAUNCH(L, KID_MIX_RES, (k_mix_first<T><<<EGRID>>>(L.kboxes, L.kework, L.part, outer_active)));
   else if (L.transonic)
     FE_LAUNCH(L, KID_MIX_RES, (k_mix_residual<T><<<GRID>>>(L.kboxes, L.kwork, L.part, first, outer_active)));
   else
     FE_LAUNCH(L, KID_MIX_RES, (kz_mix_residual<T><<<GRID>>>(L.kboxes, L.kwork, L.part, outer_active)));
 }
 template <typename T> void launch_refine_start(const Launch& L, int* outer_active) {
-  FE_LAUNCH(L, KID_MIX_RES, (k_refine_start<T><<<EGRID>>>(L.boxes, L.ework, L.part, outer_active, L.active)));
+  FE_LAUNCH(L, KID_MIX_RES, (k_refine_start<T><<<EGRID>>>(L.kboxes, L.kework, L.part, outer_active, L.active)));
   launch_cg_start<T>(L);
 }
 template <typename T> void launch_refine(const Launch& L, int* outer_active) {
@@ -1976,13 +1976,13 @@ template <typename T> void launch_refine(const Launch& L, int* outer_active) {
   launch_cg_start<T>(L);
 }
 template <typename T> void launch_mix_finish_pp(const Launch& L) {
-  FE_LAUNCH(L, KID_MIX_FIN, (k_mix_finish<T><<<EGRID>>>(L.boxes, L.ework, 1)));
+  FE_LAUNCH(L, KID_MIX_FIN, (k_mix_finish<T><<<EGRID>>>(L.kboxes, L.kework, 1)));
 }
 template <typename T> void launch_mix_accum(const Launch& L) {
-  FE_LAUNCH(L, KID_MIX_ACC, (k_mix_accum<T><<<EGRID>>>(L.boxes, L.ework)));
+  FE_LAUNCH(L, KID_MIX_ACC, (k_mix_accum<T><<<EGRID>>>(L.kboxes, L.kework)));
 }
 template <typename T> void launch_mix_finish(const Launch& L) {
-  FE_LAUNCH(L, KID_MIX_FIN, (k_mix_finish<T><<<EGRID>>>(L.boxes, L.ework, 0)));
+  FE_LAUNCH(L, KID_MIX_FIN, (k_mix_finish<T><<<EGRID>>>(L.kboxes, L.kework, 0)));
 }
 
 // Cells per block of the streamed CG kernels of one solver for the box edges

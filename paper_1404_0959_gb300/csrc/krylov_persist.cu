@@ -13,7 +13,8 @@
 // units (adjacent pairs, then pairs of pairs): a block publishes the sum of its
 // subtree, and every block adds those of its box up the rest of the tree.  So the
 // sums (and the iterates) of a box do not depend on how many blocks it was given,
-// in an ensemble or alone, and no block waits for a coordinator's value.
+// in an ensemble or alone, and no block waits for a coordinator's value.  Boxes that the device
+// cannot hold at once are launched in groups, one after the other.
 //
 // A meeting: publish, count up the box's counter, wait until all blocks have (one
 // thread per block polls), read the published sums.  Two sets of sums alternate: a
@@ -491,9 +492,14 @@ static PkKernel pk_kernel(bool bicg, int upc) {
   return upc == 1 ? kc_cg<1> : upc == 2 ? kc_cg<2> : upc == 4 ? kc_cg<4> : kc_cg<8>;
 }
 
-// The one-launch solve of a context's boxes: blocks, counters, sums, BiCGStab coefficients in one allocation.
+// The one-launch solves of a context: the blocks of the boxes that take one, in groups that the device holds at
+// once (one launch each), their counters, sums and BiCGStab coefficients, in one allocation.
+struct PkGroup {
+  int first, blocks, upc;
+};
 struct Persist {
-  int blocks = 0, upc = 0;
+  std::vector<PkGroup> groups;
+  std::vector<char> takes;  // per box
   size_t counter_bytes = 0;
   PkBlock* work = nullptr;
   unsigned* counters = nullptr;
@@ -508,50 +514,76 @@ void persist_free(Persist* P) {
   delete P;
 }
 
-// null with *rc = FE_OK: the boxes do not fit the device at once, or it has no cooperative launches.
+bool persist_takes(const Persist* P, int box) { return P && P->takes[box]; }
+
+// A box takes the one-launch solve where the device holds its blocks at once: a function of the box alone, since
+// the kernel-by-kernel solve adds its sums in another order.  The boxes that do are filled into groups at the most
+// units per block; a group then runs with the fewest that fit.  Against the kernel-by-kernel solve of all boxes of a
+// context that is too large for one launch, ms per step: CG, where that solve is bound by the FP64 pipe too and forms
+// each direction once, 3 boxes of 64^3 4.48 -> 4.66, 8 of them 9.97 -> 11.5, 64 of 32^3 to 96^3 82.0 -> 90.6;
+// BiCGStab, 8 boxes of 48^3 16.3 -> 7.8, 48 of 32^3 24.8 -> 13.1.
+// null with *rc = FE_OK: no box does, or the device has no cooperative launches.
 Persist* persist_create(const int* N, int nb, int nsm, bool bicg, cudaStream_t st, int* rc) {
   *rc = FE_OK;
   int dev = 0, coop = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
     return nullptr;
-  std::vector<long> u(nb);
-  for (int b = 0; b < nb; ++b) u[b] = ((long)N[b] * N[b] * N[b] + kPkThreads - 1) / kPkThreads;
   const int most = bicg ? kPkBicgUnits : kPkMaxUnits;
-  int upc = 1;
-  for (; upc <= most; upc *= 2) {
+  long cap[kPkMaxUnits + 1];  // resident blocks of the device, per units of a block
+  for (int upc = 1; upc <= most; upc *= 2) {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pk_kernel(bicg, upc), kPkThreads, 0) != cudaSuccess)
       return nullptr;
-    const long cap = (long)std::min(per_sm, kPkPerSm) * nsm;
-    long blocks = 0, largest = 0;
-    for (int b = 0; b < nb; ++b) {
-      const long q = (u[b] + upc - 1) / upc;
-      blocks += q;
-      largest = std::max(largest, q);
+    cap[upc] = (long)std::min(per_sm, kPkPerSm) * nsm;
+  }
+  auto units = [&](int b) { return ((long)N[b] * N[b] * N[b] + kPkThreads - 1) / kPkThreads; };
+  auto blocks = [&](int b, int upc) { return (units(b) + upc - 1) / upc; };
+  auto fits = [&](const std::vector<int>& g, int upc) {
+    long sum = 0, largest = 0;
+    for (int b : g) {
+      sum += blocks(b, upc);
+      largest = std::max(largest, blocks(b, upc));
     }
-    if (blocks <= cap && largest <= (long)kPkLeaves * kPkThreads) break;
-  }
-  if (upc > most) return nullptr;
-  std::vector<PkBlock> work;
-  long cells = 0;
+    return sum <= cap[upc] && largest <= (long)kPkLeaves * kPkThreads;
+  };
+  std::vector<char> takes(nb, 0);
+  std::vector<std::vector<int>> groups;
   for (int b = 0; b < nb; ++b) {
-    const int b0 = (int)work.size();
-    for (long q = 0; q < u[b]; q += upc)
-      work.push_back(PkBlock{b, (int)q, (int)std::min<long>(upc, u[b] - q), b0, cells});
-    cells += (long)N[b] * N[b] * N[b];
+    if (!fits({b}, most)) continue;
+    takes[b] = 1;
+    if (!groups.empty()) {
+      groups.back().push_back(b);
+      if (fits(groups.back(), most)) continue;
+      groups.back().pop_back();
+    }
+    groups.push_back({b});
   }
+  if (groups.empty()) return nullptr;
   Persist* P = new (std::nothrow) Persist();
   if (!P) {
     *rc = FE_ERR_OOM;
     return nullptr;
   }
-  P->blocks = (int)work.size();
-  P->upc = upc;
   P->bicg = bicg;
+  P->takes = takes;
+  std::vector<PkBlock> work;
+  long cells = 0;
+  for (const std::vector<int>& g : groups) {
+    int upc = 1;
+    while (!fits(g, upc)) upc *= 2;
+    const int first = (int)work.size();
+    for (int b : g) {
+      const int b0 = (int)work.size();
+      for (long q = 0; q < units(b); q += upc)
+        work.push_back(PkBlock{b, (int)q, (int)std::min<long>(upc, units(b) - q), b0, cells});
+      cells += (long)N[b] * N[b] * N[b];
+    }
+    P->groups.push_back(PkGroup{first, (int)work.size() - first, upc});
+  }
   P->counter_bytes = ((size_t)nb * kPkLine * sizeof(unsigned) + 255) / 256 * 256;
   const size_t wb = (work.size() * sizeof(PkBlock) + 255) / 256 * 256;
-  const size_t sb = ((size_t)P->blocks * 4 * sizeof(double) + 255) / 256 * 256;
+  const size_t sb = (work.size() * 4 * sizeof(double) + 255) / 256 * 256;
   const size_t cb = bicg ? (size_t)cells * kPkCoef * sizeof(double) : 0;
   if (cudaMalloc(&P->work, wb + P->counter_bytes + sb + cb) != cudaSuccess) {
     cudaGetLastError();
@@ -573,17 +605,21 @@ Persist* persist_create(const int* N, int nb, int nsm, bool bicg, cudaStream_t s
   return P;
 }
 
-// The whole solve of every box from K_B into K_X (FP64 fields; psi, D^{-1} and the scalars in place).
+// The whole solve of every box that takes one, from K_B into K_X (FP64 fields; psi, D^{-1} and the scalars in place).
 int launch_persist(const Launch& L) {
   Persist* P = L.persist;
   if (cudaMemsetAsync(P->counters, 0, P->counter_bytes, L.st) != cudaSuccess) return FE_ERR_CUDA;
-  const BoxDev* boxes = L.boxes;
-  void* args[] = {&boxes, &P->work, &P->sums, &P->counters, &P->coef};
-  cudaError_t e = cudaSuccess;
-  FE_LAUNCH(L, KID_SOLVE,
-            (e = cudaLaunchCooperativeKernel((const void*)pk_kernel(P->bicg, P->upc), dim3(P->blocks),
-                                             dim3(kPkThreads), args, 0, L.st)));
-  return e == cudaSuccess ? FE_OK : FE_ERR_CUDA;
+  for (const PkGroup& g : P->groups) {
+    const BoxDev* boxes = L.boxes;
+    PkBlock* work = P->work + g.first;
+    void* args[] = {&boxes, &work, &P->sums, &P->counters, &P->coef};
+    cudaError_t e = cudaSuccess;
+    FE_LAUNCH(L, KID_SOLVE,
+              (e = cudaLaunchCooperativeKernel((const void*)pk_kernel(P->bicg, g.upc), dim3(g.blocks),
+                                               dim3(kPkThreads), args, 0, L.st)));
+    if (e != cudaSuccess) return FE_ERR_CUDA;
+  }
+  return FE_OK;
 }
 
 }  // namespace fe
