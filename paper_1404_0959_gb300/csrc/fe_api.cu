@@ -652,6 +652,13 @@ static int pull_scalars(fe_ctx* c) {
   return FE_OK;
 }
 
+// After pull_scalars: a kernel of the finished step or solve gave up a bounded wait, its results are not to be used.
+static bool gave_up(const fe_ctx* c) {
+  for (int b = 0; b < c->nb; ++b)
+    if (c->hsc[(size_t)b * NSC + SC_KERR] != 0.0) return true;
+  return false;
+}
+
 static int push_scalar(fe_ctx* c, int box, int idx, double v) {
   c->hsc[(size_t)box * NSC + idx] = v;
   CK(cudaMemcpyAsync(c->dsc + (size_t)box * NSC + idx, c->hsc + (size_t)box * NSC + idx, sizeof(double),
@@ -1275,9 +1282,9 @@ static int step_once(fe_ctx* c, bool commit = true) {
   if (!commit) return FE_OK;
   int rc = pull_scalars(c);
   if (rc != FE_OK) return rc;
+  if (gave_up(c)) return FE_ERR_CUDA;
   for (int b = 0; b < c->nb; ++b) {
     const double* sc = c->hsc + (size_t)b * NSC;
-    if (sc[SC_KERR] != 0.0) return FE_ERR_CUDA;
     if (sc[SC_BAD] > 0.0 || !std::isfinite(sc[SC_DT])) return FE_ERR_NONFINITE;
     for (int kk = 0; kk < nc; ++kk)
       if (!(sc[SC_RES0 + kk] <= c->prm.p_tol * (1.0 + 1e-3))) return FE_ERR_NOT_CONVERGED;
@@ -1466,12 +1473,13 @@ static int solve_box(fe_ctx* c, int box, const void* b, void* x, double dt, doub
     inf.iters = (int)s[SC_ITSUM];
     inf.rel_res_true = s[SC_ORES];
   }
-  bool conv = s[SC_CONV] != 0.0;
+  const bool conv = s[SC_CONV] != 0.0, failed = gave_up(c);
   if (info) *info = inf;
   // restore the step scalars (tolerance, cap, dt) of every box
   memcpy(c->hsc, saved.data(), saved.size() * sizeof(double));
   CK(cudaMemcpyAsync(c->dsc, c->hsc, (size_t)c->nb * NSC * sizeof(double), cudaMemcpyHostToDevice, c->st));
   CK(cudaStreamSynchronize(c->st));
+  if (failed) return FE_ERR_CUDA;
   return conv ? FE_OK : FE_ERR_NOT_CONVERGED;
 }
 
