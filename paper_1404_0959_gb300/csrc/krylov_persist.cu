@@ -37,7 +37,10 @@ constexpr int kPkWarps = kPkThreads / 32;
 constexpr int kPkPerSm = 4;      // resident blocks per SM asked for (128 registers)
 constexpr int kPkMaxUnits = 8;   // units per block, at most
 constexpr int kPkLeaves = 8;     // published sums per thread, at most: 1024 blocks of a box
-constexpr int kPkSpins = 1 << 22;
+#ifndef FE_PK_SPINS
+#define FE_PK_SPINS (1 << 22)  // polls of a meeting's counter before a block gives up: seconds
+#endif
+constexpr int kPkSpins = FE_PK_SPINS;
 constexpr int kPkLine = 32;      // words between the counters of two boxes (one line each)
 
 // A block's place: box, its first unit, its units, the box's first block and first cell among all boxes.
