@@ -42,6 +42,8 @@ void persist_free(Persist* P);
 UNet* unet_create(int N, bool training, int* rc);
 void unet_destroy(UNet* U);
 long unet_param_count();
+void unet_queue_error(UNet* U, cudaStream_t st);
+bool unet_failed(UNet* U, cudaStream_t st);
 int unet_set_weights(UNet* U, const float* host, cudaStream_t st);
 int unet_get_weights(UNet* U, float* host, int which, cudaStream_t st);
 template <typename T> void unet_apply_sc(UNet*, const T*, const T*, double*, int, double, cudaStream_t);
@@ -648,15 +650,17 @@ static int field_slot(const fe_ctx* c, int field, int set) {
 
 static int pull_scalars(fe_ctx* c) {
   CK(cudaMemcpyAsync(c->hsc, c->dsc, (size_t)c->nb * NSC * sizeof(double), cudaMemcpyDeviceToHost, c->st));
+  if (c->unet) unet_queue_error(c->unet, c->st);
   CK(cudaStreamSynchronize(c->st));
   return FE_OK;
 }
 
-// After pull_scalars: a kernel of the finished step or solve gave up a bounded wait, its results are not to be used.
-static bool gave_up(const fe_ctx* c) {
-  for (int b = 0; b < c->nb; ++b)
-    if (c->hsc[(size_t)b * NSC + SC_KERR] != 0.0) return true;
-  return false;
+// After pull_scalars: a kernel of the finished step or solve, or a convolution of its network, gave up a bounded
+// wait; its results are not to be used.
+static bool gave_up(fe_ctx* c) {
+  bool bad = c->unet && unet_failed(c->unet, c->st);
+  for (int b = 0; b < c->nb; ++b) bad = bad || c->hsc[(size_t)b * NSC + SC_KERR] != 0.0;
+  return bad;
 }
 
 static int push_scalar(fe_ctx* c, int box, int idx, double v) {

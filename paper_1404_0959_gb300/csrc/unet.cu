@@ -616,6 +616,7 @@ struct UNet {
   bool trained = false;
   int use_tc = 1;      // stride-1 layers on the fifth-generation tensor cores where they fit
   int* err = nullptr;  // device flag: a tensor-core convolution gave up a bounded wait
+  int* herr = nullptr;  // pinned copy of it
   int nsm = 152;
 };
 
@@ -663,6 +664,7 @@ static int unet_alloc(UNet& U, int N, bool training) {
       U.nsm = nsm;
   }
   U.xfer = (float*)A(unet_param_count() * 4);
+  if (cudaMallocHost(&U.herr, sizeof(int)) != cudaSuccess) return FE_ERR_OOM;
   if (!U.xfer || !U.in16 || !U.e1a || !U.e1b || !U.d1 || !U.e2 || !U.d2 || !U.e3 || !U.u2 || !U.u1 || !U.out32 || !U.err)
     return FE_ERR_OOM;
   size_t wtotal = 0;
@@ -716,6 +718,8 @@ static int unet_alloc(UNet& U, int N, bool training) {
 static void unet_free(UNet& U) {
   for (void* p : U.allocs) cudaFree(p);
   U.allocs.clear();
+  if (U.herr) cudaFreeHost(U.herr);
+  U.herr = nullptr;
 }
 
 static int ew(long n) {
@@ -1107,6 +1111,18 @@ static double host_sum(const double* dpart, int nb, cudaStream_t st) {
   return s;
 }
 
+// Queue the copy of the flag behind the work on st; after the stream has been waited for, unet_failed says whether
+// a convolution of that work gave up, and clears the flag.
+void unet_queue_error(UNet* U, cudaStream_t st) {
+  cudaMemcpyAsync(U->herr, U->err, sizeof(int), cudaMemcpyDeviceToHost, st);
+}
+bool unet_failed(UNet* U, cudaStream_t st) {
+  if (*U->herr == 0) return false;
+  cudaMemsetAsync(U->err, 0, sizeof(int), st);
+  *U->herr = 0;
+  return true;
+}
+
 UNet* unet_create(int N, bool training, int* rc) {
   UNet* U = new UNet();
   *rc = unet_alloc(*U, N, training);
@@ -1211,13 +1227,9 @@ int unet_apply(UNet* U, const T* r, const T* dinv, double dt, double ih, float* 
                                          U->in16);
   unet_forward(*U, st);
   k_direction<T><<<ew(n), 256, 0, st>>>(r, dinv, U->out32, rms * d0, n, z);
-  int herr = 0;
-  cudaMemcpyAsync(&herr, U->err, sizeof(int), cudaMemcpyDeviceToHost, st);
+  unet_queue_error(U, st);
   cudaStreamSynchronize(st);
-  if (herr) {
-    cudaMemsetAsync(U->err, 0, sizeof(int), st);
-    return FE_ERR_CUDA;
-  }
+  if (unet_failed(U, st)) return FE_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? FE_OK : FE_ERR_CUDA;
 }
 
@@ -1236,10 +1248,12 @@ int unet_train_step(UNet* U, const T* r, const T* e, const T* dinv, double dt, d
   if (!(rms > 0.0)) return FE_ERR_INVALID_ARG;
   k_pack_input<T><<<ew(v0), 256, 0, st>>>(r, dinv, v0, 1.0 / (rms * d0), 3.0 * dt * ih * ih, U->in16);
   unet_forward(*U, st);
+  unet_queue_error(U, st);
   // target into gsk0 (fp32 scratch), its norm, then loss and dL/dy
   float* tgt = U->gsk0;
   k_target<T><<<nb, 256, 0, st>>>(r, e, dinv, v0, 1.0 / (rms * d0), tgt, U->part);
   const double tt = host_sum(U->part, nb, st);
+  if (unet_failed(U, st)) return FE_ERR_CUDA;  // before any weight moves
   if (!(tt > 0.0)) return FE_ERR_INVALID_ARG;
   k_loss_grad<<<nb, 256, 0, st>>>(U->out32, tgt, v0, 1.0 / tt, U->dy8, U->part);
   *loss = host_sum(U->part, nb, st) / tt;

@@ -116,3 +116,65 @@ def test_solve_reports_a_wait_that_ran_out(fake, transonic):
     fake.effects = {}
     assert solve(s, 24) == fe.FE_ERR_NOT_CONVERGED  # kernels that do nothing converge to nothing
     s.close()
+
+
+class TcConvArgs(ctypes.Structure):
+    _fields_ = [("s0", ctypes.c_void_p), ("s1", ctypes.c_void_p), ("c0", ctypes.c_int), ("c1", ctypes.c_int),
+                ("m0", ctypes.c_int), ("m1", ctypes.c_int), ("No", ctypes.c_int), ("W", ctypes.c_void_p),
+                ("bias", ctypes.c_void_p), ("out", ctypes.c_void_p), ("out32", ctypes.c_void_p),
+                ("relu", ctypes.c_int), ("err", ctypes.c_void_p)]
+
+
+def learned(precision):
+    s = fe.Solver([dict(N=128, tau_p=[], Y0=[])], stream=0, solver=fe.FE_FCG_LEARNED, precision=precision)
+    w = np.zeros(fe.lib().fe_preconditioner_size(), dtype=np.float32)
+    assert fe.lib().fe_load_preconditioner(s.ctx, w.ctypes.data, w.size) == fe.FE_OK
+    return s
+
+
+def give_up_convolution(name, gx, args):
+    err = ctypes.cast(args[0], ctypes.POINTER(TcConvArgs))[0].err
+    ctypes.cast(err, ctypes.POINTER(ctypes.c_int))[0] = 1
+
+
+def train(s):
+    r = np.zeros(128 ** 3, dtype=np.float32)
+    loss = ctypes.c_double()
+    return fe.lib().fe_precond_train_step(s.ctx, 0, r.ctypes.data, r.ctypes.data, 0.1, 1e-3, ctypes.byref(loss))
+
+
+def one(i):
+    def effect(name, gx, args):
+        ctypes.cast(pointer(args, i), ctypes.POINTER(ctypes.c_double))[0] = 1.0
+    return effect
+
+
+def test_training_step_with_an_unfinished_convolution(fake):
+    """No weight is updated from activations of a convolution that gave up; the step fails, the next does not."""
+    s = learned(fe.FE_FP32_MIXED)
+    sums = {"k_sumsq": one(2), "k_target": one(6)}  # the norms of the residual and of the target
+    fake.effects = dict(sums, k_conv_ring=give_up_convolution)
+    assert train(s) == fe.FE_ERR_CUDA
+    assert fake.ran("k_conv_ring") and not fake.ran("k_adam")
+    fake.effects = sums
+    assert train(s) == fe.FE_OK and fake.ran("k_adam")
+    s.close()
+
+
+@pytest.mark.parametrize("what", ["solve", "step"])
+def test_learned_solve_with_an_unfinished_convolution(fake, what):
+    """The flag of a convolution that gave up fails the solve or step that ran it, and no later call."""
+    s = learned(fe.FE_FP64)
+
+    def running(name, gx, args):  # one box starts its solve
+        ctypes.cast(pointer(args, 3), ctypes.POINTER(ctypes.c_int))[0] = 1
+
+    call = (lambda: solve(s, 128, maxit=1)) if what == "solve" else (lambda: fe.lib().fe_step(s.ctx, 1, None))
+    fake.effects = {"k_cg_init": running, "k_conv_ring": give_up_convolution}
+    assert call() == fe.FE_ERR_CUDA and fake.ran("k_conv_ring")
+    fake.effects = {}
+    assert call() == (fe.FE_ERR_NOT_CONVERGED if what == "solve" else fe.FE_OK)
+    r = np.zeros(128 ** 3)
+    z = np.zeros(128 ** 3, dtype=np.float32)
+    assert fe.lib().fe_precond_apply(s.ctx, 0, r.ctypes.data, 0.1, z.ctypes.data) == fe.FE_OK
+    s.close()
