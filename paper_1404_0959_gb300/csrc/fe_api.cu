@@ -1667,6 +1667,8 @@ extern "C" int fe_autotune(fe_ctx* c, int trials, int* best_tz) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   int rc2 = set_tiling(c, best);
+  if (rc2 == FE_OK) rc2 = pull_scalars(c);
+  if (rc2 == FE_OK && gave_up(c)) rc2 = FE_ERR_CUDA;  // in a trial step: its times say nothing
   memcpy(c->hsc, saved.data(), saved.size() * sizeof(double));
   CK(cudaMemcpyAsync(c->dsc, c->hsc, saved.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
   CK(cudaStreamSynchronize(c->st));

@@ -154,6 +154,17 @@ int cudaMemcpyAsync(void* d, const void* s, size_t n, int, void*) {
   return 0;
 }
 int cudaStreamSynchronize(void*) { return 0; }
+int cudaEventCreate(void** e) {
+  *e = nullptr;
+  return 0;
+}
+int cudaEventDestroy(void*) { return 0; }
+int cudaEventRecord(void*, void*) { return 0; }
+int cudaEventSynchronize(void*) { return 0; }
+int cudaEventElapsedTime(float* ms, void*, void*) {
+  *ms = 1.f;
+  return 0;
+}
 // not reached by the tests
 #define UNUSED(f) \
   int f() { return ret(801); }
@@ -173,9 +184,4 @@ UNUSED(cudaGraphConditionalHandleCreate)
 UNUSED(cudaGraphAddNode)
 UNUSED(cudaGetSymbolAddress)
 UNUSED(cudaGetDriverEntryPointByVersion)
-UNUSED(cudaEventSynchronize)
-UNUSED(cudaEventRecord)
-UNUSED(cudaEventElapsedTime)
-UNUSED(cudaEventDestroy)
-UNUSED(cudaEventCreate)
 }

@@ -178,3 +178,20 @@ def test_learned_solve_with_an_unfinished_convolution(fake, what):
     z = np.zeros(128 ** 3, dtype=np.float32)
     assert fe.lib().fe_precond_apply(s.ctx, 0, r.ctypes.data, 0.1, z.ctypes.data) == fe.FE_OK
     s.close()
+
+
+def test_autotune_reports_a_wait_that_ran_out(fake):
+    """A trial step whose solve gives up fails fe_autotune, which puts the scalars back; the next step runs."""
+    kerr, nsc = scalar_slot("SC_KERR")
+    s = solver()
+    sc = ctypes.cast(fake.lib.fake_find(nsc * 8), ctypes.POINTER(ctypes.c_double))
+
+    def give_up(*_):
+        sc[kerr] = 1.0
+
+    fake.effects = {"kc_cg": give_up}
+    assert fe.lib().fe_autotune(s.ctx, 1, None) == fe.FE_ERR_CUDA and fake.ran("kc_cg")
+    fake.effects = {}
+    assert fe.lib().fe_step(s.ctx, 1, None) == fe.FE_OK
+    assert fe.lib().fe_autotune(s.ctx, 1, None) == fe.FE_OK
+    s.close()
