@@ -346,9 +346,10 @@ bool fft_supported(int N) { return N >= 2 && N <= kFftMaxN && radices_of(N).n >=
 
 static int fft_smem(int N) { return 2 * N * kFftLines * (int)sizeof(double2); }
 
+// the limit is one value per kernel and device, whoever launches it: always that of the longest line
 template <typename K>
-static cudaError_t fft_allow(K* kernel, int bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+static cudaError_t fft_allow(K* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, fft_smem(kFftMaxN));
 }
 
 // complex 3D transform in place (tw: the N-th roots)
@@ -356,7 +357,7 @@ static int fft3d(double2* data, int N, int inverse, const double2* tw, cudaStrea
   const Radices R = radices_of(N);
   const int lines = N * N, sm = fft_smem(N), grid = (lines + kFftLines - 1) / kFftLines;
   const long NN = (long)N * N;
-  if (fft_allow(k_fft_axis, sm) != cudaSuccess) return FE_ERR_CUDA;
+  if (fft_allow(k_fft_axis) != cudaSuccess) return FE_ERR_CUDA;
   k_fft_axis<<<grid, kFftThreads, sm, st>>>(data, N, lines, 1, N, 1, inverse, R, tw);
   k_fft_axis<<<grid, kFftThreads, sm, st>>>(data, N, lines, N, NN, N, inverse, R, tw);
   k_fft_axis<<<grid, kFftThreads, sm, st>>>(data, N, lines, lines, 0, NN, inverse, R, tw);
@@ -619,8 +620,8 @@ int spectrum(const T* u0, const T* u1, const T* u2, int N, double* host_bins, in
   double* bins = part + (size_t)kFftGrid * nb;
   constexpr int VL = 16 / sizeof(T);
   const bool vec = N % VL == 0;
-  if (fft_allow(k_fft_rows<T, VL>, sm) != cudaSuccess || fft_allow(k_fft_rows<T, 1>, sm) != cudaSuccess ||
-      fft_allow(k_fft_axis, sm) != cudaSuccess || fft_allow(k_fft_shells, sm) != cudaSuccess)
+  if (fft_allow(k_fft_rows<T, VL>) != cudaSuccess || fft_allow(k_fft_rows<T, 1>) != cudaSuccess ||
+      fft_allow(k_fft_axis) != cudaSuccess || fft_allow(k_fft_shells) != cudaSuccess)
     return FE_ERR_CUDA;
   const int pairs = (N * N + 1) / 2, gx = (pairs + kFftLines - 1) / kFftLines, gl = (lines + kFftLines - 1) / kFftLines;
   const int gs = gl < kFftGrid ? gl : kFftGrid;

@@ -911,13 +911,17 @@ static bool conv_st(const ConvArgs& a, int min_taps, cudaStream_t st) {
   while (taps > min_taps && st_bytes(a, MT, taps) > limit) taps /= 3;
   const int bytes = st_bytes(a, MT, taps);
   if (bytes > limit) return false;
-  if (cudaFuncSetAttribute(k_conv_st<NT, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+  const int nx = (a.No + st_tx(MT) - 1) / st_tx(MT), ny = (a.No + st_ty(MT) - 1) / st_ty(MT),
+            nz = (a.No + kStTz - 1) / kStTz;
+  ConvArgs arg = a;
+  void* args[] = {&arg, &taps};
+  // the limit is one value per kernel and device, whoever launches it: always the most it may be
+  if (cudaFuncSetAttribute(k_conv_st<NT, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess ||
+      cudaLaunchKernel((const void*)k_conv_st<NT, MT>, dim3(nx * ny * nz), dim3(kStThreads), args, bytes, st) !=
+          cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  const int nx = (a.No + st_tx(MT) - 1) / st_tx(MT), ny = (a.No + st_ty(MT) - 1) / st_ty(MT),
-            nz = (a.No + kStTz - 1) / kStTz;
-  k_conv_st<NT, MT><<<nx * ny * nz, kStThreads, bytes, st>>>(a, taps);
   return true;
 }
 
@@ -1036,7 +1040,16 @@ static void bwd_data(UNet& U, int l, int n_in, float* dIn, cudaStream_t st) {
   launch_conv(U, a, st);
 }
 
-static void wgrad(UNet& U, int l, Src s0, Src s1, cudaStream_t st) {
+// most shared memory of k_wgrad over output grids of 2 to 512 cells a side
+static int wg_limit() {
+  int most = 0;
+  for (int N = 2; N <= 512; ++N)
+    for (int mode : {G_SAME, G_DOWN, G_UP}) most = std::max(most, 2 * wg_stage_bytes(mode, N, 32));
+  return most;
+}
+
+// false: the launch was refused
+static bool wgrad(UNet& U, int l, Src s0, Src s1, cudaStream_t st) {
   Layer& y = U.L[l];
   WgradArgs a{s0, s1, y.cin, y.cout, U.N >> y.level_out, U.dpre, y.gw, 0};
   const long nvox = cube(a.No);
@@ -1045,9 +1058,14 @@ static void wgrad(UNet& U, int l, Src s0, Src s1, cudaStream_t st) {
   int bytes = wg_stage_bytes(s0.mode, a.No, co);
   if (s1.C) bytes = std::max(bytes, wg_stage_bytes(s1.mode, a.No, co));
   bytes = std::max(2 * bytes, 3 * co * 16 * 4);
-  cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  k_wgrad<<<dim3((unsigned)((nvox + a.chunk - 1) / a.chunk), 9, y.cin / 16 * (y.cout / co)), 8 * co, bytes, st>>>(a);
+  static const int limit = wg_limit();
+  void* args[] = {&a};
+  const bool ok =
+      cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) == cudaSuccess &&
+      cudaLaunchKernel((const void*)k_wgrad, dim3((unsigned)((nvox + a.chunk - 1) / a.chunk), 9, y.cin / 16 * (y.cout / co)),
+                       dim3(8 * co), args, bytes, st) == cudaSuccess;
   k_bgrad<<<dim3(64, y.cout / 8), 256, 0, st>>>(U.dpre, nvox, y.cout, y.gb);
+  return ok;
 }
 
 }  // namespace fe
@@ -1262,45 +1280,47 @@ int unet_train_step(UNet* U, const T* r, const T* e, const T* dinv, double dt, d
     cudaMemsetAsync(U->L[l].gb, 0, U->L[l].cout * 4, st);
   }
   Src none = src(nullptr, 0, G_SAME, 0);
+  bool ok = true;
   // out (linear)
   k_mask<<<ew(v0 * 16), 256, 0, st>>>(U->dy8, nullptr, nullptr, v0 * 16, U->dpre);
-  wgrad(*U, 8, src(U->u1, 16, G_SAME, n0), none, st);
+  ok = ok && wgrad(*U, 8, src(U->u1, 16, G_SAME, n0), none, st);
   bwd_data(*U, 8, n0, U->g0, st);
   // u1
   k_mask<<<ew(v0 * 16), 256, 0, st>>>(U->g0, nullptr, U->u1, v0 * 16, U->dpre);
-  wgrad(*U, 7, src(U->u2, 32, G_UP, n1), src(U->e1b, 16, G_SAME, n0), st);
+  ok = ok && wgrad(*U, 7, src(U->u2, 32, G_UP, n1), src(U->e1b, 16, G_SAME, n0), st);
   bwd_data(*U, 7, n0, U->g0, st);
   k_up2_back<<<ew(v1 * 32), 256, 0, st>>>(U->g0, n0, 48, 32, U->g1);
   k_slice<<<ew(v0 * 16), 256, 0, st>>>(U->g0, v0, 48, 32, 16, U->gsk0);
   // u2
   k_mask<<<ew(v1 * 32), 256, 0, st>>>(U->g1, nullptr, U->u2, v1 * 32, U->dpre);
-  wgrad(*U, 6, src(U->e3, 64, G_UP, n2), src(U->e2, 32, G_SAME, n1), st);
+  ok = ok && wgrad(*U, 6, src(U->e3, 64, G_UP, n2), src(U->e2, 32, G_SAME, n1), st);
   bwd_data(*U, 6, n1, U->g1, st);
   k_up2_back<<<ew(v2 * 64), 256, 0, st>>>(U->g1, n1, 96, 64, U->g2);
   k_slice<<<ew(v1 * 32), 256, 0, st>>>(U->g1, v1, 96, 64, 32, U->gsk1);
   // e3
   k_mask<<<ew(v2 * 64), 256, 0, st>>>(U->g2, nullptr, U->e3, v2 * 64, U->dpre);
-  wgrad(*U, 5, src(U->d2, 64, G_SAME, n2), none, st);
+  ok = ok && wgrad(*U, 5, src(U->d2, 64, G_SAME, n2), none, st);
   bwd_data(*U, 5, n2, U->g2, st);
   // d2
   k_mask<<<ew(v2 * 64), 256, 0, st>>>(U->g2, nullptr, U->d2, v2 * 64, U->dpre);
-  wgrad(*U, 4, src(U->e2, 32, G_DOWN, n1), none, st);
+  ok = ok && wgrad(*U, 4, src(U->e2, 32, G_DOWN, n1), none, st);
   bwd_data(*U, 4, n1, U->g1, st);
   // e2 (+ skip from u2)
   k_mask<<<ew(v1 * 32), 256, 0, st>>>(U->g1, U->gsk1, U->e2, v1 * 32, U->dpre);
-  wgrad(*U, 3, src(U->d1, 32, G_SAME, n1), none, st);
+  ok = ok && wgrad(*U, 3, src(U->d1, 32, G_SAME, n1), none, st);
   bwd_data(*U, 3, n1, U->g1, st);
   // d1
   k_mask<<<ew(v1 * 32), 256, 0, st>>>(U->g1, nullptr, U->d1, v1 * 32, U->dpre);
-  wgrad(*U, 2, src(U->e1b, 16, G_DOWN, n0), none, st);
+  ok = ok && wgrad(*U, 2, src(U->e1b, 16, G_DOWN, n0), none, st);
   bwd_data(*U, 2, n0, U->g0, st);
   // e1b (+ skip from u1)
   k_mask<<<ew(v0 * 16), 256, 0, st>>>(U->g0, U->gsk0, U->e1b, v0 * 16, U->dpre);
-  wgrad(*U, 1, src(U->e1a, 16, G_SAME, n0), none, st);
+  ok = ok && wgrad(*U, 1, src(U->e1a, 16, G_SAME, n0), none, st);
   bwd_data(*U, 1, n0, U->g0, st);
   // e1a
   k_mask<<<ew(v0 * 16), 256, 0, st>>>(U->g0, nullptr, U->e1a, v0 * 16, U->dpre);
-  wgrad(*U, 0, src(U->in16, 16, G_SAME, n0), none, st);
+  ok = ok && wgrad(*U, 0, src(U->in16, 16, G_SAME, n0), none, st);
+  if (cudaGetLastError() != cudaSuccess || !ok) return FE_ERR_CUDA;  // a launch was refused: no weight moves
   if (lr > 0.0) {
     U->adam_step += 1;
     const float b1 = 0.9f, b2 = 0.999f;

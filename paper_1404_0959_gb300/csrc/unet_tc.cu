@@ -654,14 +654,17 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
 // Launch if the layer fits (stride 1, output grid a multiple of 128, Cout 16 or 32, source channels
 // multiples of 16); returns 0 otherwise.  Resident planes where three planes of all slices, two units ahead and
 // the weights fit in shared memory (rows of four where they do, else of two); else the streamed form.
+// limit: the most shared memory of any layer, since it is one value per kernel and device, whoever launches it.
 template <typename K>
-static int tc_launch(K kernel, const TcConvArgs& a, int rows, int threads, int bytes, int nsm, cudaStream_t st) {
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+static int tc_launch(K kernel, TcConvArgs a, int rows, int threads, int limit, int bytes, int nsm, cudaStream_t st) {
+  const long ntiles = (long)(a.No / 128) * (a.No / rows) * a.No;
+  void* args[] = {&a};
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess ||
+      cudaLaunchKernel((const void*)kernel, dim3((unsigned)(ntiles < nsm ? ntiles : nsm)), dim3(threads), args, bytes,
+                       st) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  const long ntiles = (long)(a.No / 128) * (a.No / rows) * a.No;
-  kernel<<<(int)(ntiles < nsm ? ntiles : nsm), threads, bytes, st>>>(a);
   return 1;
 }
 
@@ -669,7 +672,7 @@ template <int COUT, int R>
 static int ring_launch(const TcConvArgs& a, int nsm, cudaStream_t st) {
   using P = TcRing<COUT, R>;
   const int nsl = (a.c0 + a.c1) / 16;
-  return P::units(nsl) ? tc_launch(k_conv_ring<COUT, R>, a, R, P::threads, P::bytes(nsl), nsm, st) : 0;
+  return P::units(nsl) ? tc_launch(k_conv_ring<COUT, R>, a, R, P::threads, P::room, P::bytes(nsl), nsm, st) : 0;
 }
 
 
@@ -681,7 +684,7 @@ int conv_tc(const TcConvArgs& a, int Cout, int nsm, cudaStream_t st) {
     case 32: {
       using P = TcPlan<32, 2>;
       return ring_launch<32, 2>(a, nsm, st) ||
-             tc_launch(k_conv_tc<32, 2>, a, tc::kR, tc::kThreads, P::bytes(), nsm, st);
+             tc_launch(k_conv_tc<32, 2>, a, tc::kR, tc::kThreads, P::bytes(), P::bytes(), nsm, st);
     }
   }
   return 0;

@@ -112,6 +112,7 @@ int __cudaGetKernel(const void** k, const void* host) {
   return 0;
 }
 int __cudaLaunchKernel(const void* k, dim3 g, dim3, void** args, size_t smem, void*) { return run(k, g, smem, args); }
+int cudaLaunchKernel(const void* k, dim3 g, dim3, void** args, size_t smem, void*) { return run(k, g, smem, args); }
 int cudaLaunchCooperativeKernel(const void* k, dim3 g, dim3, void** args, size_t smem, void*) {
   return run(k, g, smem, args);
 }

@@ -195,3 +195,51 @@ def test_autotune_reports_a_wait_that_ran_out(fake):
     assert fe.lib().fe_step(s.ctx, 1, None) == fe.FE_OK
     assert fe.lib().fe_autotune(s.ctx, 1, None) == fe.FE_OK
     s.close()
+
+
+def test_shared_memory_limits_do_not_follow_the_box(fake):
+    """The limit of a kernel's dynamic shared memory is one value per device: a context of small boxes must not lower
+    what a launch of a large one, on another thread, has just allowed."""
+    def use(N):
+        s = fe.Solver([dict(N=N, tau_p=[], Y0=[])], stream=0, solver=fe.FE_FCG_LEARNED, precision=fe.FE_FP32_MIXED)
+        w = np.zeros(fe.lib().fe_preconditioner_size(), dtype=np.float32)
+        assert fe.lib().fe_load_preconditioner(s.ctx, w.ctypes.data, w.size) == fe.FE_OK
+        r, loss = np.zeros(N ** 3, dtype=np.float32), ctypes.c_double()
+        assert fe.lib().fe_precond_train_step(s.ctx, 0, r.ctypes.data, r.ctypes.data, 0.1, 1e-3,
+                                              ctypes.byref(loss)) == fe.FE_OK
+        spec, d = np.zeros(8), fe.fe_diag()
+        assert fe.lib().fe_diagnostics(s.ctx, 0, ctypes.byref(d), spec.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+                                       8) == fe.FE_OK
+        assert fe.lib().fe_init_state(s.ctx, 0, fe.FE_INIT_SPECTRAL) == fe.FE_OK
+        s.close()
+        return {k: fake.lib.fake_limit(k.encode()) for k in set(fake.kernels)}
+
+    fake.effects = {"k_sumsq": one(2), "k_target": one(6)}
+    for large, small in ((128, 24), (256, 128)):
+        a = use(large)
+        b = use(small)
+        assert any(v > 48 * 1024 for v in a.values())
+        assert all(b[k] >= v for k, v in a.items() if k in b), [(k, v, b[k]) for k, v in a.items() if b.get(k, v) < v]
+
+
+def test_refused_launches_are_not_taken_for_done(fake):
+    """A convolution whose launch is refused runs in the next form that serves the layer; a refused weight-gradient
+    launch fails the step before any weight moves."""
+    s = learned(fe.FE_FP32_MIXED)
+    fake.effects = {"k_sumsq": one(2), "k_target": one(6)}
+    assert train(s) == fe.FE_OK
+    ring = next(k for k in fake.kernels if "k_conv_ringILi16" in k)
+    staged = [sum("k_conv_st" in k for k in fake.kernels)]
+    fake.kernels.clear()
+    fake.fail(ring)
+    assert train(s) == fe.FE_OK
+    staged.append(sum("k_conv_st" in k for k in fake.kernels) + sum("k_conv_ringILi16" in k for k in fake.kernels))
+    assert ring not in fake.kernels and staged[1] > staged[0]
+    wgrad = next(k for k in fake.kernels if "k_wgrad" in k)
+    fake.kernels.clear()
+    fake.fail(wgrad)
+    assert train(s) == fe.FE_ERR_CUDA and not fake.ran("k_adam")
+    fake.fail("cudaFuncSetAttribute")
+    fake.lib.fake_forget_limits()
+    assert train(s) == fe.FE_ERR_CUDA and not fake.ran("k_adam")
+    s.close()
