@@ -10,6 +10,8 @@
 // (per-thread, then a fixed-order warp/block tree, then the box's last block
 // adds the block partials in order).  A box whose solve has finished skips
 // every later launch, so one launch serves all boxes of an ensemble.
+#include <algorithm>
+
 #include "zbulk.cuh"
 #include "zmarch.cuh"
 #include "zring.cuh"
@@ -2013,11 +2015,21 @@ static bool bulk_set_smem(int bytes) {
 }
 // Dynamic shared memory of the streamed CG kernels of one solver for edge N
 // and `cells` per block (sets the kernels' opt-in limit); 0 if it does not fit.
+// The limit is one value per kernel and device, whichever context launches it:
+// always that of the largest edge and solver that run these blocks.
 template <typename T>
 int bulk_cg_prepare(int N, int cells, bool poly) {
+  constexpr int room = 227 * 1024;
   const int bytes = bulk_smem_bytes<T>(N, cells, poly);
-  if (bytes > 227 * 1024) return 0;
-  const bool ok = cells == kBulkCellsPoly ? bulk_set_smem<T, kBulkCellsPoly>(bytes) : bulk_set_smem<T, kBulkCells>(bytes);
+  if (bytes > room) return 0;
+  int limit = bytes;
+  for (int edge = 64; edge <= 512; edge *= 2)
+    for (const bool p : {true, false}) {
+      if (cells != kBulkCells && !p) continue;  // the larger blocks run the polynomial iteration only
+      const int b = bulk_smem_bytes<T>(edge, cells, p);
+      if (b <= room) limit = std::max(limit, b);
+    }
+  const bool ok = cells == kBulkCellsPoly ? bulk_set_smem<T, kBulkCellsPoly>(limit) : bulk_set_smem<T, kBulkCells>(limit);
   return ok ? bytes : 0;
 }
 // (row group, plane) pairs of an N^3 box

@@ -243,3 +243,24 @@ def test_refused_launches_are_not_taken_for_done(fake):
     fake.lib.fake_forget_limits()
     assert train(s) == fe.FE_ERR_CUDA and not fake.ran("k_adam")
     s.close()
+
+
+@pytest.mark.parametrize("solver_id,N0", [(fe.FE_PCG_JACOBI, 256), (fe.FE_PCG_POLY, 128)])
+def test_streamed_cg_beside_a_smaller_context(fake, solver_id, N0):
+    """A context created for smaller boxes leaves the streamed CG kernels of a living one their shared memory."""
+    def iterate(name, gx, args):  # a box starts its refined solve, and nothing ends it but the caps
+        for q in (3, 4):
+            ctypes.cast(pointer(args, q), ctypes.POINTER(ctypes.c_int))[0] = 1
+
+    a = solver((N0,), precision=fe.FE_FP32_MIXED, solver=solver_id)
+    b = solver((64,), precision=fe.FE_FP32_MIXED, solver=solver_id)
+    fake.effects = {"k_refine_start": iterate}
+    for s, N in ((a, N0), (b, 64), (a, N0)):
+        fake.kernels.clear()
+        x = np.zeros(N ** 3, dtype=np.float32)
+        info = fe.fe_solve_info()
+        rc = fe.lib().fe_solve_pressure(s.ctx, 0, x.ctypes.data, x.ctypes.data, 0.1, 1e-8, 2, ctypes.byref(info))
+        assert fake.ran("kb_cg_") and fake.lib.fake_pending_error() == 0
+        assert rc == fe.FE_ERR_NOT_CONVERGED
+    a.close()
+    b.close()
