@@ -525,19 +525,24 @@ bool persist_takes(const Persist* P, int box) { return P && P->takes[box]; }
 // context that is too large for one launch, ms per step: CG, where that solve is bound by the FP64 pipe too and forms
 // each direction once, 3 boxes of 64^3 4.48 -> 4.66, 8 of them 9.97 -> 11.5, 64 of 32^3 to 96^3 82.0 -> 90.6;
 // BiCGStab, 8 boxes of 48^3 16.3 -> 7.8, 48 of 32^3 24.8 -> 13.1.
-// null with *rc = FE_OK: no box does, or the device has no cooperative launches.
+// null with *rc = FE_OK: no box does, the device has no cooperative launches or no memory for the solves (the boxes
+// then iterate kernel by kernel).  No CUDA error is left behind in that case.
 Persist* persist_create(const int* N, int nb, int nsm, bool bicg, cudaStream_t st, int* rc) {
   *rc = FE_OK;
   int dev = 0, coop = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
+    cudaGetLastError();
     return nullptr;
+  }
   const int most = bicg ? kPkBicgUnits : kPkMaxUnits;
   long cap[kPkMaxUnits + 1];  // resident blocks of the device, per units of a block
   for (int upc = 1; upc <= most; upc *= 2) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pk_kernel(bicg, upc), kPkThreads, 0) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pk_kernel(bicg, upc), kPkThreads, 0) != cudaSuccess) {
+      cudaGetLastError();
       return nullptr;
+    }
     cap[upc] = (long)std::min(per_sm, kPkPerSm) * nsm;
   }
   auto units = [&](int b) { return ((long)N[b] * N[b] * N[b] + kPkThreads - 1) / kPkThreads; };
@@ -592,7 +597,6 @@ Persist* persist_create(const int* N, int nb, int nsm, bool bicg, cudaStream_t s
     cudaGetLastError();
     P->work = nullptr;
     persist_free(P);
-    *rc = FE_ERR_OOM;
     return nullptr;
   }
   char* base = reinterpret_cast<char*>(P->work) + wb;

@@ -264,3 +264,33 @@ def test_streamed_cg_beside_a_smaller_context(fake, solver_id, N0):
         assert rc == fe.FE_ERR_NOT_CONVERGED
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("solver_id", [fe.FE_PCG_JACOBI, fe.FE_BICGSTAB_JACOBI])
+def test_without_one_launch_solves(fake, solver_id):
+    """A failed occupancy query, or no memory for the one-launch solves, leaves no error behind and the kernels that
+    solved such boxes without them; every other failed allocation refuses the context and gives all memory back."""
+    kw = dict(transonic=solver_id == fe.FE_BICGSTAB_JACOBI, solver=solver_id)
+    fake.fail("cudaOccupancy")
+    s = solver(**kw)
+    assert fake.lib.fake_pending_error() == 0
+    fake.fail()
+    assert solve(s, 24) == fe.FE_ERR_NOT_CONVERGED and not fake.ran("kc_")
+    s.close()
+    created = 0
+    for n in range(64):
+        fake.lib.fake_fail_alloc(n)
+        try:
+            s = solver(**kw)
+        except fe.FeError as e:
+            assert e.code == fe.FE_ERR_OOM and fake.lib.fake_allocations() == 0
+            continue
+        if fake.lib.fake_fail_alloc_left() >= 0:  # all allocations made
+            s.close()
+            break
+        created += 1
+        assert fake.lib.fake_pending_error() == 0
+        fake.kernels.clear()
+        assert solve(s, 24) == fe.FE_ERR_NOT_CONVERGED and not fake.ran("kc_")
+        s.close()
+    assert created == 1 and n > 8
