@@ -340,20 +340,20 @@ static int tz_default(const fe_ctx* c) {
 }
 
 // (Re)build the work lists for the tile depths tzb (tzb[b] = 0: the built-in depth) and upload the
-// descriptors.  Grows the partial-sum buffer when needed.
+// descriptors.  Grows the partial-sum buffer when needed.  FE_ERR_OOM leaves the context as it was.
 static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
   std::vector<int2> work, ework, kwork, kework;
-  std::vector<BoxDev> kbox;
+  std::vector<BoxDev> box = c->hbox, kbox;
   const int tz0 = tz_default(c);
   long total = 0;
-  for (int b = 0; b < c->nb; ++b) total += (long)c->hbox[b].N * c->hbox[b].N * c->hbox[b].N;
+  for (int b = 0; b < c->nb; ++b) total += (long)box[b].N * box[b].N * box[b].N;
   for (int b = 0; b < c->nb; ++b) {
-    tile_box(c->hbox[b], tzb[b] > 0 ? tzb[b] : tz0, b, work);
-    chunk_box(c->hbox[b], chunk_for(c, total), b, ework);
+    tile_box(box[b], tzb[b] > 0 ? tzb[b] : tz0, b, work);
+    chunk_box(box[b], chunk_for(c, total), b, ework);
   }
-  c->ring_ok = 2;
+  int ring_ok = 2;
   for (int b = 0; b < c->nb; ++b)
-    c->ring_ok = std::min(c->ring_ok, c->hbox[b].N % 2 ? 0 : c->hbox[b].N % (c->fp64 ? 2 : 4) ? 1 : 2);
+    ring_ok = std::min(ring_ok, box[b].N % 2 ? 0 : box[b].N % (c->fp64 ? 2 : 4) ? 1 : 2);
   // plane-streaming blocks (FP32 fields; FP64 contexts are bound by the FP64
   // pipe and keep the z-marching kernel): every box with N in {64, 128, 256,
   // 512}, a persistent grid of the resident blocks per SM x SMs shared out by cells
@@ -362,14 +362,14 @@ static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
   bool stream = !c->prm.transonic && !c->fp64;
   long scells = 0;
   for (int b = 0; b < c->nb && stream; ++b) {
-    const int N = c->hbox[b].N;
+    const int N = box[b].N;
     stream = N >= 64 && N <= 512 && (N & (N - 1)) == 0;
     scells += (long)N * N * N;
   }
   int bcells = 0;
   if (stream) {
     int maxN = 0, minN = 1 << 30;
-    for (int b = 0; b < c->nb; ++b) maxN = std::max(maxN, c->hbox[b].N), minN = std::min(minN, c->hbox[b].N);
+    for (int b = 0; b < c->nb; ++b) maxN = std::max(maxN, box[b].N), minN = std::min(minN, box[b].N);
     const bool poly = c->prm.solver == FE_PCG_POLY;
     bcells = c->fp64 ? bulk_cg_cells<double>(minN, maxN, poly) : bulk_cg_cells<float>(minN, maxN, poly);
     bsmem = c->fp64 ? bulk_cg_prepare<double>(maxN, bcells, poly) : bulk_cg_prepare<float>(maxN, bcells, poly);
@@ -379,7 +379,7 @@ static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
     stream = per_sm > 0;
     const long grid = (long)per_sm * c->nsm;
     for (int b = 0; b < c->nb && stream; ++b) {
-      BoxDev& B = c->hbox[b];
+      BoxDev& B = box[b];
       const long N = B.N, planes = bulk_cg_pairs(B.N, bcells);
       long nb = (grid * N * N * N + scells - 1) / scells;
       nb = std::max(1L, std::min(nb, planes / 4));
@@ -392,11 +392,11 @@ static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
     bwork.clear();
     bsmem = 0;
     bcells = 0;
-    for (int b = 0; b < c->nb; ++b) c->hbox[b].btile0 = c->hbox[b].bntiles = 0;
+    for (int b = 0; b < c->nb; ++b) box[b].btile0 = box[b].bntiles = 0;
   }
   int nkloop = 0, nkeloop = 0;
   if (c->fp64) {
-    kbox = c->hbox;
+    kbox = box;
     for (const bool one_launch : {false, true}) {
       for (int b = 0; b < c->nb; ++b) {
         const int N = kbox[b].N;
@@ -407,51 +407,56 @@ static int set_tiling(fe_ctx* c, const std::vector<int>& tzb) {
       if (!one_launch) nkloop = (int)kwork.size(), nkeloop = (int)kework.size();
     }
   }
-  CK(cudaStreamSynchronize(c->st));
   const int need = (int)std::max({work.size(), ework.size(), bwork.size(), kwork.size(), kework.size()});
-  cudaFree(c->dbwork);
-  c->dbwork = nullptr;
-  if (!bwork.empty() && cudaMalloc(&c->dbwork, bwork.size() * sizeof(int2)) != cudaSuccess) return FE_ERR_OOM;
-  if (!bwork.empty())
-    CK(cudaMemcpyAsync(c->dbwork, bwork.data(), bwork.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
-  c->nbblocks = (int)bwork.size();
-  c->bsmem = bsmem;
-  c->bcells = bcells;
-  cudaFree(c->dkwork);
-  cudaFree(c->dkework);
-  c->dkwork = c->dkework = nullptr;
-  if (c->fp64) {
-    if ((!c->dkbox && cudaMalloc(&c->dkbox, c->nb * sizeof(BoxDev)) != cudaSuccess) ||
-        cudaMalloc(&c->dkwork, kwork.size() * sizeof(int2)) != cudaSuccess ||
-        cudaMalloc(&c->dkework, kework.size() * sizeof(int2)) != cudaSuccess)
-      return FE_ERR_OOM;
-    c->nkblocks = (int)kwork.size();
-    c->nkeblocks = (int)kework.size();
-    c->nkloop = nkloop;
-    c->nkeloop = nkeloop;
-    CK(cudaMemcpyAsync(c->dkework, kework.data(), kework.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(c->dkwork, kwork.data(), kwork.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(c->dkbox, kbox.data(), c->nb * sizeof(BoxDev), cudaMemcpyHostToDevice, c->st));
+  // The new lists beside the old ones: where one cannot be had the context keeps its old tiling whole.
+  std::vector<void*> got;
+  bool oom = false;
+  auto room = [&](size_t bytes) -> void* {
+    void* p = nullptr;
+    if (bytes == 0 || oom) return nullptr;
+    oom = cudaMalloc(&p, bytes) != cudaSuccess;
+    if (oom) return nullptr;
+    got.push_back(p);
+    return p;
+  };
+  auto list = [&](const std::vector<int2>& v) { return (int2*)room(v.size() * sizeof(int2)); };
+  int2 *dwork = list(work), *dework = list(ework), *dbwork = list(bwork), *dkwork = list(kwork), *dkework = list(kework);
+  BoxDev* dkbox = (BoxDev*)room(kbox.size() * sizeof(BoxDev));
+  double* dpart = need > c->npart ? (double*)room((size_t)need * MAXP * sizeof(double)) : nullptr;
+  if (oom) {
+    for (void* p : got) cudaFree(p);
+    cudaGetLastError();  // the refused allocation is this call's verdict, no later one's
+    return FE_ERR_OOM;
   }
-  if ((int)work.size() != c->nblocks || (int)ework.size() != c->neblocks || !c->dpart || need > c->npart) {
-    cudaFree(c->dwork);
-    cudaFree(c->dework);
+  CK(cudaStreamSynchronize(c->st));
+  for (void* p : {(void*)c->dwork, (void*)c->dework, (void*)c->dbwork, (void*)c->dkwork, (void*)c->dkework, (void*)c->dkbox})
+    cudaFree(p);
+  if (dpart) {
     cudaFree(c->dpart);
-    c->dwork = c->dework = nullptr;
-    c->dpart = nullptr;
-    c->npart = 0;
-    if (cudaMalloc(&c->dwork, work.size() * sizeof(int2)) != cudaSuccess ||
-        cudaMalloc(&c->dework, ework.size() * sizeof(int2)) != cudaSuccess ||
-        cudaMalloc(&c->dpart, (size_t)need * MAXP * sizeof(double)) != cudaSuccess)
-      return FE_ERR_OOM;
+    c->dpart = dpart;
     c->npart = need;
   }
-  c->nblocks = (int)work.size();
-  c->neblocks = (int)ework.size();
-  c->tzb = tzb;
   drop_graphs(c);
-  CK(cudaMemcpyAsync(c->dwork, work.data(), work.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->dework, ework.data(), ework.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
+  c->hbox = box;
+  c->ring_ok = ring_ok;
+  c->tzb = tzb;
+  c->bsmem = bsmem;
+  c->bcells = bcells;
+  c->nkloop = nkloop;
+  c->nkeloop = nkeloop;
+  auto put = [&](int2*& d, int& n, int2* p, const std::vector<int2>& v) {
+    d = p;
+    n = (int)v.size();
+    return n == 0 || cudaMemcpyAsync(p, v.data(), v.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st) == cudaSuccess;
+  };
+  c->dkbox = dkbox;
+  bool ok = put(c->dwork, c->nblocks, dwork, work);
+  ok = put(c->dework, c->neblocks, dework, ework) && ok;
+  ok = put(c->dbwork, c->nbblocks, dbwork, bwork) && ok;
+  ok = put(c->dkwork, c->nkblocks, dkwork, kwork) && ok;
+  ok = put(c->dkework, c->nkeblocks, dkework, kework) && ok;
+  if (!ok) return FE_ERR_CUDA;
+  if (dkbox) CK(cudaMemcpyAsync(dkbox, kbox.data(), c->nb * sizeof(BoxDev), cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(c->dbox, c->hbox.data(), c->nb * sizeof(BoxDev), cudaMemcpyHostToDevice, c->st));
   CK(cudaStreamSynchronize(c->st));
   return FE_OK;

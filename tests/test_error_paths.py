@@ -294,3 +294,33 @@ def test_without_one_launch_solves(fake, solver_id):
         assert solve(s, 24) == fe.FE_ERR_NOT_CONVERGED and not fake.ran("kc_")
         s.close()
     assert created == 1 and n > 8
+
+
+@pytest.mark.parametrize("precision,sizes", [(fe.FE_FP64, (24, 100)), (fe.FE_FP32_MIXED, (64, 64)),
+                                             (fe.FE_FP32_MIXED, (24, 40))])
+def test_tiling_that_does_not_fit_in_memory(fake, precision, sizes):
+    """When an allocation of new work lists fails the context keeps its old ones whole: a step launches no kernel on a
+    list that is gone or shorter than its grid."""
+    s = solver(sizes, precision=precision)
+    lists, bad = [], []
+
+    def check(name, gx, args):
+        lists.append(name)
+        if not fake.lib.fake_room(pointer(args, 0)) or fake.lib.fake_room(pointer(args, 1)) < gx * 8:
+            bad.append(name)
+
+    for n in range(16):
+        fake.lib.fake_fail_alloc(n)
+        rc = fe.lib().fe_set_tiling(s.ctx, 1 + n % 3)
+        done = fake.lib.fake_fail_alloc_left() >= 0
+        fake.lib.fake_fail_alloc(-1)
+        assert rc == (fe.FE_OK if done else fe.FE_ERR_OOM)
+        fake.effects = {"PKNS_6BoxDevEPK4int2": check}
+        assert fe.lib().fe_step(s.ctx, 1, None) == fe.FE_OK
+        solve(s, sizes[0])
+        fake.effects = {}
+        assert not bad, (n, bad)
+        if done:
+            break
+    assert done and n >= 2 and len(lists) > 20
+    s.close()
