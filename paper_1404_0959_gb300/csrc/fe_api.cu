@@ -585,6 +585,7 @@ extern "C" int fe_create(const fe_params* prm, void* stream, fe_ctx** out) {
   if (rc == FE_OK) rc = set_tiling(c, 0);
   if (rc != FE_OK) {
     fe_destroy(c);
+    if (rc == FE_ERR_OOM) cudaGetLastError();  // this call's verdict, no later one's
     return rc;
   }
   *out = c;

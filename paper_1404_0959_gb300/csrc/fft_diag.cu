@@ -570,7 +570,10 @@ int ic_spectral(T* u0, T* u1, T* u2, int N, uint64_t seed, double k0, double mac
   const long n = (long)N * N * N;
   const int nb = ew_grid(n);
   double2* buf = nullptr;  // three complex fields, the roots of unity, the block sums
-  if (cudaMalloc(&buf, (3 * n + N) * sizeof(double2) + nb * sizeof(double)) != cudaSuccess) return FE_ERR_OOM;
+  if (cudaMalloc(&buf, (3 * n + N) * sizeof(double2) + nb * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    return FE_ERR_OOM;
+  }
   double2* tw = buf + 3 * n;
   double* part = reinterpret_cast<double*>(tw + N);
   k_roots<<<1, 256, 0, st>>>(tw, N);

@@ -1145,6 +1145,7 @@ UNet* unet_create(int N, bool training, int* rc) {
   UNet* U = new UNet();
   *rc = unet_alloc(*U, N, training);
   if (*rc != FE_OK) {
+    cudaGetLastError();  // of the refused allocation
     unet_free(*U);
     delete U;
     return nullptr;
@@ -1383,7 +1384,10 @@ int unet_activation(UNet* U, int l, float* host, long count, cudaStream_t st) {
   }
   if (count != n) return FE_ERR_INVALID_ARG;
   float* d = nullptr;
-  if (cudaMalloc(&d, n * 4) != cudaSuccess) return FE_ERR_OOM;
+  if (cudaMalloc(&d, n * 4) != cudaSuccess) {
+    cudaGetLastError();
+    return FE_ERR_OOM;
+  }
   k_bf16_to_f32<<<ew(n), 256, 0, st>>>(p, n, d);
   cudaMemcpyAsync(host, d, n * 4, cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);

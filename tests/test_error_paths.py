@@ -324,3 +324,39 @@ def test_tiling_that_does_not_fit_in_memory(fake, precision, sizes):
             break
     assert done and n >= 2 and len(lists) > 20
     s.close()
+
+
+def test_refused_allocations_leave_no_error_behind(fake):
+    """FE_ERR_OOM of one call is not reported again by the next check, of this context or of another."""
+    s = fe.Solver([dict(N=24, tau_p=[], Y0=[])], stream=0, solver=fe.FE_FGMRES_LEARNED, precision=fe.FE_FP32_MIXED)
+    w = np.zeros(fe.lib().fe_preconditioner_size(), dtype=np.float32)
+    act = np.zeros(24 ** 3 * 16, dtype=np.float32)
+    diag, stats, total, area = fe.fe_diag(), fe.fe_les_stats(), ctypes.c_longlong(), ctypes.c_double()
+    f = np.zeros(24 ** 3, dtype=np.float32)
+    lib, p = fe.lib(), f.ctypes.data
+
+    def create():
+        return solver((24,), precision=fe.FE_FP32_MIXED).close() or fe.FE_OK
+
+    calls = [create, lambda: lib.fe_init_state(s.ctx, 0, fe.FE_INIT_SPECTRAL),
+             lambda: lib.fe_load_preconditioner(s.ctx, w.ctypes.data, w.size),
+             lambda: lib.fe_precond_activation(s.ctx, 0, act.ctypes.data, act.size),
+             lambda: lib.fe_diagnostics(s.ctx, 0, ctypes.byref(diag), None, 0),
+             lambda: lib.fe_les_apriori(s.ctx, 0, 2, 0.17, ctypes.byref(stats), None),
+             lambda: lib.fe_isosurface(s.ctx, 0, p, 0.5, None, 0, ctypes.byref(total), ctypes.byref(area)),
+             lambda: lib.fe_raster_depth(s.ctx, None, 0, 16, 1.0, p)]
+    for call in calls:
+        for n in range(64):
+            lib.fake_fail_alloc(n)
+            try:
+                rc = call()
+            except fe.FeError as e:
+                rc = e.code
+            done = lib.fake_fail_alloc_left() >= 0
+            lib.fake_fail_alloc(-1)
+            assert rc == (fe.FE_OK if done else fe.FE_ERR_OOM), (calls.index(call), n)
+            assert lib.fake_pending_error() == 0, (calls.index(call), n)
+            if done:
+                break
+        assert done and n >= 1
+    s.close()
