@@ -1469,7 +1469,17 @@ static int solve_box(fe_ctx* c, int box, const void* b, void* x, double dt, doub
   c->prm.p_maxit = maxit;
   rc = pressure_solve<T>(c);
   c->prm.p_maxit = save_maxit;
-  if (rc != FE_OK) return rc;
+  // the step scalars (tolerance, cap, dt) of every box as they were, whatever the solve's verdict
+  auto restore = [&]() -> int {
+    memcpy(c->hsc, saved.data(), saved.size() * sizeof(double));
+    CK(cudaMemcpyAsync(c->dsc, c->hsc, (size_t)c->nb * NSC * sizeof(double), cudaMemcpyHostToDevice, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    return FE_OK;
+  };
+  if (rc != FE_OK) {
+    restore();
+    return rc;
+  }
   if (c->fp64) launch_true_res<T>(c->L(), K_X);
   CK(cudaMemcpyAsync(x, B.f[fused_refine(c) ? K_XH : K_X], bytes, cudaMemcpyDeviceToDevice, c->st));
   rc = pull_scalars(c);
@@ -1485,10 +1495,8 @@ static int solve_box(fe_ctx* c, int box, const void* b, void* x, double dt, doub
   }
   const bool conv = s[SC_CONV] != 0.0, failed = gave_up(c);
   if (info) *info = inf;
-  // restore the step scalars (tolerance, cap, dt) of every box
-  memcpy(c->hsc, saved.data(), saved.size() * sizeof(double));
-  CK(cudaMemcpyAsync(c->dsc, c->hsc, (size_t)c->nb * NSC * sizeof(double), cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));
+  rc = restore();
+  if (rc != FE_OK) return rc;
   if (failed) return FE_ERR_CUDA;
   return conv ? FE_OK : FE_ERR_NOT_CONVERGED;
 }

@@ -360,3 +360,14 @@ def test_refused_allocations_leave_no_error_behind(fake):
                 break
         assert done and n >= 1
     s.close()
+
+
+def test_refused_solve_leaves_the_step_scalars(fake):
+    """fe_solve_pressure without a loaded network is refused; its tolerance, cap and dt do not stay for the steps."""
+    _, nsc = scalar_slot("SC_KERR")
+    s = fe.Solver([dict(N=24, tau_p=[], Y0=[])], stream=0, solver=fe.FE_FCG_LEARNED)
+    sc = ctypes.cast(fake.lib.fake_find(nsc * 8), ctypes.POINTER(ctypes.c_double))
+    before = [sc[q] for q in range(nsc)]
+    assert solve(s, 24, tol=0.5) == fe.FE_ERR_UNSUPPORTED
+    assert [sc[q] for q in range(nsc)] == before
+    s.close()
