@@ -22,7 +22,6 @@
 #include <cuda_bf16.h>
 
 #include <cstring>
-#include <type_traits>
 #include <vector>
 
 #include "fe_internal.cuh"
@@ -949,7 +948,7 @@ static bool launch_conv_st(const UNet& U, const ConvArgs& a, cudaStream_t st) {
     case 2: return (big && conv_st<2, 8>(a, 1, st)) || (mid && conv_st<2, 4>(a, 1, st)) || conv_st<2, 2>(a, 1, st);
     case 4: return (mid && conv_st<4, 4>(a, 1, st)) || conv_st<4, 2>(a, 1, st);
     case 6: return (mid && conv_st<6, 4>(a, 1, st)) || conv_st<6, 2>(a, 1, st);
-    case 8: return conv_st<8, 2>(a, 1, st) || conv_st<8, 4>(a, 1, st);
+    case 8: return conv_st<8, 2>(a, 1, st);
     case 12: return conv_st<12, 2>(a, 1, st);
   }
   return false;
@@ -972,18 +971,20 @@ static void launch_conv(const UNet& U, const ConvArgs& a, cudaStream_t st) {
   if (launch_conv_st(U, a, st)) return;
   const long nvox = cube(a.No);
   const int grid = (int)((nvox + 16 * CONV_MT * CONV_WARPS - 1) / (16 * CONV_MT * CONV_WARPS));
-  auto run = [&](auto nt) {
-    constexpr int NT = decltype(nt)::value;
-    if (a.s0.mode == G_DOWN_T) k_conv<NT, true><<<grid, CONV_WARPS * 32, 0, st>>>(a);
-    else k_conv<NT, false><<<grid, CONV_WARPS * 32, 0, st>>>(a);
-  };
+  const int threads = CONV_WARPS * 32;
+  const bool down_t = a.s0.mode == G_DOWN_T;  // data gradients of the stride-2 layers: into 16 or 32 channels
   switch (a.Cout / 8) {
-    case 1: run(std::integral_constant<int, 1>()); break;
-    case 2: run(std::integral_constant<int, 2>()); break;
-    case 4: run(std::integral_constant<int, 4>()); break;
-    case 6: run(std::integral_constant<int, 6>()); break;
-    case 8: run(std::integral_constant<int, 8>()); break;
-    case 12: run(std::integral_constant<int, 12>()); break;
+    case 2:
+      if (down_t) k_conv<2, true><<<grid, threads, 0, st>>>(a);
+      else k_conv<2, false><<<grid, threads, 0, st>>>(a);
+      break;
+    case 4:
+      if (down_t) k_conv<4, true><<<grid, threads, 0, st>>>(a);
+      else k_conv<4, false><<<grid, threads, 0, st>>>(a);
+      break;
+    case 6: k_conv<6, false><<<grid, threads, 0, st>>>(a); break;
+    case 8: k_conv<8, false><<<grid, threads, 0, st>>>(a); break;
+    case 12: k_conv<12, false><<<grid, threads, 0, st>>>(a); break;
   }
 }
 
