@@ -476,12 +476,16 @@ __global__ void __launch_bounds__((TcRing<COUT, R>::threads), 1) k_conv_ring(TcC
     int i = 0;        // tile of the block
     unsigned ub = 0;  // first unit of the tile's lower plane
     bool ok = true;
+    if (t0 + me < t1) {  // this warp's first tile begins with unit me nsl, 2 nsl further in the second run
+      const int first = me * nsl + ((int)(t0 % No) + me < No ? 0 : 2 * nsl);
+      ok = __all_sync(0xffffffffu, first < NU || mbar_wait(primed, 0));
+    }
     for (long t = t0; t < t1 && ok;) {
       int x0, y0, zs;
       const int n = run_of(t, x0, y0, zs);
       for (int j = 0; j < n && ok; ++j, ++i, ub += nsl) {
         if (i % NB != me) continue;
-        bool w = i >= NB ? mbar_wait(acc_empty + me, (unsigned)((i / NB - 1) & 1)) : (int)ub < NU || mbar_wait(primed, 0);
+        bool w = i < NB || mbar_wait(acc_empty + me, (unsigned)((i / NB - 1) & 1));
         for (int sl = 0; sl < nsl && ok; ++sl) {
           unsigned slot[3];
 #pragma unroll
