@@ -609,7 +609,7 @@ struct UNet {
   // training buffers
   float *g0 = nullptr, *g1 = nullptr, *g2 = nullptr, *gsk0 = nullptr, *gsk1 = nullptr, *dy8 = nullptr;
   bf16* dpre = nullptr;
-  double* part = nullptr;
+  double* part = nullptr;  // block sums of a reduction, then `err`: one copy brings both
   int adam_step = 0;
   std::vector<void*> allocs;
   bool trained = false;
@@ -635,6 +635,11 @@ int conv_tc(const TcConvArgs& a, int Cout, int nsm, cudaStream_t st);
 
 static long cube(long n) { return n * n * n; }
 
+static int ew(long n) {
+  long g = (n + 255) / 256;
+  return (int)(g < 152L * 8 ? g : 152L * 8);
+}
+
 static int unet_alloc(UNet& U, int N, bool training) {
   U.N = N;
   const long n0 = cube(N), n1 = cube(N / 2), n2 = cube(N / 4);
@@ -654,8 +659,11 @@ static int unet_alloc(UNet& U, int N, bool training) {
   U.u2 = (bf16*)A(n1 * 32 * 2);
   U.u1 = (bf16*)A(n0 * 16 * 2);
   U.out32 = (float*)A(n0 * 4);
-  U.err = (int*)A(sizeof(int));
-  if (U.err) cudaMemset(U.err, 0, sizeof(int));
+  U.part = (double*)A((ew(n0) + 1) * sizeof(double));
+  if (U.part) {
+    cudaMemset(U.part, 0, (ew(n0) + 1) * sizeof(double));
+    U.err = (int*)(U.part + ew(n0));
+  }
   {
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -708,8 +716,7 @@ static int unet_alloc(UNet& U, int N, bool training) {
     U.gsk1 = (float*)A(n1 * 32 * 4);
     U.dy8 = (float*)A(n0 * 16 * 4);
     U.dpre = (bf16*)A(n0 * 64 * 2 > n1 * 96 * 2 ? n0 * 64 * 2 : n1 * 96 * 2);
-    U.part = (double*)A(4096 * 8);
-    if (!U.g0 || !U.g1 || !U.g2 || !U.gsk0 || !U.gsk1 || !U.dy8 || !U.dpre || !U.part) return FE_ERR_OOM;
+    if (!U.g0 || !U.g1 || !U.g2 || !U.gsk0 || !U.gsk1 || !U.dy8 || !U.dpre) return FE_ERR_OOM;
   }
   return FE_OK;
 }
@@ -719,11 +726,6 @@ static void unet_free(UNet& U) {
   U.allocs.clear();
   if (U.herr) cudaFreeHost(U.herr);
   U.herr = nullptr;
-}
-
-static int ew(long n) {
-  long g = (n + 255) / 256;
-  return (int)(g < 152L * 8 ? g : 152L * 8);
 }
 
 // ---- weight and bias gradients ---------------------------------------------------------------
@@ -1121,15 +1123,6 @@ __global__ void k_scale_to_f32(const T* a, long n, double s, float* out) {
     out[q] = (float)((double)a[q] * s);
 }
 
-static double host_sum(const double* dpart, int nb, cudaStream_t st) {
-  std::vector<double> h(nb);
-  cudaMemcpyAsync(h.data(), dpart, nb * sizeof(double), cudaMemcpyDeviceToHost, st);
-  cudaStreamSynchronize(st);
-  double s = 0.0;
-  for (int b = 0; b < nb; ++b) s += h[b];
-  return s;
-}
-
 // Queue the copy of the flag behind the work on st; after the stream has been waited for, unet_failed says whether
 // a convolution of that work gave up, and clears the flag.
 void unet_queue_error(UNet* U, cudaStream_t st) {
@@ -1140,6 +1133,20 @@ bool unet_failed(UNet* U, cudaStream_t st) {
   cudaMemsetAsync(U->err, 0, sizeof(int), st);
   *U->herr = 0;
   return true;
+}
+
+// Sum of the nb = ew(N^3) block sums in U.part, added in order; *failed: whether a convolution gave up (unet_failed).
+static double host_sum(UNet& U, int nb, cudaStream_t st, bool* failed = nullptr) {
+  std::vector<double> h(nb + 1);
+  cudaMemcpyAsync(h.data(), U.part, (nb + 1) * sizeof(double), cudaMemcpyDeviceToHost, st);
+  cudaStreamSynchronize(st);
+  if (failed) {
+    memcpy(U.herr, &h[nb], sizeof(int));
+    *failed = unet_failed(&U, st);
+  }
+  double s = 0.0;
+  for (int b = 0; b < nb; ++b) s += h[b];
+  return s;
 }
 
 UNet* unet_create(int N, bool training, int* rc) {
@@ -1231,7 +1238,7 @@ static void precond_scales(UNet* U, const T* r, double dt, double ih, cudaStream
   const long n = cube(U->N);
   const int nb = ew(n);
   k_sumsq<T><<<nb, 256, 0, st>>>(r, n, U->part);
-  const double rr = host_sum(U->part, nb, st);
+  const double rr = host_sum(*U, nb, st);
   *rms = rr > 0.0 ? sqrt(rr / (double)n) : 0.0;
   *d0 = 1.0 / (1.0 / dt + 3.0 * dt * ih * ih);
 }
@@ -1240,7 +1247,6 @@ static void precond_scales(UNet* U, const T* r, double dt, double ih, cudaStream
 template <typename T>
 int unet_apply(UNet* U, const T* r, const T* dinv, double dt, double ih, float* z, cudaStream_t st) {
   const long n = cube(U->N);
-  if (!U->part) return FE_ERR_UNSUPPORTED;
   double rms, d0;
   precond_scales<T>(U, r, dt, ih, st, &rms, &d0);
   k_pack_input<T><<<ew(n), 256, 0, st>>>(r, dinv, n, rms > 0.0 ? 1.0 / (rms * d0) : 0.0, 3.0 * dt * ih * ih,
@@ -1268,15 +1274,15 @@ int unet_train_step(UNet* U, const T* r, const T* e, const T* dinv, double dt, d
   if (!(rms > 0.0)) return FE_ERR_INVALID_ARG;
   k_pack_input<T><<<ew(v0), 256, 0, st>>>(r, dinv, v0, 1.0 / (rms * d0), 3.0 * dt * ih * ih, U->in16);
   unet_forward(*U, st);
-  unet_queue_error(U, st);
   // target into gsk0 (fp32 scratch), its norm, then loss and dL/dy
   float* tgt = U->gsk0;
   k_target<T><<<nb, 256, 0, st>>>(r, e, dinv, v0, 1.0 / (rms * d0), tgt, U->part);
-  const double tt = host_sum(U->part, nb, st);
-  if (unet_failed(U, st)) return FE_ERR_CUDA;  // before any weight moves
+  bool failed = false;
+  const double tt = host_sum(*U, nb, st, &failed);
+  if (failed) return FE_ERR_CUDA;  // before any weight moves
   if (!(tt > 0.0)) return FE_ERR_INVALID_ARG;
   k_loss_grad<<<nb, 256, 0, st>>>(U->out32, tgt, v0, 1.0 / tt, U->dy8, U->part);
-  *loss = host_sum(U->part, nb, st) / tt;
+  *loss = host_sum(*U, nb, st) / tt;
   for (int l = 0; l < kNL; ++l) {
     cudaMemsetAsync(U->L[l].gw, 0, 27L * U->L[l].cin * U->L[l].cout * 4, st);
     cudaMemsetAsync(U->L[l].gb, 0, U->L[l].cout * 4, st);
