@@ -27,8 +27,15 @@
  *  - Device pointers are borrowed: the caller keeps them alive and issues
  *    its own work on the stream given to fe_create (work is ordered on that
  *    stream).  Host pointers are read/written synchronously before return.
- *  - The context owns all of its device memory (allocated in fe_create,
- *    freed in fe_destroy).  Calls on one context must not run concurrently.
+ *  - The context owns all of its device memory: allocated in fe_create, but
+ *    for the network (fe_load_preconditioner) and the work memory of the
+ *    analysis calls (their first call, as stated there; grown where a larger
+ *    box asks, kept after that); freed in fe_destroy.  An FP64 context with
+ *    FE_BICGSTAB_JACOBI holds 13 more doubles per cell of the boxes whose
+ *    solves run in one launch.  Calls on one context must not run
+ *    concurrently.  FE_ERR_OOM of a call leaves the context usable as it was.
+ *  - FE_ERR_CUDA of a step, solve, training step or autotune also says that a
+ *    kernel gave up one of its bounded waits: the result is not to be used.
  */
 #ifndef FE_H
 #define FE_H
@@ -254,12 +261,16 @@ int fe_solve_pressure(fe_ctx* ctx, int box, const void* b, void* x, double dt,
 /* Turbulence diagnostics of one box (Sec. 2 par. 1: spectrum, enstrophy,
  * kinetic energy, Taylor microscale; Fig. 1: density r.m.s.).  spectrum:
  * NULL or a host array of nbins doubles, E(k) = sum over modes with
- * round(|k|) = k of |u_hat|^2 / (2 N^6). */
+ * round(|k|) = k of |u_hat|^2 / (2 N^6).  Work memory is allocated on the
+ * first call and kept by the context: block sums, and with a spectrum a half
+ * spectrum of 16 N^2 (N/2 + 1) bytes (1.1 GB at 512^3); FE_ERR_OOM if it cannot
+ * be. */
 int fe_diagnostics(fe_ctx* ctx, int box, fe_diag* out, double* spectrum, int nbins);
 
 /* Q criterion (|Omega|^2 - |S|^2)/2 of the current velocity of a box into a
  * device array of N^3 context-precision values (Fig. 3 of the paper shows
- * Q iso-surfaces). */
+ * Q iso-surfaces).  Evaluated in double for either precision and rounded
+ * once, so that it holds where strain and rotation cancel. */
 int fe_q_criterion(fe_ctx* ctx, int box, void* q_dev);
 
 /* Iso-surface of a cell field (Fig. 3 of the paper shows iso-surfaces of Q;
@@ -295,7 +306,7 @@ int fe_isosurface(fe_ctx* ctx, int box, const void* field, double iso, double* t
  * E_01 Z_2) / ((E_12 + E_20) + E_01) in FP32, the smallest non-negative depth
  * kept, +inf where nothing is covered.  depth: device array of width^2 floats,
  * row py * width + px.  Each step is one correctly rounded operation in this
- * order. */
+ * order.  The centres (8 width bytes) are kept by the context. */
 int fe_raster_depth(fe_ctx* ctx, const double* tri, long long ntri, int width, double extent, float* depth);
 
 /* A-priori analysis for large-eddy simulation (Sec. 1 names LES of the plume
@@ -419,7 +430,14 @@ int fe_plane_streaming_active(const fe_ctx* ctx);
 /* Tile depth of the stencil kernels: every kernel launch covers all boxes
  * with 32 x 8-cell column tiles that walk tz z-planes.  fe_set_tiling sets tz
  * for every box, fe_set_box_tiling for one (0 = built-in default, chosen
- * from the context's boxes so that the tiles fill the multiprocessors).  fe_autotune times `trials` trial steps (computed from
+ * from the context's boxes so that the tiles fill the multiprocessors).  Cell
+ * values do not depend on the depth, sums over a box are added by tiles: FP64
+ * pressure solves take their order from the box alone, so a box iterates the
+ * same in any context; in FE_FP32_MIXED contexts the float-pair sums of a box,
+ * and with them the last bits of its iterates, can differ from those of the
+ * same box in another context.  (The kernels of odd and even N round
+ * differently, and one odd N puts all boxes of a context on the former.)
+ * fe_autotune times `trials` trial steps (computed from
  * the current state and discarded: the state and clock are unchanged) for
  * tz in {4, 8, 16, 24, 32, 48, 64} for all boxes, then, when the boxes have several
  * sizes, for each size in turn (largest first) with the other boxes fixed;

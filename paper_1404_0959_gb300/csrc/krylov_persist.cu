@@ -18,10 +18,10 @@
 //
 // A meeting: publish, count up the box's counter, wait until all blocks have (one
 // thread per block polls), read the published sums.  Two sets of sums alternate: a
-// block can be at most one meeting ahead of another.  Measured with 256 threads per
-// block: 3.2 us for 54 blocks, 3.4 us for 152, 4.1 us for 304, against 3.3, 5.7 and
-// 10.9 us where every block polls every other's sum, and 3.2 us at 152 through
-// clusters of eight.  The counters are cleared before each launch.  Waits are
+// block can be at most one meeting ahead of another.  A meeting alone, in a probe
+// with 256 threads per block (the kernels have 128): 3.2 us for 54 blocks, 3.4 us for
+// 152, 4.1 us for 304, against 3.3, 5.7 and 10.9 us where every block polls every
+// other's sum, and 3.2 us at 152 through clusters of eight.  The counters are cleared before each launch.  Waits are
 // bounded: a block that gives up sets SC_KERR, finishes, and leaves the others to
 // their own limits.
 #include <algorithm>

@@ -14,11 +14,15 @@
 // (16-wide channel groups keep every K step of the tensor-core GEMM full).
 //
 // Activations are channels-last BF16 (voxel-major, channels contiguous).
-// Convolutions are implicit GEMMs on the tensor cores (mma.sync m16n8k16,
-// BF16 x BF16 -> FP32): rows = voxels gathered per tap, K = input channels,
-// columns = output channels.  The same gather kernel serves the forward pass
-// and the data gradient (transposed weights, negated taps); the weight
-// gradient is a GEMM over voxels with FP32 atomics per CTA.
+// Convolutions are implicit GEMMs on the tensor cores (BF16 x BF16 -> FP32):
+// rows = voxels per tap, K = input channels, columns = output channels.
+// Stride-1 layers on grids of a multiple of 128 run on tcgen05.mma
+// (unet_tc.cu); other layers and the data gradients of stride 1 (transposed
+// weights, negated taps) on k_conv_st, operands staged in shared memory
+// (mma.sync m16n8k16); the data gradients of stride 2 and the deepest
+// stride-2 layer on k_conv, which gathers its operands and serves any layer
+// the others refuse.  The weight gradient (k_wgrad) is a GEMM over voxels
+// from staged rows, one FP32 atomic per weight and chunk of voxels.
 #include <cuda_bf16.h>
 
 #include <cstring>
