@@ -1,6 +1,6 @@
 """The tensor-memory convolution with resident planes on other numbers of blocks than this chip's 152: a block's
 first run of planes may then be shorter than one tile per issuing warp, and an issuer's first tile lie beyond the
-ring's first fill (121 to 159 blocks: 48 -> 16 and 32 -> 32 channels)."""
+ring's first fill (most numbers that are no multiple of four, 48 -> 16 and 32 -> 32 channels)."""
 import ctypes
 
 import pytest
